@@ -71,6 +71,9 @@ struct ea_handle {
     std::vector<unsigned char> lazy_w;  // PASS_LAZY: worker i's e holds its last u (see lazy_residual)
     bool lazy_s = false;                // PASS_LAZY: e_s holds the last w
     bool lazy_staged = false;           // PASS_LAZY broadcast: every tile's worker messages fit the staging
+    // The last launch held the SMs at their largest shared memory for more than one tile per CTA: the
+    // next one waits for it, so that the SMs are empty and take the round's own split (launch_pdl).
+    bool split_full = false;
     bool wscales_pending = false;       // PASS_LAZY workers: a message's scales are not formed yet
     int n_compressed = 0;
     bool has_message = false;
@@ -90,6 +93,14 @@ int fail(ea_handle *h, int code, const char *fmt, ...)
     if (h) h->err = buf;
     else g_last_error = buf;
     return code;
+}
+
+// Whether the handle's next launch may overlap the one before it.
+bool may_overlap(ea_handle *h)
+{
+    const bool overlap = !h->split_full;
+    h->split_full = false;
+    return overlap;
 }
 
 int check_cuda(ea_handle *h, cudaError_t e, const char *what)
@@ -479,7 +490,7 @@ int finalize_scales(ea_handle *h, const QHost &q, const double *partials, float 
     f.q = device_quant(q);
     f.partials = partials;
     f.scales = scales;
-    return check_cuda(h, launch_finalize(f, h->stream), "finalize launch");
+    return check_cuda(h, launch_finalize(f, h->stream, may_overlap(h)), "finalize launch");
 }
 
 // PASS_LAZY worker messages: the scales of all n messages in one launch, from each worker's own
@@ -495,7 +506,7 @@ int finalize_worker_scales(ea_handle *h)
     f.n_msgs = h->cfg.n;
     f.partials_stride = h->qw.n_pairs;
     f.scales_stride = h->lay.wscale_stride;
-    const int r = check_cuda(h, launch_finalize(f, h->stream), "finalize launch");
+    const int r = check_cuda(h, launch_finalize(f, h->stream, may_overlap(h)), "finalize launch");
     if (r == EA_OK) h->wscales_pending = false;
     return r;
 }
@@ -516,7 +527,7 @@ int second_pass(ea_handle *h, const QHost &q, const double *partials, float *buf
     e.seed = h->cfg.seed;
     e.id = id;
     e.t = static_cast<uint32_t>(h->t);
-    return check_cuda(h, launch_encode(e, h->stream), "encode launch");
+    return check_cuda(h, launch_encode(e, h->stream, may_overlap(h)), "encode launch");
 }
 
 }  // namespace
@@ -724,8 +735,9 @@ int ea_worker_compress(ea_handle *h, int32_t worker, const float *g)
         a.gp = device_group_plan(h->qw, h->epoch_w);
         r = check_cuda(h, launch_worker_grouped(W ? MODE_W : MODE_S, a, h->qw.grid, h->stream), "worker launch");
         if (r == EA_OK) ++h->epoch_w;
+        h->split_full = true;
     } else {
-        r = check_cuda(h, launch_worker(W ? MODE_W : MODE_S, a, h->stream), "worker launch");
+        r = check_cuda(h, launch_worker(W ? MODE_W : MODE_S, a, h->stream, may_overlap(h)), "worker launch");
     }
     if (r == EA_OK && h->qw.pass == PASS_STASH) r = second_pass(h, h->qw, a.partials, a.e, a.words, a.scales, a.id);
     if (r != EA_OK) return r;
@@ -783,8 +795,10 @@ int ea_server_step(ea_handle *h)
         a.gp = device_group_plan(h->qs, h->epoch_s);
         r = check_cuda(h, launch_server_grouped(W ? MODE_W : MODE_S, a, h->qs.grid, h->stream), "server launch");
         if (r == EA_OK) ++h->epoch_s;
+        h->split_full = true;
     } else {
         r = check_cuda(h, launch_server(W ? MODE_W : MODE_S, a, h->stream), "server launch");
+        if (h->splan.enabled && h->splan.grid < h->n_tiles) h->split_full = true;
     }
     if (r == EA_OK && h->qs.pass == PASS_STASH)
         r = second_pass(h, h->qs, h->spartials, h->es, h->scodes, h->sscales, static_cast<uint32_t>(h->cfg.n));
@@ -810,7 +824,7 @@ int ea_worker_apply(ea_handle *h, float *x)
     a.q = device_quant(h->qs);
     a.words = h->scodes;
     a.scales = h->sscales;
-    return check_cuda(h, launch_apply(a, h->stream), "apply launch");
+    return check_cuda(h, launch_apply(a, h->stream, may_overlap(h)), "apply launch");
 }
 
 int ea_set_hparams(ea_handle *h, float alpha, float beta1, float beta2)
@@ -886,7 +900,7 @@ int ea_get_view(const ea_handle *h, int32_t which, int32_t index, void **dev_ptr
             ra.out = h->rview;
             ra.q = device_quant(h->qw);
             ra.scales = h->wscales + index * h->lay.wscale_stride;
-            int r = check_cuda(hm, launch_lazy_resid(ra, h->stream), "residual launch");
+            int r = check_cuda(hm, launch_lazy_resid(ra, h->stream, may_overlap(hm)), "residual launch");
             if (r == EA_OK) r = check_cuda(hm, cudaStreamSynchronize(h->stream), "stream synchronize");
             if (r != EA_OK) return r;
             p = h->rview;
@@ -902,7 +916,7 @@ int ea_get_view(const ea_handle *h, int32_t which, int32_t index, void **dev_ptr
             ra.out = h->rview;
             ra.q = device_quant(h->qs);
             ra.scales = h->sscales;
-            int r = check_cuda(hm, launch_lazy_resid(ra, h->stream), "residual launch");
+            int r = check_cuda(hm, launch_lazy_resid(ra, h->stream, may_overlap(hm)), "residual launch");
             if (r == EA_OK) r = check_cuda(hm, cudaStreamSynchronize(h->stream), "stream synchronize");
             if (r != EA_OK) return r;
             p = h->rview;

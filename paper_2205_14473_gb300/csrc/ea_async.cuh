@@ -115,21 +115,38 @@ __device__ __forceinline__ void report_status(uint32_t *status, uint32_t code)
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// Launch `kernel` with programmatic stream serialization (see pdl_trigger / pdl_wait).
+// How an SM's 256 KB are split between L1 and shared memory, as a percentage of the largest shared
+// memory (228 KB): 44 asks for 100 KB, which holds the resident CTAs of every kernel but the staged
+// and grouped ones.  The rest is L1, where every load in flight takes its line: 8 TB/s at ~0.8 us is
+// ~40 KB of reads in flight per SM, more than the 28 KB that the largest split leaves.
+constexpr int kCarveoutPercent = 44;
+
+// Launch `kernel` with programmatic stream serialization (see pdl_trigger / pdl_wait), or, with
+// overlap = false, after everything before it on the stream has finished.
+//
+// An SM changes its split only when it is empty, and dependent launches fill it with the next
+// kernel's CTAs before the last one's have left, so a split stays as long as the chain does.  The
+// kernels of a chain therefore ask for the same one, and the first kernel after a staged or grouped
+// server, which run at the largest, is launched with overlap = false (the caller's job).  With the
+// driver's own choice, rounds queued one behind another ran their worker passes at the server's
+// split: 17.73 ms at d = 400,000,007, n = 8 (1-bit 4096-blocks), where a round on its own took
+// 14.02 ms; every kernel at the largest split measured 18.27 ms.
 template <class... KArgs, class... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                       Args &&...args)
+cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool overlap,
+                       int carveout, Args &&...args)
 {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    attr[0].val.sharedMemCarveout = carveout;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = overlap ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 

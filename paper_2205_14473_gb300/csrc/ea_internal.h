@@ -203,7 +203,8 @@ struct ApplyArgs {
     const float *scales;
 };
 
-cudaError_t launch_worker(int mode, const WorkerArgs &a, cudaStream_t s);
+// overlap: the launch may begin before its predecessor has finished (see launch_pdl).
+cudaError_t launch_worker(int mode, const WorkerArgs &a, cudaStream_t s, bool overlap = true);
 // The one-pass kernels of PASS_GROUPED (cooperative launches of `grid` CTAs) and their shapes.
 cudaError_t launch_worker_grouped(int mode, const WorkerArgs &a, int grid, cudaStream_t s);
 cudaError_t worker_grouped_shape(int mode, int qk, GroupedShape *out);
@@ -224,10 +225,10 @@ cudaError_t launch_server_for_qs(const ServerArgs &a, cudaStream_t s);
 
 // The server kernel for the placement and the broadcast quantizer kind of `a` (ea_api.cu).
 cudaError_t launch_server(int mode, const ServerArgs &a, cudaStream_t s);
-cudaError_t launch_finalize(const FinalizeArgs &a, cudaStream_t s);
-cudaError_t launch_encode(const EncodeArgs &a, cudaStream_t s);
-cudaError_t launch_lazy_resid(const ResidArgs &a, cudaStream_t s);
-cudaError_t launch_apply(const ApplyArgs &a, cudaStream_t s);
+cudaError_t launch_finalize(const FinalizeArgs &a, cudaStream_t s, bool overlap = true);
+cudaError_t launch_encode(const EncodeArgs &a, cudaStream_t s, bool overlap = true);
+cudaError_t launch_lazy_resid(const ResidArgs &a, cudaStream_t s, bool overlap = true);
+cudaError_t launch_apply(const ApplyArgs &a, cudaStream_t s, bool overlap = true);
 cudaError_t launch_fill(float *p, int64_t count, float value, cudaStream_t s);
 
 // Record the text that ea_last_error(NULL) reports for a failure that has no handle.

@@ -550,10 +550,10 @@ static cudaError_t launch_server_lazy_st(const ServerArgs &a, cudaStream_t s)
 {
     const dim3 grid(static_cast<unsigned>(a.n_tiles)), block(kThreads);
     switch (a.qw.kind) {
-    case QK_SIGN: return launch_pdl(server_lazy_kernel<MODE, QK_SIGN, STAGED>, grid, block, 0, s, a);
-    case QK_UNIF: return launch_pdl(server_lazy_kernel<MODE, QK_UNIF, STAGED>, grid, block, 0, s, a);
-    case QK_POW2: return launch_pdl(server_lazy_kernel<MODE, QK_POW2, STAGED>, grid, block, 0, s, a);
-    default: return launch_pdl(server_lazy_kernel<MODE, QK_IDENT, STAGED>, grid, block, 0, s, a);
+    case QK_SIGN: return launch_pdl(server_lazy_kernel<MODE, QK_SIGN, STAGED>, grid, block, 0, s, true, kCarveoutPercent, a);
+    case QK_UNIF: return launch_pdl(server_lazy_kernel<MODE, QK_UNIF, STAGED>, grid, block, 0, s, true, kCarveoutPercent, a);
+    case QK_POW2: return launch_pdl(server_lazy_kernel<MODE, QK_POW2, STAGED>, grid, block, 0, s, true, kCarveoutPercent, a);
+    default: return launch_pdl(server_lazy_kernel<MODE, QK_IDENT, STAGED>, grid, block, 0, s, true, kCarveoutPercent, a);
     }
 }
 
@@ -969,13 +969,11 @@ static cudaError_t launch_server_staged(const ServerArgs &a, cudaStream_t s)
     if (!attr_set[dev].load(std::memory_order_acquire)) {
         e = cudaFuncSetAttribute(server_staged_kernel<MODE, QW, QS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  kServerMaxDynSmem);
-        if (e == cudaSuccess)  // all of the SM's unified L1 / shared memory as shared memory
-            e = cudaFuncSetAttribute(server_staged_kernel<MODE, QW, QS>,
-                                     cudaFuncAttributePreferredSharedMemoryCarveout, 100);
         if (e != cudaSuccess) return e;
         attr_set[dev].store(true, std::memory_order_release);
     }
-    return launch_pdl(server_staged_kernel<MODE, QW, QS>, dim3(a.plan.grid), dim3(kThreads + 32), a.plan.smem_bytes, s, a);
+    return launch_pdl(server_staged_kernel<MODE, QW, QS>, dim3(a.plan.grid), dim3(kThreads + 32), a.plan.smem_bytes, s,
+                      true, cudaSharedmemCarveoutMaxShared, a);
 }
 
 
@@ -1021,16 +1019,16 @@ cudaError_t launch_server_for_qs(const ServerArgs &a, cudaStream_t s)
     switch (a.qw.kind) {
     case QK_SIGN:
         if (a.plan.enabled) return launch_server_staged<MODE, QK_SIGN, QS>(a, s);
-        return launch_pdl(server_kernel<MODE, QK_SIGN, QS>, grid, block, 0, s, a);
+        return launch_pdl(server_kernel<MODE, QK_SIGN, QS>, grid, block, 0, s, true, kCarveoutPercent, a);
     case QK_UNIF:
         if (a.plan.enabled) return launch_server_staged<MODE, QK_UNIF, QS>(a, s);
-        return launch_pdl(server_kernel<MODE, QK_UNIF, QS>, grid, block, 0, s, a);
+        return launch_pdl(server_kernel<MODE, QK_UNIF, QS>, grid, block, 0, s, true, kCarveoutPercent, a);
     case QK_POW2:
         if (a.plan.enabled) return launch_server_staged<MODE, QK_POW2, QS>(a, s);
-        return launch_pdl(server_kernel<MODE, QK_POW2, QS>, grid, block, 0, s, a);
+        return launch_pdl(server_kernel<MODE, QK_POW2, QS>, grid, block, 0, s, true, kCarveoutPercent, a);
     default:
         if (a.plan.enabled) return launch_server_staged<MODE, QK_IDENT, QS>(a, s);
-        return launch_pdl(server_kernel<MODE, QK_IDENT, QS>, grid, block, 0, s, a);
+        return launch_pdl(server_kernel<MODE, QK_IDENT, QS>, grid, block, 0, s, true, kCarveoutPercent, a);
     }
     return cudaGetLastError();
 }

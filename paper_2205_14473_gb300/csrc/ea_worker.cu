@@ -391,22 +391,22 @@ __global__ void fill_kernel(float *p, int64_t count, float value)
 // ------------------------------------------------------------------------------- launchers
 
 template <int MODE>
-static cudaError_t launch_worker_mode(const WorkerArgs &a, cudaStream_t s)
+static cudaError_t launch_worker_mode(const WorkerArgs &a, cudaStream_t s, bool overlap)
 {
     const dim3 grid(static_cast<unsigned>(a.n_tiles)), block(kThreads);
     if (a.pass == PASS_LAZY)
-        return a.q.kind == QK_SIGN ? launch_pdl(worker_lazy_kernel<MODE>, grid, block, 0, s, a) : cudaErrorNotSupported;
+        return a.q.kind == QK_SIGN ? launch_pdl(worker_lazy_kernel<MODE>, grid, block, 0, s, overlap, kCarveoutPercent, a) : cudaErrorNotSupported;
     switch (a.q.kind) {
-    case QK_SIGN: return launch_pdl(worker_kernel<MODE, QK_SIGN>, grid, block, 0, s, a);
-    case QK_UNIF: return launch_pdl(worker_kernel<MODE, QK_UNIF>, grid, block, 0, s, a);
-    case QK_POW2: return launch_pdl(worker_kernel<MODE, QK_POW2>, grid, block, 0, s, a);
-    default: return launch_pdl(worker_kernel<MODE, QK_IDENT>, grid, block, 0, s, a);
+    case QK_SIGN: return launch_pdl(worker_kernel<MODE, QK_SIGN>, grid, block, 0, s, overlap, kCarveoutPercent, a);
+    case QK_UNIF: return launch_pdl(worker_kernel<MODE, QK_UNIF>, grid, block, 0, s, overlap, kCarveoutPercent, a);
+    case QK_POW2: return launch_pdl(worker_kernel<MODE, QK_POW2>, grid, block, 0, s, overlap, kCarveoutPercent, a);
+    default: return launch_pdl(worker_kernel<MODE, QK_IDENT>, grid, block, 0, s, overlap, kCarveoutPercent, a);
     }
 }
 
-cudaError_t launch_worker(int mode, const WorkerArgs &a, cudaStream_t s)
+cudaError_t launch_worker(int mode, const WorkerArgs &a, cudaStream_t s, bool overlap)
 {
-    return mode == MODE_W ? launch_worker_mode<MODE_W>(a, s) : launch_worker_mode<MODE_S>(a, s);
+    return mode == MODE_W ? launch_worker_mode<MODE_W>(a, s, overlap) : launch_worker_mode<MODE_S>(a, s, overlap);
 }
 
 // The grouped kernel exists for the uniform grid (a scaled-sign message takes PASS_LAZY).
@@ -426,19 +426,19 @@ cudaError_t launch_worker_grouped(int mode, const WorkerArgs &a, int grid, cudaS
                           : grouped_launch(worker_grouped_kernel<MODE_S, QK_UNIF>, a, grid, slots, s);
 }
 
-cudaError_t launch_finalize(const FinalizeArgs &a, cudaStream_t s)
+cudaError_t launch_finalize(const FinalizeArgs &a, cudaStream_t s, bool overlap)
 {
     const dim3 grid(static_cast<unsigned>(a.q.grp.n_groups), static_cast<unsigned>(a.n_msgs > 1 ? a.n_msgs : 1)),
         block(kThreads);
-    if (a.q.kind == QK_SIGN) return launch_pdl(finalize_kernel<QK_SIGN>, grid, block, 0, s, a);
-    return launch_pdl(finalize_kernel<QK_UNIF>, grid, block, 0, s, a);
+    if (a.q.kind == QK_SIGN) return launch_pdl(finalize_kernel<QK_SIGN>, grid, block, 0, s, overlap, kCarveoutPercent, a);
+    return launch_pdl(finalize_kernel<QK_UNIF>, grid, block, 0, s, overlap, kCarveoutPercent, a);
 }
 
-cudaError_t launch_encode(const EncodeArgs &a, cudaStream_t s)
+cudaError_t launch_encode(const EncodeArgs &a, cudaStream_t s, bool overlap)
 {
     const dim3 grid(static_cast<unsigned>(a.n_tiles)), block(kThreads);
-    if (a.q.kind == QK_SIGN) return launch_pdl(encode_kernel<QK_SIGN>, grid, block, 0, s, a);
-    return launch_pdl(encode_kernel<QK_UNIF>, grid, block, 0, s, a);
+    if (a.q.kind == QK_SIGN) return launch_pdl(encode_kernel<QK_SIGN>, grid, block, 0, s, overlap, kCarveoutPercent, a);
+    return launch_pdl(encode_kernel<QK_UNIF>, grid, block, 0, s, overlap, kCarveoutPercent, a);
 }
 
 // The residual u - Q(u) of the u kept by PASS_LAZY, into a.out, one CTA per tile (a view of it).
@@ -458,21 +458,21 @@ __global__ void __launch_bounds__(kThreads) lazy_resid_kernel(const ResidArgs a)
         if (4 * slot_of(tile, k) < a.d) store4(a.out, slot_of(tile, k), a.d, u[k]);
 }
 
-cudaError_t launch_lazy_resid(const ResidArgs &a, cudaStream_t s)
+cudaError_t launch_lazy_resid(const ResidArgs &a, cudaStream_t s, bool overlap)
 {
     const dim3 grid(static_cast<unsigned>((a.d + kTile - 1) / kTile)), block(kThreads);
     if (a.q.kind != QK_SIGN) return cudaErrorNotSupported;
-    return launch_pdl(lazy_resid_kernel, grid, block, 0, s, a);
+    return launch_pdl(lazy_resid_kernel, grid, block, 0, s, overlap, kCarveoutPercent, a);
 }
 
-cudaError_t launch_apply(const ApplyArgs &a, cudaStream_t s)
+cudaError_t launch_apply(const ApplyArgs &a, cudaStream_t s, bool overlap)
 {
     const dim3 grid(static_cast<unsigned>((a.d + kTile - 1) / kTile)), block(kThreads);
     switch (a.q.kind) {
-    case QK_SIGN: return launch_pdl(apply_kernel<QK_SIGN>, grid, block, 0, s, a);
-    case QK_UNIF: return launch_pdl(apply_kernel<QK_UNIF>, grid, block, 0, s, a);
-    case QK_POW2: return launch_pdl(apply_kernel<QK_POW2>, grid, block, 0, s, a);
-    default: return launch_pdl(apply_kernel<QK_IDENT>, grid, block, 0, s, a);
+    case QK_SIGN: return launch_pdl(apply_kernel<QK_SIGN>, grid, block, 0, s, overlap, kCarveoutPercent, a);
+    case QK_UNIF: return launch_pdl(apply_kernel<QK_UNIF>, grid, block, 0, s, overlap, kCarveoutPercent, a);
+    case QK_POW2: return launch_pdl(apply_kernel<QK_POW2>, grid, block, 0, s, overlap, kCarveoutPercent, a);
+    default: return launch_pdl(apply_kernel<QK_IDENT>, grid, block, 0, s, overlap, kCarveoutPercent, a);
     }
 }
 
