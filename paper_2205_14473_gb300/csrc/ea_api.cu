@@ -190,10 +190,15 @@ int setup_quant(const ea_quantizer &q, int64_t d, const char *name, QHost &out)
             out.tile_group[t] = static_cast<int32_t>(gi);
         }
     }
-    // One pass when every group is exactly one tile; otherwise partial norms per (tile, group).
+    // One pass when every group is exactly one tile, or a tile is a whole number of groups that are
+    // a whole number of chunks each; otherwise partial norms per (tile, group).  512-blocks, 4-bit
+    // stochastic grid, d = 15,000,001: one worker message took 313 us in the three launches of the
+    // latter (104 us, 106 us for the 29,297 scales, 103 us).
     const bool block_tiles = out.gkind == GK_BLOCK && out.G == kTile;
     const bool single_tile = out.n_groups == 1 && d <= kTile;
-    if (block_tiles || single_tile) {
+    if (out.gkind == GK_BLOCK && out.log2G >= kLog2Chunk && out.G < kTile) {
+        out.pass = PASS_SHORT;
+    } else if (block_tiles || single_tile) {
         out.pass = PASS_FUSED;
     } else {
         out.pass = PASS_STASH;
@@ -410,14 +415,15 @@ uint64_t message_bits(const QHost &q, int64_t d)
 }
 
 // Shared-memory staging of the server's inputs (see server_staged_kernel): one stage holds a
-// tile's e_s (+ m_s, v_s) and the n workers' code chunks and scales.  Enabled when both messages
-// have one scale per 4096-tile (or none) and two stages fit in 200 KB.
+// tile's e_s (+ m_s, v_s) and the n workers' code chunks and scales.  Enabled when the scale groups of
+// both messages lie inside 4096-tiles (or there are none) and one stage fits in 200 KB.
 StagePlan make_server_plan(const ea_config &c, const QHost &qw, const QHost &qs, int64_t n_tiles, int sms)
 {
     StagePlan P{};
-    const bool qs_ok = !qs.has_scales || qs.pass == PASS_FUSED;
-    const bool qw_ok = !qw.has_scales || qw.pass == PASS_FUSED;
-    if (!qs_ok || !qw_ok || sms <= 0) return P;
+    auto in_tile = [](const QHost &q) { return !q.has_scales || q.pass == PASS_FUSED || q.pass == PASS_SHORT; };
+    if (!in_tile(qs) || !in_tile(qw) || sms <= 0) return P;
+    P.short_blocks = qs.pass == PASS_SHORT || qw.pass == PASS_SHORT;
+    const uint32_t scales = qw.pass == PASS_SHORT ? static_cast<uint32_t>(kTile / qw.G) : 1u;  // of one worker
     const bool server_adam = c.placement == EA_ADAM_AT_SERVER;
     uint32_t off = 0;
     P.off_a = off;
@@ -434,7 +440,7 @@ StagePlan make_server_plan(const ea_config &c, const QHost &qw, const QHost &qs,
     if (codes > 100 * 1024) return P;
     off += static_cast<uint32_t>(codes);
     P.off_scales = off;
-    off += static_cast<uint32_t>(align_up(4 * static_cast<size_t>(c.n), 16));
+    off += static_cast<uint32_t>(align_up(4 * static_cast<size_t>(c.n) * scales, 16));
     P.stage_bytes = static_cast<uint32_t>(align_up(off, 128));
     // As many resident CTAs per SM as shared memory holds with one stage each (the kernel's
     // registers allow server_ctas_per_sm; the EA_Q_* kinds are the kernels' QK_* values), then as

@@ -287,7 +287,7 @@ __device__ __forceinline__ float decode1(uint32_t code, float s, const QParams &
 }
 
 template <int QK>
-__device__ __forceinline__ constexpr bool has_scale()
+__host__ __device__ __forceinline__ constexpr bool has_scale()
 {
     return QK == QK_SIGN || QK == QK_UNIF;
 }
@@ -359,6 +359,16 @@ __device__ __forceinline__ int64_t tile_single_group(const Grouping &g, int64_t 
     }
     const int64_t g0 = g.tile_group[tile];
     return g.offsets[g0 + 1] > last ? g0 : -1;
+}
+
+// Short blocks: power-of-two blocks of 128 .. 2048 coordinates (of 4096: the same with one block per
+// tile).  A chunk, the 128 coordinates that one warp holds in one slot, then lies in one block and a
+// block in one tile, so a tile's scales are formed inside its CTA (chunk_scales) and a warp reads
+// one scale per slot.  log2 of the chunks per block; 5 (the whole tile) for every other grouping that
+// has one scale per tile.
+__host__ __device__ __forceinline__ int chunk_shift(const Grouping &g)
+{
+    return (g.gkind == GK_BLOCK && g.log2G >= kLog2Chunk && g.log2G < 12) ? g.log2G - kLog2Chunk : 5;
 }
 
 // The segments (GK_SEG) of one tile, for per-coordinate lookups from shared memory: the tile's

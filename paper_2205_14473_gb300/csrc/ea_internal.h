@@ -21,6 +21,8 @@ constexpr uint32_t kServerMaxDynSmem = 200 * 1024;
 constexpr uint32_t kSmemPerSm = 228 * 1024;
 constexpr uint32_t kSmemReservedPerCta = 1024;
 constexpr int kWarps = kThreads / 32;
+// A chunk: the coordinates of one warp in one slot; a tile has kChunks of them.
+constexpr int kLog2Chunk = 7, kChunk = 1 << kLog2Chunk, kChunks = kTile / kChunk;
 // Shared-memory staging of a server tile's worker scales: at most kStagedTileGroups of Q_w's groups
 // meet one tile, and n times that many scales fit in kWorkerScales.
 constexpr int kWorkerScales = 512;
@@ -72,7 +74,7 @@ inline float bias_correction(float beta, int64_t t1)
 
 // How the scale of a message is formed.
 enum Pass : int {
-    PASS_FUSED = 0,   // every group lies inside one tile: reduce, encode and store in one pass
+    PASS_FUSED = 0,   // one group per tile: reduce, encode and store in one pass
     PASS_STASH = 1,   // groups span tiles: store the input in the residual buffer plus one
                       // partial norm per (tile, group); finalize_kernel and encode_kernel finish
     PASS_GROUPED = 2, // groups span tiles, one cooperative pass: the input stays in shared memory
@@ -81,6 +83,8 @@ enum Pass : int {
                       // writes them with the partial norms and keeps u itself in the residual
                       // buffer; finalize_kernel forms the scales, and e = u - Q(u) is formed from
                       // (u, s) where it is next needed (the next round's pass, or a view)
+    , PASS_SHORT = 4  // several groups per tile, each a whole number of warp slots (power-of-two
+                      // blocks of 128 .. 2048): one pass, a scale per chunk (see chunk_scales)
 };
 
 // The one-pass plan for scale groups that span tiles.  The vector is cut into waves, coordinate
@@ -129,6 +133,7 @@ struct WorkerArgs {
 // tile's inputs; byte offsets are relative to the stage start and 128-byte aligned.
 struct StagePlan {
     int enabled;               // 0: use the direct-load kernel
+    int short_blocks;          // Q_w or Q_s has several scales per tile (PASS_SHORT)
     int stages;                // pipeline depth
     int grid;                  // persistent CTAs
     uint32_t stage_bytes;      // bytes of one stage
@@ -136,7 +141,7 @@ struct StagePlan {
     uint32_t off_a, off_b, off_c, off_d;  // up to four 16 KB state tiles (kernel-specific meaning)
     uint32_t off_codes;        // n code chunks of code_chunk bytes
     uint32_t code_chunk;       // bytes of one worker's codes for one tile (4096 b / 8)
-    uint32_t off_scales;       // n worker scales (binary32)
+    uint32_t off_scales;       // the n workers' scales of the tile (binary32)
 };
 
 struct ServerArgs {
@@ -222,6 +227,8 @@ cudaError_t server_grouped_shape(int mode, int qw, int qs, GroupedShape *out);
 // instantiated only in its own translation unit, ea_server_<mode>_q<QS>.cu.
 template <int MODE, int QS>
 cudaError_t launch_server_for_qs(const ServerArgs &a, cudaStream_t s);
+template <int MODE, int QS>
+cudaError_t launch_server_short(const ServerArgs &a, cudaStream_t s);
 
 // The server kernel for the placement and the broadcast quantizer kind of `a` (ea_api.cu).
 cudaError_t launch_server(int mode, const ServerArgs &a, cudaStream_t s);

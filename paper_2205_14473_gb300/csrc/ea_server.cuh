@@ -682,7 +682,9 @@ __device__ __forceinline__ void unif_decode_sum(const unsigned char *codes, int 
 // NW: the worker count when it is 8, known at compile time (the per-worker bounds, the average's
 // division and the decode loops then fold; for scaled-sign workers the table is the whole average
 // and the per-worker path is not compiled in), or 0 for a count known at run time.
-template <int MODE, int QW, int QS, bool FULL, int NW>
+// SHORT: one of the messages has several scales per tile (short blocks): the workers' values are
+// decoded with the chunk's scale, one per warp, slot and worker, and Q_s takes chunk_scales.
+template <int MODE, int QW, int QS, bool FULL, int NW, bool SHORT>
 __device__ __forceinline__ bool server_staged_tile(const ServerArgs &a, int64_t tile, const unsigned char *st,
                                                    bool ok, uint64_t *empty, int Lw, float Lwf, const float *utab,
                                                    float *wtab, const uint32_t (&flip)[8], TileSmem &sm)
@@ -700,8 +702,43 @@ __device__ __forceinline__ bool server_staged_tile(const ServerArgs &a, int64_t 
     bool done = false;
     // wtab is rebuilt below; the previous tile's reads of it end at its scale reduction's barrier,
     // which a Q_s without scales does not have
-    if constexpr (!has_scale<QS>() && (QW == QK_SIGN || QW == QK_UNIF)) compute_sync();
-    if constexpr (QW == QK_SIGN) {
+    if constexpr (!SHORT && !has_scale<QS>() && (QW == QK_SIGN || QW == QK_UNIF)) compute_sync();
+    if constexpr (SHORT) {
+        done = true;
+        if (!compute_all(ok)) return false;
+#pragma unroll
+        for (int k = 0; k < kSlots; ++k)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[k][i] = 0.0f;
+        const int sh = chunk_shift(a.qw.grp), per = kChunks >> sh;  // scales of one worker in the tile
+        const int warp = threadIdx.x >> 5;
+#pragma unroll 2
+        for (int w = 0; w < n; ++w) {
+            const uint32_t *cw = reinterpret_cast<const uint32_t *>(st + P.off_codes + static_cast<size_t>(w) * P.code_chunk);
+            const float *ws = sc + w * per;
+#pragma unroll
+            for (int k = 0; k < kSlots; ++k) {
+                const float s = has_scale<QW>() ? ws[(k * kWarps + warp) >> sh] : 0.0f;
+                const int ls = k * kThreads + threadIdx.x;
+                uint32_t c[4];
+                if constexpr (QW == QK_SIGN) {
+                    const uint32_t nib = cw[ls >> 3] >> (4 * (ls & 7));
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) c[i] = (nib >> i) & 1u;
+                } else {
+                    load_codes4_smem(cw, ls, bw, c);
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    acc[k][i] = __fadd_rn(acc[k][i], decode1<QW>(c[i], s, a.qw, Lwf, Lw, utab));
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < kSlots; ++k)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[k][i] = pow2n ? __fmul_rn(acc[k][i], inv_n) : __fdiv_rn(acc[k][i], nf);
+    }
+    if constexpr (!SHORT && QW == QK_SIGN) {
       {
         done = NW == 8 || n <= 8;
         // Scaled-sign workers: the worker-order sum of the first m = min(n, 8) workers depends
@@ -751,7 +788,7 @@ __device__ __forceinline__ bool server_staged_tile(const ServerArgs &a, int64_t 
         }
       }
     }
-    if (!done) {
+    if (!SHORT && !done) {
         // scaled-sign workers (n > 8): acc already holds the sum of workers 0..7
         constexpr bool partial = QW == QK_SIGN;
         if constexpr (!partial) {
@@ -834,6 +871,7 @@ __device__ __forceinline__ bool server_staged_tile(const ServerArgs &a, int64_t 
             float step = acc[k][i];
             if (MODE == MODE_S) step = adam_step(step, ms[i], vs[i], a.hp);
             u[i] = (FULL || j0 + i < d) ? __fadd_rn(step, es[i]) : 0.0f;  // invalid u are 0
+            if constexpr (SHORT) continue;  // chunk_scales forms its own sums
             if constexpr (QS == QK_SIGN) df_accumulate(l1, fabsf(u[i]));
             else mx = fmaxf(mx, fabsf(u[i]));
         }
@@ -843,8 +881,15 @@ __device__ __forceinline__ bool server_staged_tile(const ServerArgs &a, int64_t 
             store4<FULL>(a.vs, q, d, vs);
         }
     }
-    finish_tile_smem<QS, FULL, false>(ubuf, l1, mx, tile, d, a.qs, a.words, a.scales, a.es, a.ef, a.seed,
-                                      static_cast<uint32_t>(a.n), a.t, sm);
+    if constexpr (SHORT && has_scale<QS>()) {
+        chunk_scales<QS>(USmem{ubuf}, tile, d, chunk_shift(a.qs.grp), a.scales, sm);
+        encode_store<QS, FULL, false>(USmem{ubuf}, ChunkScales{sm.csc}, tile, d, a.qs, a.words, a.es, a.ef, a.seed,
+                                      static_cast<uint32_t>(a.n), a.t,
+                                      (QS == QK_UNIF && a.qs.bits <= 8) ? sm.qtab : nullptr);
+    } else {
+        finish_tile_smem<QS, FULL, false>(ubuf, l1, mx, tile, d, a.qs, a.words, a.scales, a.es, a.ef, a.seed,
+                                          static_cast<uint32_t>(a.n), a.t, sm);
+    }
     // the stage is no longer read: hand it back to the producer
     __syncwarp();
     if ((threadIdx.x & 31) == 0) mbar_arrive(empty);
@@ -856,8 +901,9 @@ __device__ __forceinline__ bool server_staged_tile(const ServerArgs &a, int64_t 
 // m_s, v_s with Adam at the server) and the n workers' code chunks with bulk copies, and the n
 // worker scales with 4-byte cp.async, into a ring of stages guarded by full/empty mbarriers; the
 // compute warps decode, average, re-quantize and write e_s and the broadcast straight to HBM.
-// Used when Q_s scales are per 4096-tile (or absent) and Q_w's are per 4096-tile (or absent).
-template <int MODE, int QW, int QS>
+// Used when the scale groups of Q_s and Q_w lie inside 4096-tiles (or are absent); SHORT: some tile
+// holds several.
+template <int MODE, int QW, int QS, bool SHORT>
 __global__ void __launch_bounds__(kThreads + 32, server_ctas_per_sm(MODE, QW, QS)) server_staged_kernel(const ServerArgs a)
 {
     extern __shared__ __align__(128) unsigned char dsm[];
@@ -920,7 +966,15 @@ __global__ void __launch_bounds__(kThreads + 32, server_ctas_per_sm(MODE, QW, QS
             }
             if (scaled_w) {
                 float *sc = reinterpret_cast<float *>(st + P.off_scales);
-                for (int w = lane; w < a.n; w += 32) cp_async4(sc + w, a.wscales + w * a.wscales_stride + tile);
+                if constexpr (SHORT) {
+                    // worker w's scales of the tile, at w * per; past the last group the stream's
+                    // padding is read (a multiple of 64 scales)
+                    const int lp = 5 - chunk_shift(a.qw.grp), per = 1 << lp;
+                    for (int i = lane; i < a.n * per; i += 32)
+                        cp_async4(sc + i, a.wscales + (i >> lp) * a.wscales_stride + tile * per + (i & (per - 1)));
+                } else {
+                    for (int w = lane; w < a.n; w += 32) cp_async4(sc + w, a.wscales + w * a.wscales_stride + tile);
+                }
                 cp_async_arrive_noinc(&full[s]);
             }
         }
@@ -945,10 +999,17 @@ __global__ void __launch_bounds__(kThreads + 32, server_ctas_per_sm(MODE, QW, QS
         // bounded wait; the tile's first barrier makes every compute thread agree on the outcome
         const bool ok = mbar_wait(&full[s], static_cast<uint32_t>((it / S) & 1));
         const unsigned char *st = stage0 + static_cast<size_t>(s) * P.stage_bytes;
-        const bool go = (tile + 1) * kTile <= d
-            ? (n8 ? server_staged_tile<MODE, QW, QS, true, 8>(a, tile, st, ok, &empty[s], Lw, Lwf, use_tab ? utab : nullptr, wtab, flip, sm)
-                  : server_staged_tile<MODE, QW, QS, true, 0>(a, tile, st, ok, &empty[s], Lw, Lwf, use_tab ? utab : nullptr, wtab, flip, sm))
-            : server_staged_tile<MODE, QW, QS, false, 0>(a, tile, st, ok, &empty[s], Lw, Lwf, use_tab ? utab : nullptr, wtab, flip, sm);
+        const float *ut = use_tab ? utab : nullptr;
+        const bool whole = (tile + 1) * kTile <= d;
+        bool go;
+        if constexpr (SHORT) {
+            go = whole ? server_staged_tile<MODE, QW, QS, true, 0, true>(a, tile, st, ok, &empty[s], Lw, Lwf, ut, wtab, flip, sm)
+                       : server_staged_tile<MODE, QW, QS, false, 0, true>(a, tile, st, ok, &empty[s], Lw, Lwf, ut, wtab, flip, sm);
+        } else {
+            go = !whole ? server_staged_tile<MODE, QW, QS, false, 0, false>(a, tile, st, ok, &empty[s], Lw, Lwf, ut, wtab, flip, sm)
+                 : n8   ? server_staged_tile<MODE, QW, QS, true, 8, false>(a, tile, st, ok, &empty[s], Lw, Lwf, ut, wtab, flip, sm)
+                        : server_staged_tile<MODE, QW, QS, true, 0, false>(a, tile, st, ok, &empty[s], Lw, Lwf, ut, wtab, flip, sm);
+        }
         if (!go) {
             if (threadIdx.x == 0) report_status(a.status, kStatusTimeout);
             break;
@@ -956,8 +1017,8 @@ __global__ void __launch_bounds__(kThreads + 32, server_ctas_per_sm(MODE, QW, QS
     }
 }
 
-template <int MODE, int QW, int QS>
-static cudaError_t launch_server_staged(const ServerArgs &a, cudaStream_t s)
+template <int MODE, int QW, int QS, bool SHORT>
+static cudaError_t launch_server_staged_kernel(const ServerArgs &a, cudaStream_t s)
 {
     // Function attributes are per device: one flag per device ordinal.  Two threads that race on a
     // first launch both set the same values, which is harmless.
@@ -967,15 +1028,21 @@ static cudaError_t launch_server_staged(const ServerArgs &a, cudaStream_t s)
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
     if (!attr_set[dev].load(std::memory_order_acquire)) {
-        e = cudaFuncSetAttribute(server_staged_kernel<MODE, QW, QS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(server_staged_kernel<MODE, QW, QS, SHORT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  kServerMaxDynSmem);
         if (e != cudaSuccess) return e;
         attr_set[dev].store(true, std::memory_order_release);
     }
-    return launch_pdl(server_staged_kernel<MODE, QW, QS>, dim3(a.plan.grid), dim3(kThreads + 32), a.plan.smem_bytes, s,
-                      true, cudaSharedmemCarveoutMaxShared, a);
+    return launch_pdl(server_staged_kernel<MODE, QW, QS, SHORT>, dim3(a.plan.grid), dim3(kThreads + 32),
+                      a.plan.smem_bytes, s, true, cudaSharedmemCarveoutMaxShared, a);
 }
 
+template <int MODE, int QW, int QS>
+static cudaError_t launch_server_staged(const ServerArgs &a, cudaStream_t s)
+{
+    if (a.plan.short_blocks) return launch_server_short<MODE, QS>(a, s);
+    return launch_server_staged_kernel<MODE, QW, QS, false>(a, s);
+}
 
 // The grouped server for one placement and broadcast kind (the uniform grid only).
 template <int MODE, int QS>

@@ -1,0 +1,5 @@
+// The staged server of messages with several scales per tile: Adam at the workers, broadcast kind QK_SIGN.
+#include "ea_server_short.cuh"
+namespace ea {
+template cudaError_t launch_server_short<MODE_W, QK_SIGN>(const ServerArgs &a, cudaStream_t s);
+}

@@ -1,0 +1,5 @@
+// The staged server of messages with several scales per tile: Adam at the workers, broadcast kind QK_POW2.
+#include "ea_server_short.cuh"
+namespace ea {
+template cudaError_t launch_server_short<MODE_W, QK_POW2>(const ServerArgs &a, cudaStream_t s);
+}

@@ -14,6 +14,7 @@ struct TileSmem {
     uint32_t redm[kWarps];
     double bcast;
     float bcastf;
+    float csc[kChunks];  // PASS_SHORT: the scale of each chunk
     float qtab[256];  // the uniform grid's fl(i / L) of the tile's own quantizer (build_qtab)
 };
 
@@ -42,6 +43,80 @@ struct USmem {
         o[0] = v.x, o[1] = v.y, o[2] = v.z, o[3] = v.w;
     }
 };
+
+// The scale of a tile's encode: one for the tile (a float), or one per chunk (short blocks), read
+// once per slot by each warp.
+struct ChunkScales {
+    const float *csc;
+};
+__device__ __forceinline__ float slot_scale(float s, int) { return s; }
+__device__ __forceinline__ float slot_scale(ChunkScales s, int k) { return s.csc[k * kWarps + (threadIdx.x >> 5)]; }
+template <class Scale>
+constexpr bool kPerSlot = false;
+template <>
+constexpr bool kPerSlot<ChunkScales> = true;
+
+// PASS_SHORT: the scales of the tile's blocks of 2^sh chunks, from u read through `src`, into
+// sm.csc (one per chunk) and scales[].  A warp reduces its four chunks at once: for the scaled sign
+// the compensated pairs of four slots are exchanged by halves, so that five shuffle levels take six
+// pair additions (each lane keeps 2, 1, then 1 pair) instead of twenty.  Warp 0 then combines the
+// 32 chunk results, one per lane, over the blocks.  Two barriers; all 256 threads call it.
+template <int QK, class USrc>
+__device__ __forceinline__ void chunk_scales(const USrc &src, int64_t tile, int64_t d, int sh, float *scales,
+                                             TileSmem &sm)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    auto shfl = [](DF v, int o) { return DF{__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)}; };
+    static_assert(kSlots == 4 && kChunks == 32, "two halvings over the slots; one chunk per lane of warp 0");
+    if constexpr (QK == QK_SIGN) {
+        DF p[kSlots];
+#pragma unroll
+        for (int k = 0; k < kSlots; ++k) {
+            float uk[4];
+            src.get(k, uk);
+            p[k] = DF{0.0f, 0.0f};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) df_accumulate(p[k], fabsf(uk[i]));  // invalid u are 0
+        }
+        const bool h16 = lane & 16, h8 = lane & 8;
+        const DF a = df_add(h16 ? p[2] : p[0], shfl(h16 ? p[0] : p[2], 16));
+        const DF b = df_add(h16 ? p[3] : p[1], shfl(h16 ? p[1] : p[3], 16));
+        DF c = df_add(h8 ? b : a, shfl(h8 ? a : b, 8));  // lane: slot lane / 8
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) c = df_add(c, shfl(c, o));
+        if ((lane & 7) == 0) sm.red256[(lane >> 3) * kWarps + warp] = c;
+    } else {
+#pragma unroll
+        for (int k = 0; k < kSlots; ++k) {
+            float uk[4];
+            src.get(k, uk);
+            const float mx = fmaxf(fmaxf(fabsf(uk[0]), fabsf(uk[1])), fmaxf(fabsf(uk[2]), fabsf(uk[3])));
+            const uint32_t m = __reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(0.0f, mx)));
+            if (lane == 0) sm.red256[k * kWarps + warp].hi = __uint_as_float(m);
+        }
+    }
+    compute_sync();
+    if (warp == 0) {
+        const int64_t base = tile * kTile + ((lane >> sh) << (sh + kLog2Chunk));  // the block's first coordinate
+        const int64_t left = d - base;
+        const int len = left < (kChunk << sh) ? static_cast<int>(left) : kChunk << sh;
+        float s = 0.0f;
+        if constexpr (QK == QK_SIGN) {
+            DF v = sm.red256[lane];
+            for (int o = 1; o < (1 << sh); o <<= 1) v = df_add(v, shfl(v, o));
+            if (len > 0 && (len & (len - 1)) == 0)
+                s = __fmul_rn(__fadd_rn(v.hi, v.lo), __uint_as_float(static_cast<uint32_t>(127 - __ffs(len) + 1) << 23));
+            else if (len > 0)
+                s = sign_scale(static_cast<double>(v.hi) + static_cast<double>(v.lo), len);
+        } else {
+            s = sm.red256[lane].hi;
+            for (int o = 1; o < (1 << sh); o <<= 1) s = fmaxf(s, __shfl_xor_sync(0xffffffffu, s, o));
+        }
+        sm.csc[lane] = s;
+        if (len > 0 && (lane & ((1 << sh) - 1)) == 0) scales[tile * (kChunks >> sh) + (lane >> sh)] = s;
+    }
+    compute_sync();
+}
 
 // Example 1's grid index of u (|u| <= s, s > 0) without a division.  z = RN(u / s) and y = RN(z L)
 // are stood in for by z' = RN(u r), y' = RN(z' L) with r = RN(1 / s), which the caller computes
@@ -77,8 +152,8 @@ enum EncVar : int { ENC_PLAIN = 0, ENC_UZERO, ENC_UDET_TAB, ENC_UDET_DIV, ENC_US
 
 // BITS: the code width as a compile-time constant (0: code_bits of the kind, or q.bits).
 // Only the coordinates of [lo, d) are encoded and stored (lo: 0, or the start of a word and a slot).
-template <int QK, bool FULL, bool BALLOT, int VAR, int BITS, class USrc>
-__device__ __forceinline__ void encode_store_v(const USrc &src, float s, int64_t tile, int64_t d,
+template <int QK, bool FULL, bool BALLOT, int VAR, int BITS, class USrc, class Scale>
+__device__ __forceinline__ void encode_store_v(const USrc &src, Scale sc, int64_t tile, int64_t d,
                                                const QParams &q, uint32_t *words, float *resid, int ef,
                                                uint64_t seed, uint32_t id, uint32_t t, const float *qtab,
                                                int64_t lo = 0)
@@ -89,15 +164,18 @@ __device__ __forceinline__ void encode_store_v(const USrc &src, float s, int64_t
     const int bits = BITS ? BITS : code_bits<QK>(q);
     const int L = (QK == QK_UNIF) ? unif_L(bits) : 0;
     const float Lf = static_cast<float>(L);
-    float r = 0.0f, m = 0.0f;
-    if (GRID) {
-        r = (s >= 0x1p-125f && s <= 0x1p125f) ? __frcp_rn(s) : __int_as_float(0x7fc00000);
-        m = __fmul_rn(Lf, 0x1p-20f);
-    }
+    float s = 0.0f, r = 0.0f, m = 0.0f;
+    auto take_scale = [&](int k) {  // a zero scale gives r = NaN, and unif_index then index 0
+        s = slot_scale(sc, k);
+        if (GRID) r = (s >= 0x1p-125f && s <= 0x1p125f) ? __frcp_rn(s) : __int_as_float(0x7fc00000);
+    };
+    if (GRID) m = __fmul_rn(Lf, 0x1p-20f);
+    if constexpr (!kPerSlot<Scale>) take_scale(0);
 #pragma unroll
     for (int k = 0; k < kSlots; ++k) {
         const int64_t qs = slot_of(tile, k);
         const int64_t j0 = 4 * qs;
+        if constexpr (kPerSlot<Scale>) take_scale(k);
         float U[4] = {0.f, 0.f, 0.f, 0.f};
         if (STO && (FULL || j0 < d)) uniforms4(seed, id, t, j0, U);
         float uk[4];
@@ -140,44 +218,46 @@ __device__ __forceinline__ void encode_store_v(const USrc &src, float s, int64_t
 // FULL: the whole tile lies inside [0, d), so no coordinate needs a bounds check.
 // Example 1 with a compile-time width: for b <= 8 the caller passes qtab (fl(i/L) of the tile's
 // quantizer) and the decode is a table read; 16-bit grids divide.
-template <int QK, bool FULL, bool BALLOT, int BITS, class USrc>
-__device__ __forceinline__ void encode_store_unif(const USrc &u, float s, int64_t tile, int64_t d,
+template <int QK, bool FULL, bool BALLOT, int BITS, class USrc, class Scale>
+__device__ __forceinline__ void encode_store_unif(const USrc &u, Scale sc, int64_t tile, int64_t d,
                                                   const QParams &q, uint32_t *words, float *resid, int ef,
                                                   uint64_t seed, uint32_t id, uint32_t t, const float *qtab,
                                                   int64_t lo = 0)
 {
     constexpr bool tab = BITS <= 8;
-    if (!(s > 0.0f))
-        encode_store_v<QK, FULL, BALLOT, ENC_UZERO, BITS>(u, s, tile, d, q, words, resid, ef, seed, id, t, qtab, lo);
+    bool zero = false;
+    if constexpr (!kPerSlot<Scale>) zero = !(sc > 0.0f);
+    if (zero)
+        encode_store_v<QK, FULL, BALLOT, ENC_UZERO, BITS>(u, sc, tile, d, q, words, resid, ef, seed, id, t, qtab, lo);
     else if (q.stochastic)
-        encode_store_v<QK, FULL, BALLOT, tab ? ENC_USTO_TAB : ENC_USTO_DIV, BITS>(u, s, tile, d, q, words, resid, ef,
+        encode_store_v<QK, FULL, BALLOT, tab ? ENC_USTO_TAB : ENC_USTO_DIV, BITS>(u, sc, tile, d, q, words, resid, ef,
                                                                                seed, id, t, qtab, lo);
     else
-        encode_store_v<QK, FULL, BALLOT, tab ? ENC_UDET_TAB : ENC_UDET_DIV, BITS>(u, s, tile, d, q, words, resid, ef,
+        encode_store_v<QK, FULL, BALLOT, tab ? ENC_UDET_TAB : ENC_UDET_DIV, BITS>(u, sc, tile, d, q, words, resid, ef,
                                                                                seed, id, t, qtab, lo);
 }
 
 // Encode and store a tile; the variant (and a configured code width) is chosen once per tile.
-template <int QK, bool FULL, bool BALLOT, class USrc>
-__device__ __forceinline__ void encode_store(const USrc &u, float s, int64_t tile, int64_t d,
+template <int QK, bool FULL, bool BALLOT, class USrc, class Scale>
+__device__ __forceinline__ void encode_store(const USrc &u, Scale sc, int64_t tile, int64_t d,
                                              const QParams &q, uint32_t *words, float *resid, int ef,
                                              uint64_t seed, uint32_t id, uint32_t t, const float *qtab,
                                              int64_t lo = 0)
 {
     if constexpr (QK == QK_UNIF) {
         switch (q.bits) {  // the widths ea_init accepts
-        case 2: encode_store_unif<QK, FULL, BALLOT, 2>(u, s, tile, d, q, words, resid, ef, seed, id, t, qtab, lo); break;
-        case 4: encode_store_unif<QK, FULL, BALLOT, 4>(u, s, tile, d, q, words, resid, ef, seed, id, t, qtab, lo); break;
-        case 8: encode_store_unif<QK, FULL, BALLOT, 8>(u, s, tile, d, q, words, resid, ef, seed, id, t, qtab, lo); break;
-        default: encode_store_unif<QK, FULL, BALLOT, 16>(u, s, tile, d, q, words, resid, ef, seed, id, t, qtab, lo); break;
+        case 2: encode_store_unif<QK, FULL, BALLOT, 2>(u, sc, tile, d, q, words, resid, ef, seed, id, t, qtab, lo); break;
+        case 4: encode_store_unif<QK, FULL, BALLOT, 4>(u, sc, tile, d, q, words, resid, ef, seed, id, t, qtab, lo); break;
+        case 8: encode_store_unif<QK, FULL, BALLOT, 8>(u, sc, tile, d, q, words, resid, ef, seed, id, t, qtab, lo); break;
+        default: encode_store_unif<QK, FULL, BALLOT, 16>(u, sc, tile, d, q, words, resid, ef, seed, id, t, qtab, lo); break;
         }
     } else if constexpr (QK == QK_POW2) {
         if (q.bits == 4)
-            encode_store_v<QK, FULL, BALLOT, ENC_PLAIN, 4>(u, s, tile, d, q, words, resid, ef, seed, id, t, qtab, lo);
+            encode_store_v<QK, FULL, BALLOT, ENC_PLAIN, 4>(u, sc, tile, d, q, words, resid, ef, seed, id, t, qtab, lo);
         else
-            encode_store_v<QK, FULL, BALLOT, ENC_PLAIN, 8>(u, s, tile, d, q, words, resid, ef, seed, id, t, qtab, lo);
+            encode_store_v<QK, FULL, BALLOT, ENC_PLAIN, 8>(u, sc, tile, d, q, words, resid, ef, seed, id, t, qtab, lo);
     } else {
-        encode_store_v<QK, FULL, BALLOT, ENC_PLAIN, 0>(u, s, tile, d, q, words, resid, ef, seed, id, t, qtab, lo);
+        encode_store_v<QK, FULL, BALLOT, ENC_PLAIN, 0>(u, sc, tile, d, q, words, resid, ef, seed, id, t, qtab, lo);
     }
 }
 
@@ -208,10 +288,11 @@ constexpr int PASS_LAZY_ONE = 16;
 
 // The tile's end for a quantizer with scale groups, u read through `src` (URegs or USmem).
 //   PASS_FUSED: the tile is exactly one scale group (blocks of 4096): reduce, encode, store.
+//   PASS_SHORT: the tile is several groups of whole chunks: the same with a scale per chunk.
 //   PASS_STASH: store u in resid and one partial norm per (tile, group) for finalize/encode.
 // BALLOT: pack 1-bit codes with __ballot_sync (worker kernels) or with shuffles (the server, whose
 // tile loop is instruction-bound).
-// PASS: PASS_FUSED or PASS_STASH as a compile-time constant (the other path is then not compiled
+// PASS: PASS_FUSED, PASS_SHORT or PASS_STASH as a compile-time constant (the other path is then not compiled
 // in), or -1 to follow `pass`.
 // part_idx (PASS_LAZY_ONE): where the tile's partial norm goes, looked up early by the caller.
 template <int QK, bool FULL = false, bool BALLOT = true, int PASS = -1, class USrc>
@@ -253,6 +334,12 @@ __device__ __forceinline__ void finish_tile(const USrc &src, int64_t tile, int64
             if (threadIdx.x == 0) scales[tile] = s;
             // sm.qtab was filled by build_qtab before the reduction's barrier
             encode_store<QK, FULL, BALLOT>(src, s, tile, d, q, words, resid, ef, seed, id, t,
+                                           (QK == QK_UNIF && q.bits <= 8) ? sm.qtab : nullptr);
+            return;
+        }
+        if (pass == PASS_SHORT) {
+            chunk_scales<QK>(src, tile, d, chunk_shift(q.grp), scales, sm);
+            encode_store<QK, FULL, BALLOT>(src, ChunkScales{sm.csc}, tile, d, q, words, resid, ef, seed, id, t,
                                            (QK == QK_UNIF && q.bits <= 8) ? sm.qtab : nullptr);
             return;
         }

@@ -102,6 +102,9 @@ __global__ void __launch_bounds__(kThreads, MODE == MODE_S ? 4 : 3)
     if (a.pass == PASS_FUSED) {
         if (full) worker_tile<MODE, QK, true, PASS_FUSED>(a, tile, ubuf, sm);
         else worker_tile<MODE, QK, false, PASS_FUSED>(a, tile, ubuf, sm);
+    } else if (has_scale<QK>() && a.pass == PASS_SHORT) {
+        if (full) worker_tile<MODE, QK, true, PASS_SHORT>(a, tile, ubuf, sm);
+        else worker_tile<MODE, QK, false, PASS_SHORT>(a, tile, ubuf, sm);
     } else {
         if (full) worker_tile<MODE, QK, true, PASS_STASH>(a, tile, ubuf, sm);
         else worker_tile<MODE, QK, false, PASS_STASH>(a, tile, ubuf, sm);
@@ -280,9 +283,12 @@ __global__ void __launch_bounds__(kThreads, 2) encode_kernel(const EncodeArgs a)
 // 4 B read + 4 B written + b/8 B of code.  BITS: the code width as a compile-time constant.  The
 // loads of x and of the raw code words are issued first; the fl(i/L) table of the uniform grid
 // (b <= 8) is built while they are in flight, and the codes are unpacked after its barrier.
-// TILE_SCALE: the scales are 4096-blocks, one per tile (then no group lookup is compiled in; that
-// instantiation measured 4% faster than one carrying the lookup as well).
-template <int QK, bool FULL, int BITS, bool TILE_SCALE>
+// SCALES: where a coordinate's scale is.  AS_TILE: 4096-blocks, one per tile (then no group lookup is
+// compiled in; that instantiation measured 4% faster than one carrying the lookup as well);
+// AS_SLOT: power-of-two blocks of 128 and more, one per warp and slot, loaded with the slot;
+// AS_ANY: a group lookup.
+enum ApplyScales : int { AS_TILE, AS_SLOT, AS_ANY };
+template <int QK, bool FULL, int BITS, int SCALES>
 __device__ __forceinline__ void apply_tile(const ApplyArgs &a, int64_t tile, float *qtab_s)
 {
     const int64_t d = a.d;
@@ -291,6 +297,7 @@ __device__ __forceinline__ void apply_tile(const ApplyArgs &a, int64_t tile, flo
     const int L = (QK == QK_UNIF) ? unif_L(bits) : 0;
     const float Lf = static_cast<float>(L);
     float x[kSlots][4];
+    float s_slot[kSlots];
     uint4 raw[kSlots];  // the slot's code bits: .x for b <= 8, .x .y for b = 16, all four for b = 32
 #pragma unroll
     for (int k = 0; k < kSlots; ++k) {
@@ -298,6 +305,7 @@ __device__ __forceinline__ void apply_tile(const ApplyArgs &a, int64_t tile, flo
         load4<FULL>(a.x, q, d, x[k]);
         raw[k] = make_uint4(0u, 0u, 0u, 0u);
         if (FULL || 4 * q < d) {
+            if constexpr (has_scale<QK>() && SCALES == AS_SLOT) s_slot[k] = __ldg(a.scales + ((4 * q) >> G.log2G));
             if constexpr (bits <= 8) {
                 raw[k].x = __ldg(a.words + ((q * bits) >> 3));
             } else if constexpr (bits == 16) {
@@ -314,10 +322,10 @@ __device__ __forceinline__ void apply_tile(const ApplyArgs &a, int64_t tile, flo
         __syncthreads();
     }
     // one scale for the whole tile: 4096-blocks, or a tile inside one group
-    const int64_t g1 = !has_scale<QK>() ? 0 : TILE_SCALE ? tile : tile_single_group(G, tile, d);
-    const bool tile_scale = TILE_SCALE || g1 >= 0;
-    const float s_tile = (has_scale<QK>() && tile_scale) ? __ldg(a.scales + g1) : 0.0f;
-    const int64_t hint = first_group_of_tile(G, tile);
+    const int64_t g1 = (!has_scale<QK>() || SCALES == AS_SLOT) ? 0 : SCALES == AS_TILE ? tile : tile_single_group(G, tile, d);
+    const bool tile_scale = SCALES != AS_ANY || g1 >= 0;
+    const float s_tile = (has_scale<QK>() && SCALES != AS_SLOT && tile_scale) ? __ldg(a.scales + g1) : 0.0f;
+    const int64_t hint = SCALES == AS_ANY ? first_group_of_tile(G, tile) : 0;
 #pragma unroll
     for (int k = 0; k < kSlots; ++k) {
         const int64_t q = slot_of(tile, k);
@@ -336,7 +344,7 @@ __device__ __forceinline__ void apply_tile(const ApplyArgs &a, int64_t tile, flo
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             if (FULL || j0 + i < d) {
-                float s = s_tile;
+                float s = SCALES == AS_SLOT ? s_slot[k] : s_tile;
                 if (has_scale<QK>() && !tile_scale) s = __ldg(a.scales + group_of(G, j0 + i, hint));
                 x[k][i] = __fsub_rn(x[k][i], decode1<QK>(c[i], s, a.q, Lf, L, qtab));
             }
@@ -351,11 +359,14 @@ __device__ __forceinline__ void apply_body(const ApplyArgs &a, float *qtab_s)
     const int64_t tile = blockIdx.x;
     const bool full = (tile + 1) * kTile <= a.d;
     if (a.q.grp.gkind == GK_BLOCK && a.q.grp.G == kTile) {
-        if (full) apply_tile<QK, true, BITS, true>(a, tile, qtab_s);
-        else apply_tile<QK, false, BITS, true>(a, tile, qtab_s);
+        if (full) apply_tile<QK, true, BITS, AS_TILE>(a, tile, qtab_s);
+        else apply_tile<QK, false, BITS, AS_TILE>(a, tile, qtab_s);
+    } else if (has_scale<QK>() && a.q.grp.gkind == GK_BLOCK && a.q.grp.log2G >= kLog2Chunk) {
+        if (full) apply_tile<QK, true, BITS, AS_SLOT>(a, tile, qtab_s);
+        else apply_tile<QK, false, BITS, AS_SLOT>(a, tile, qtab_s);
     } else {
-        if (full) apply_tile<QK, true, BITS, false>(a, tile, qtab_s);
-        else apply_tile<QK, false, BITS, false>(a, tile, qtab_s);
+        if (full) apply_tile<QK, true, BITS, AS_ANY>(a, tile, qtab_s);
+        else apply_tile<QK, false, BITS, AS_ANY>(a, tile, qtab_s);
     }
 }
 

@@ -134,6 +134,27 @@ def test_staged_server_several_tiles_per_cta(qw, qs, placement):
     _run_host(cfg, 2, seed=37, grad_scale=1e-3)
 
 
+@pytest.mark.parametrize("qw,qs", [
+    (W.sign_q(128), W.sign_q(2048)),
+    (W.uniform_q(4, 512, True), W.uniform_q(8, 512, False)),
+    (W.sign_q(1024), W.uniform_q(16, 256, True)),
+    (W.uniform_q(8, 128, False), W.sign_q(4096)),          # one side only, either way
+    (W.uniform_q(2, 4096, False), W.uniform_q(4, 1024, False)),
+    (W.pow2_q(-20, -5, 8), W.sign_q(256)),
+    (W.sign_q(512), W.identity_q()),
+    (W.sign_q(0), W.uniform_q(8, 512, False)),             # the direct server: whole-vector workers
+    (W.uniform_q(4, 256, True), W.sign_q(0)),              # the lazy server
+])
+@pytest.mark.parametrize("d,n,placement", [
+    (1, 1, ea.ADAM_AT_WORKER), (127, 2, ea.ADAM_AT_SERVER), (2049, 9, ea.ADAM_AT_WORKER),
+    (8192, 3, ea.ADAM_AT_WORKER), (12_289, 17, ea.ADAM_AT_SERVER), (4096 * 456 * 2 + 4095, 3, ea.ADAM_AT_WORKER)])
+def test_short_blocks(qw, qs, d, n, placement):
+    """Power-of-two blocks of 128 .. 2048: a tile holds several scales (ragged last blocks and tiles,
+    blocks longer than the vector, several tiles per persistent server CTA)."""
+    cfg = ea.EAConfig(d=d, n=n, qw=qw, qs=qs, alpha=1e-3, placement=placement, seed=d)
+    _run_host(cfg, 2 if d > 100_000 else 3, seed=d + n, grad_scale=1e-3)
+
+
 def test_two_pass_scale_beyond_the_grouped_capacity():
     """A whole-vector scale over 12.3 million coordinates: more tiles than the one-pass grouped
     kernels hold in shared memory at once (about 1,800 on a GB300).  The uniform-grid broadcast
