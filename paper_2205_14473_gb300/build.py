@@ -16,7 +16,7 @@ CSRC = os.path.join(PKG, "csrc")
 LIBDIR = os.path.join(PKG, "_lib")
 LIB = os.path.join(LIBDIR, "libea.so")
 SOURCES = ["ea_api.cu", "ea_worker.cu", "ea_noalloc.cu", "ea_selftest.cu"] + [
-    f"ea_server_{part}{m}_q{q}.cu" for q in (2, 1, 3, 0) for part in ("", "short_") for m in "sw"]
+    f"ea_server_{part}{m}_q{q}.cu" for q in (2, 1, 3, 0) for part in ("", "general_") for m in "sw"]
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 # binary32 per operation: no FMA contraction, IEEE division and square root, denormals kept
 FLAGS = ["-gencode", "arch=compute_103a,code=sm_103a", "-O3", "-lineinfo", "-std=c++17", "--fmad=false",

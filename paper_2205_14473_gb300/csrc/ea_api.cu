@@ -29,20 +29,20 @@ struct QHost {
     int64_t G = 0, n_groups = 1, n_words = 0, n_pairs = 0;
     bool has_scales = false;
     std::vector<int64_t> offsets;     // GK_SEG
-    std::vector<int32_t> tile_group;  // GK_SEG
+    std::vector<TileRef> ref;         // groups that span tiles: every tile's groups
     std::vector<int64_t> pair_base;   // PASS_STASH, PASS_GROUPED
     std::vector<int64_t> cuts;        // PASS_GROUPED: the waves
     int grid = 0, slots = 0;          // PASS_GROUPED: persistent CTAs and tile slots per CTA
     // device copies (inside the workspace)
     int64_t *d_offsets = nullptr, *d_pair_base = nullptr, *d_cuts = nullptr;
-    int32_t *d_tile_group = nullptr;
+    TileRef *d_ref = nullptr;
     unsigned long long *d_arrive = nullptr;  // PASS_GROUPED: the wave barrier's counter
 };
 
 // Sizes of every workspace buffer, in the order they are carved.
 struct Layout {
     size_t e_w, m_w, v_w, e_s, m_s, v_s, codes_w, scales_w, codes_s, scales_s, partials;
-    size_t off_w, tg_w, pb_w, off_s, tg_s, pb_s, status;
+    size_t off_w, ref_w, pb_w, off_s, ref_s, pb_s, status;
     size_t cuts_w, arr_w, cuts_s, arr_s;  // the grouped pass (groups that span tiles)
     size_t rview;                         // PASS_LAZY: where a residual view is formed
     int64_t dpad, wcode_stride, wscale_stride;
@@ -183,17 +183,11 @@ int setup_quant(const ea_quantizer &q, int64_t d, const char *name, QHost &out)
         if (out.offsets.back() != d)
             return fail(nullptr, EA_E_INVAL, "%s: segment lengths sum to %lld, not d = %lld", name,
                         static_cast<long long>(out.offsets.back()), static_cast<long long>(d));
-        out.tile_group.resize(n_tiles);
-        int64_t gi = 0;
-        for (int64_t t = 0; t < n_tiles; ++t) {
-            while (out.offsets[gi + 1] <= t * kTile) ++gi;
-            out.tile_group[t] = static_cast<int32_t>(gi);
-        }
     }
     // One pass when every group is exactly one tile, or a tile is a whole number of groups that are
     // a whole number of chunks each; otherwise partial norms per (tile, group).  512-blocks, 4-bit
     // stochastic grid, d = 15,000,001: one worker message took 313 us in the three launches of the
-    // latter (104 us, 106 us for the 29,297 scales, 103 us).
+    // latter (104 us, 106 us for the 29,297 scales, 103 us); the round of 8 workers 2620 us against 749.
     const bool block_tiles = out.gkind == GK_BLOCK && out.G == kTile;
     const bool single_tile = out.n_groups == 1 && d <= kTile;
     if (out.gkind == GK_BLOCK && out.log2G >= kLog2Chunk && out.G < kTile) {
@@ -212,6 +206,21 @@ int setup_quant(const ea_quantizer &q, int64_t d, const char *name, QHost &out)
             out.pair_base[gi + 1] = out.pair_base[gi] + ((e - 1) / kTile - b / kTile + 1);
         }
         out.n_pairs = out.pair_base.back();
+        if (out.gkind != GK_WHOLE) {
+            out.ref.resize(n_tiles);
+            auto group_end = [&](int64_t gi) {
+                return out.gkind == GK_BLOCK ? std::min(d, (gi + 1) * out.G) : out.offsets[gi + 1];
+            };
+            int64_t g0 = 0, part = 0;
+            for (int64_t t = 0; t < n_tiles; ++t) {
+                const int64_t hi = std::min(d, (t + 1) * kTile);
+                int64_t g = g0;
+                while (group_end(g) < hi) ++g;  // the group of the tile's last coordinate
+                out.ref[t] = TileRef{g0, part * 8192 + (g - g0 + 1)};
+                part += g - g0 + 1;
+                g0 = group_end(g) == hi ? g + 1 : g;
+            }
+        }
     }
     return EA_OK;
 }
@@ -263,10 +272,10 @@ Layout make_layout(const ea_config &c, const QHost &qw, const QHost &qs)
     L.partials = (lazy_w ? static_cast<size_t>(c.n) * qw.n_pairs + qs.n_pairs
                          : static_cast<size_t>(std::max(qw.n_pairs, qs.n_pairs))) * sizeof(double);
     L.off_w = qw.gkind == GK_SEG ? qw.offsets.size() * 8 : 0;
-    L.tg_w = qw.gkind == GK_SEG ? static_cast<size_t>(n_tiles) * 4 : 0;
+    L.ref_w = qw.ref.size() * sizeof(TileRef);
     L.pb_w = qw.pass == PASS_STASH ? qw.pair_base.size() * 8 : 0;
     L.off_s = qs.gkind == GK_SEG ? qs.offsets.size() * 8 : 0;
-    L.tg_s = qs.gkind == GK_SEG ? static_cast<size_t>(n_tiles) * 4 : 0;
+    L.ref_s = qs.ref.size() * sizeof(TileRef);
     L.pb_s = qs.pass == PASS_STASH ? qs.pair_base.size() * 8 : 0;
     L.status = 4;
     // the grouped pass, whenever groups span tiles (ea_init picks it when its waves fit)
@@ -282,7 +291,7 @@ Layout make_layout(const ea_config &c, const QHost &qw, const QHost &qs)
 size_t layout_bytes(const Layout &L)
 {
     const size_t parts[] = {L.e_w, L.m_w, L.v_w, L.e_s, L.m_s, L.v_s, L.codes_w, L.scales_w, L.codes_s,
-                            L.scales_s, L.partials, L.off_w, L.tg_w, L.pb_w, L.off_s, L.tg_s, L.pb_s, L.status,
+                            L.scales_s, L.partials, L.off_w, L.ref_w, L.pb_w, L.off_s, L.ref_s, L.pb_s, L.status,
                             L.cuts_w, L.arr_w, L.cuts_s, L.arr_s, L.rview};
     size_t total = 0;
     for (size_t p : parts) total += align_up(p, kAlign);
@@ -297,7 +306,7 @@ Grouping device_grouping(const QHost &q)
     g.G = q.G;
     g.n_groups = q.n_groups;
     g.offsets = q.d_offsets;
-    g.tile_group = q.d_tile_group;
+    g.ref = q.d_ref;
     g.pair_base = q.d_pair_base;
     return g;
 }
@@ -370,18 +379,12 @@ void try_grouped(QHost &q, int64_t d, int64_t n_tiles, const GroupedShape &shape
 }
 
 // The most of q's scale groups that meet one 4096-tile.
-int64_t max_groups_per_tile(const QHost &q, int64_t d, int64_t n_tiles)
+int64_t max_groups_per_tile(const QHost &q)
 {
     if (!q.has_scales || q.gkind == GK_WHOLE) return 1;
     if (q.gkind == GK_BLOCK) return (kTile - 1) / q.G + 2;  // a bound
     int64_t most = 1;
-    for (int64_t t = 0; t < n_tiles; ++t) {
-        const int64_t last = std::min((t + 1) * kTile, d) - 1;
-        const int64_t g0 = q.tile_group[static_cast<size_t>(t)];
-        int64_t g = g0;
-        while (q.offsets[static_cast<size_t>(g + 1)] <= last) ++g;
-        most = std::max(most, g - g0 + 1);
-    }
+    for (const TileRef &r : q.ref) most = std::max<int64_t>(most, r.ng());
     return most;
 }
 
@@ -416,13 +419,20 @@ uint64_t message_bits(const QHost &q, int64_t d)
 
 // Shared-memory staging of the server's inputs (see server_staged_kernel): one stage holds a
 // tile's e_s (+ m_s, v_s) and the n workers' code chunks and scales.  Enabled when the scale groups of
-// both messages lie inside 4096-tiles (or there are none) and one stage fits in 200 KB.
+// both messages lie inside 4096-tiles or are whole tiles (or there are none) and one stage fits in
+// 200 KB.  Where a group spans tiles: d = 30,000,000 with one scale, four workers' 8-bit grid messages and
+// broadcast: the round took 1312 us with a server CTA per tile that loads directly (383 us of it the
+// server's), 1042 us staged.
 StagePlan make_server_plan(const ea_config &c, const QHost &qw, const QHost &qs, int64_t n_tiles, int sms)
 {
     StagePlan P{};
-    auto in_tile = [](const QHost &q) { return !q.has_scales || q.pass == PASS_FUSED || q.pass == PASS_SHORT; };
-    if (!in_tile(qs) || !in_tile(qw) || sms <= 0) return P;
-    P.short_blocks = qs.pass == PASS_SHORT || qw.pass == PASS_SHORT;
+    // groups of whole tiles that span several: the vector, or blocks of a multiple of 4096
+    auto spans = [](const QHost &q) { return q.pass == PASS_STASH || q.pass == PASS_LAZY; };
+    auto takes = [&](const QHost &q) {
+        return !spans(q) || q.gkind == GK_WHOLE || (q.gkind == GK_BLOCK && q.G % kTile == 0);
+    };
+    if (!takes(qs) || !takes(qw) || sms <= 0) return P;
+    P.general = spans(qs) || spans(qw) || qs.pass == PASS_SHORT || qw.pass == PASS_SHORT;
     const uint32_t scales = qw.pass == PASS_SHORT ? static_cast<uint32_t>(kTile / qw.G) : 1u;  // of one worker
     const bool server_adam = c.placement == EA_ADAM_AT_SERVER;
     uint32_t off = 0;
@@ -639,10 +649,10 @@ int ea_init(const ea_config *cfg, void *workspace, size_t workspace_bytes, void 
     h->partials = reinterpret_cast<double *>(take(L.partials));
     h->spartials = h->partials;
     h->qw.d_offsets = reinterpret_cast<int64_t *>(take(L.off_w));
-    h->qw.d_tile_group = reinterpret_cast<int32_t *>(take(L.tg_w));
+    h->qw.d_ref = reinterpret_cast<TileRef *>(take(L.ref_w));
     h->qw.d_pair_base = reinterpret_cast<int64_t *>(take(L.pb_w));
     h->qs.d_offsets = reinterpret_cast<int64_t *>(take(L.off_s));
-    h->qs.d_tile_group = reinterpret_cast<int32_t *>(take(L.tg_s));
+    h->qs.d_ref = reinterpret_cast<TileRef *>(take(L.ref_s));
     h->qs.d_pair_base = reinterpret_cast<int64_t *>(take(L.pb_s));
     h->status = reinterpret_cast<uint32_t *>(take(L.status));
     h->qw.d_cuts = reinterpret_cast<int64_t *>(take(L.cuts_w));
@@ -659,7 +669,7 @@ int ea_init(const ea_config *cfg, void *workspace, size_t workspace_bytes, void 
     if (h->qs.pass == PASS_STASH && h->qs.kind == EA_Q_SIGN_L1) {
         h->qs.pass = PASS_LAZY;
         // the server stages a tile's worker codes and scales in shared memory when they fit
-        const int64_t g = max_groups_per_tile(h->qw, cfg->d, h->n_tiles);
+        const int64_t g = max_groups_per_tile(h->qw);
         h->lazy_staged = static_cast<int64_t>(cfg->n) * h->qw.bits <= 32 &&
                          g <= kStagedTileGroups && cfg->n * g <= kWorkerScales;
     }
@@ -692,10 +702,10 @@ int ea_init(const ea_config *cfg, void *workspace, size_t workspace_bytes, void 
         if (r == EA_OK && n) r = check_cuda(h, cudaMemcpyAsync(dst, src, n, cudaMemcpyHostToDevice, s), "table upload");
     };
     upload(h->qw.d_offsets, h->qw.offsets.data(), L.off_w);
-    upload(h->qw.d_tile_group, h->qw.tile_group.data(), L.tg_w);
+    upload(h->qw.d_ref, h->qw.ref.data(), L.ref_w);
     upload(h->qw.d_pair_base, h->qw.pair_base.data(), L.pb_w);
     upload(h->qs.d_offsets, h->qs.offsets.data(), L.off_s);
-    upload(h->qs.d_tile_group, h->qs.tile_group.data(), L.tg_s);
+    upload(h->qs.d_ref, h->qs.ref.data(), L.ref_s);
     upload(h->qs.d_pair_base, h->qs.pair_base.data(), L.pb_s);
     upload(h->qw.d_cuts, h->qw.cuts.data(), h->qw.cuts.size() * 8);
     upload(h->qs.d_cuts, h->qs.cuts.data(), h->qs.cuts.size() * 8);
@@ -792,9 +802,14 @@ int ea_server_step(ea_handle *h)
     int r = finalize_worker_scales(h);
     if (r != EA_OK) return r;
     if (h->qs.pass == PASS_LAZY) {
-        r = check_cuda(h, W ? launch_server_lazy<MODE_W>(a, h->lazy_staged, h->stream)
-                            : launch_server_lazy<MODE_S>(a, h->lazy_staged, h->stream),
-                       "server launch");
+        if (h->splan.enabled) {
+            r = check_cuda(h, launch_server(W ? MODE_W : MODE_S, a, h->stream), "server launch");
+            if (h->splan.grid < h->n_tiles) h->split_full = true;
+        } else {
+            r = check_cuda(h, W ? launch_server_lazy<MODE_W>(a, h->lazy_staged, h->stream)
+                                : launch_server_lazy<MODE_S>(a, h->lazy_staged, h->stream),
+                           "server launch");
+        }
         if (r == EA_OK) r = finalize_scales(h, h->qs, h->spartials, h->sscales);
         if (r == EA_OK) h->lazy_s = h->cfg.error_feedback != 0;
     } else if (h->qs.pass == PASS_GROUPED) {

@@ -177,6 +177,17 @@ __device__ __forceinline__ float block_max_all(float a, uint32_t *red)
     return __uint_as_float(__reduce_max_sync(0xffffffffu, lane < kWarps ? red[lane] : 0u));
 }
 
+// CTA-wide maximum of non-negative values, valid in warp 0 only; one barrier.  `red` may be reused
+// after the next barrier.
+__device__ __forceinline__ float block_max_warp0(float a, uint32_t *red)
+{
+    const uint32_t b = __reduce_max_sync(0xffffffffu, __float_as_uint(a));
+    const int lane = threadIdx.x & 31;
+    if (lane == 0) red[threadIdx.x >> 5] = b;
+    compute_sync();
+    return threadIdx.x < 32 ? __uint_as_float(__reduce_max_sync(0xffffffffu, lane < kWarps ? red[lane] : 0u)) : 0.0f;
+}
+
 // CTA-wide maximum of non-negative values (exact: compares bit patterns).
 __device__ __forceinline__ float block_max(float a, uint32_t *red, float *bcast)
 {
@@ -343,7 +354,7 @@ __device__ __forceinline__ int64_t first_group_of_tile(const Grouping &g, int64_
 {
     if (g.gkind == GK_WHOLE) return 0;
     if (g.gkind == GK_BLOCK) return g.log2G >= 0 ? (tile * kTile) >> g.log2G : (tile * kTile) / g.G;
-    return g.tile_group[tile];
+    return g.ref ? g.ref[tile].g0 : 0;
 }
 
 // The group that holds every coordinate of tile `tile` (of [0, d)), or -1 when the tile spans a
@@ -357,8 +368,22 @@ __device__ __forceinline__ int64_t tile_single_group(const Grouping &g, int64_t 
         const int64_t g0 = first_group_of_tile(g, tile);
         return group_of(g, last, g0) == g0 ? g0 : -1;
     }
-    const int64_t g0 = g.tile_group[tile];
-    return g.offsets[g0 + 1] > last ? g0 : -1;
+    if (!g.ref) return 0;  // one segment, one tile
+    const TileRef r = g.ref[tile];
+    return r.ng() == 1 ? r.g0 : -1;
+}
+
+// The groups of tile `tile` (uniform over the CTA).  Reads only tables written when the handle was
+// made, so a kernel may call it before its predecessor has finished.
+__device__ __forceinline__ TileRef tile_ref(const Grouping &g, int64_t tile, int64_t d)
+{
+    if (g.gkind == GK_WHOLE) return {0, tile * 8192 + 1};
+    if (g.ref) {
+        const longlong2 v = __ldg(reinterpret_cast<const longlong2 *>(g.ref) + tile);
+        return {v.x, v.y};
+    }
+    const int64_t last = min(tile * kTile + static_cast<int64_t>(kTile), d) - 1, g0 = first_group_of_tile(g, tile);
+    return {g0, g.gkind == GK_BLOCK ? group_of(g, last, g0) - g0 + 1 : 1};
 }
 
 // Short blocks: power-of-two blocks of 128 .. 2048 coordinates (of 4096: the same with one block per
@@ -384,16 +409,9 @@ struct TileGroups {
 __device__ __forceinline__ void cache_tile_groups(const Grouping &g, int64_t tile, int64_t d, TileGroups &tg)
 {
     const int64_t tl = tile * kTile;
-    const int64_t n_tiles = (d + kTile - 1) / kTile;
-    const int64_t g0 = g.tile_group[tile];
-    int64_t last;  // the group holding the tile's last coordinate
-    if (tile + 1 < n_tiles) {
-        const int64_t gn = g.tile_group[tile + 1];
-        last = g.offsets[gn] == tl + kTile ? gn - 1 : gn;
-    } else {
-        last = g.n_groups - 1;
-    }
-    const int nb = static_cast<int>(last - g0);
+    const TileRef r = tile_ref(g, tile, d);
+    const int64_t g0 = r.g0;
+    const int nb = r.ng() - 1;
     if (threadIdx.x == 0) {
         tg.g0 = g0;
         tg.nb = nb;

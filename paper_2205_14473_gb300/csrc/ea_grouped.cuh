@@ -47,8 +47,9 @@ __device__ __forceinline__ void range_partials(const float4 *ub, int64_t tile, i
                                                const QParams &q, double *partials, GroupSmem &gs, int &turn)
 {
     const Grouping &G = q.grp;
+    const TileRef ref = tile_ref(G, tile, d);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int64_t gi = group_of(G, lo, first_group_of_tile(G, tile));; ++gi, ++turn) {
+    for (int64_t gi = ref.ng() == 1 ? ref.g0 : group_of(G, lo, ref.g0);; ++gi, ++turn) {
         const int64_t gb = group_begin(G, gi, d), ge = group_end(G, gi, d);
         const int64_t a = max(gb, lo), b = min(ge, hi);
         const int par = turn & 1;
@@ -74,7 +75,7 @@ __device__ __forceinline__ void range_partials(const float4 *ub, int64_t tile, i
                 DF t = gs.red[par][0];
 #pragma unroll
                 for (int w = 1; w < kWarps; ++w) t = df_add(t, gs.red[par][w]);
-                partials[G.pair_base[gi] + (tile - gb / kTile)] = static_cast<double>(t.hi) + static_cast<double>(t.lo);
+                partials[ref.part() + (gi - ref.g0)] = static_cast<double>(t.hi) + static_cast<double>(t.lo);
             }
         } else {
             float mx = 0.0f;
@@ -94,7 +95,7 @@ __device__ __forceinline__ void range_partials(const float4 *ub, int64_t tile, i
                 uint32_t t = gs.redm[par][0];
 #pragma unroll
                 for (int w = 1; w < kWarps; ++w) t = max(t, gs.redm[par][w]);
-                partials[G.pair_base[gi] + (tile - gb / kTile)] = static_cast<double>(__uint_as_float(t));
+                partials[ref.part() + (gi - ref.g0)] = static_cast<double>(__uint_as_float(t));
             }
         }
         if (ge >= hi) break;

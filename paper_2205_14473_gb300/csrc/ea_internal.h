@@ -42,6 +42,23 @@ constexpr int server_ctas_per_sm(int mode, int qw, int qs)
     return (mode == MODE_W && qw == QK_SIGN && qs == QK_SIGN) ? 4 : 3;
 }
 
+// What a tile has to know of its scale groups, in one 16-byte load that no other lookup waits for: the
+// group of its first coordinate, how many groups meet it (1 .. 4096) and where its first partial norm
+// goes.  Group g0 + i of the tile has its partial at part + i: a later group starts in the tile, which
+// is its first pair, and the one before it ends there, which was its last.
+struct alignas(16) TileRef {
+    int64_t g0;
+    int64_t part_ng;  // part * 8192 + groups
+#ifdef __CUDACC__
+    __host__ __device__
+#endif
+    int ng() const { return static_cast<int>(part_ng & 8191); }
+#ifdef __CUDACC__
+    __host__ __device__
+#endif
+    int64_t part() const { return part_ng >> 13; }
+};
+
 // How a message's scale groups tile the vector.
 struct Grouping {
     int gkind;
@@ -49,7 +66,8 @@ struct Grouping {
     int64_t G;                  // GK_BLOCK: block length
     int64_t n_groups;
     const int64_t *offsets;     // GK_SEG: n_groups + 1 offsets (device)
-    const int32_t *tile_group;  // GK_SEG: first group that intersects each 4096-tile (device)
+    const TileRef *ref;         // every tile's groups (device); null for GK_WHOLE, and where every
+                                // group lies inside one tile
     const int64_t *pair_base;   // n_groups + 1: first partial-sum slot of each group (device)
 };
 
@@ -133,7 +151,7 @@ struct WorkerArgs {
 // tile's inputs; byte offsets are relative to the stage start and 128-byte aligned.
 struct StagePlan {
     int enabled;               // 0: use the direct-load kernel
-    int short_blocks;          // Q_w or Q_s has several scales per tile (PASS_SHORT)
+    int general;               // Q_w or Q_s has several scales per tile, or one for several
     int stages;                // pipeline depth
     int grid;                  // persistent CTAs
     uint32_t stage_bytes;      // bytes of one stage
@@ -228,7 +246,7 @@ cudaError_t server_grouped_shape(int mode, int qw, int qs, GroupedShape *out);
 template <int MODE, int QS>
 cudaError_t launch_server_for_qs(const ServerArgs &a, cudaStream_t s);
 template <int MODE, int QS>
-cudaError_t launch_server_short(const ServerArgs &a, cudaStream_t s);
+cudaError_t launch_server_general(const ServerArgs &a, cudaStream_t s);
 
 // The server kernel for the placement and the broadcast quantizer kind of `a` (ea_api.cu).
 cudaError_t launch_server(int mode, const ServerArgs &a, cudaStream_t s);

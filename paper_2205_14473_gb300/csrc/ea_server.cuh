@@ -142,6 +142,11 @@ __global__ void __launch_bounds__(kThreads, 2) server_kernel(const ServerArgs a)
     const int64_t d = a.d;
 
     pdl_trigger();
+    TileRef ref{};
+    if (has_scale<QS>() && a.pass == PASS_STASH) {
+        ref = tile_ref(a.qs.grp, tile, d);
+        if (threadIdx.x == 0) sm.part = ref.part();
+    }
     build_qtab<QS>(a.qs, sm.qtab);  // read after the scale reduction's barrier
     const float *utab = build_worker_utab<QW>(a, utab_s);
     if (utab) __syncthreads();
@@ -180,18 +185,18 @@ __global__ void __launch_bounds__(kThreads, 2) server_kernel(const ServerArgs a)
         }
     }
     finish_tile<QS>(URegs{u}, tile, d, a.qs, a.words, a.scales, a.es, a.ef, a.pass, a.seed,
-                    static_cast<uint32_t>(a.n), a.t, a.partials, sm);
+                    static_cast<uint32_t>(a.n), a.t, a.partials, sm, ref);
 }
 
 // Phase one of a grouped server tile: w (the average, after the Adam step with Adam at the server,
 // plus e_s) of the coordinate range [lo, hi) of tile `tile` (0 elsewhere) into ub; m_s and v_s
-// updated and stored in the range.  FULL: the range is the whole tile.
+// updated and stored in the range.  FULL: the range is the whole tile.  rs: Q_s's groups (LAZY).
 template <int MODE, int QW, bool FULL, bool LAZY = false>
 __device__ __forceinline__ void server_u_range(const ServerArgs &a, int64_t tile, int64_t lo, int64_t hi, float4 *ub,
-                                               const float *utab, float *stab, TileGroups &tg)
+                                               const float *utab, float *stab, TileGroups &tg, const TileRef &rs)
 {
     LazyScale lzs{};
-    if (LAZY && a.lazy_in) lzs = lazy_scale_of_tile(a.qs, a.scales, tile, a.d);
+    if (LAZY && a.lazy_in) lzs = lazy_scale_of_tile(rs, a.scales);
     float acc[kSlots][4];
     decode_sum_direct<QW>(a, tile, utab, stab, tg, acc);
     const float nf = static_cast<float>(a.n);
@@ -360,23 +365,20 @@ __device__ __forceinline__ void decode_sum_staged(const ServerArgs &a, int64_t t
 // average, after the Adam step with Adam at the server, plus e_s) of the range [lo, hi) then
 // replaces the codes in ub (0 outside the range); m_s, v_s are updated and stored in the range.
 // Returns false, having done nothing, when the tile's scale table would not fit (the caller then
-// takes server_u_range).
+// takes server_u_range).  rw, rs: the tile's groups of Q_w and (LAZY) Q_s, which the caller looked up
+// early; tgs: room for Q_s's segments of a tile that holds several (LAZY).
 template <int MODE, int QW, bool FULL, bool LAZY = false>
 __device__ __forceinline__ bool server_u_staged(const ServerArgs &a, int64_t tile, int64_t lo, int64_t hi, float4 *ub,
-                                                const float *utab, float *stab, float *wsc, GroupSmem &gs)
+                                                const float *utab, float *stab, float *wsc, GroupSmem &gs,
+                                                const TileRef &rw, const TileRef &rs, TileGroups *tgs)
 {
     const int64_t d = a.d;
     const int n = a.n;
     const int bw = code_bits<QW>(a.qw);
     const Grouping &GW = a.qw.grp;
-    int64_t gw0 = 0;
-    int ngw = 1;
-    if (has_scale<QW>()) {
-        gw0 = first_group_of_tile(GW, tile);
-        const int64_t last = min(tile * kTile + static_cast<int64_t>(kTile), d) - 1;
-        ngw = static_cast<int>(group_of(GW, last, gw0) - gw0 + 1);
-        if (n * ngw > kWorkerScales || ngw > kStagedTileGroups) return false;
-    }
+    const int64_t gw0 = has_scale<QW>() ? rw.g0 : 0;
+    const int ngw = has_scale<QW>() ? rw.ng() : 1;
+    if (n * ngw > kWorkerScales || ngw > kStagedTileGroups) return false;
     const bool seg = has_scale<QW>() && ngw > 1 && GW.gkind == GK_SEG;
     float es[kSlots][4], ms[kSlots][4], vs[kSlots][4];
     bool in[kSlots];
@@ -394,8 +396,11 @@ __device__ __forceinline__ bool server_u_staged(const ServerArgs &a, int64_t til
             }
         }
     }
-    compute_sync();  // the slot's and the tables' previous readers are done
-    const int chunk_words = kTile * bw / 32;
+    LazyScale lzs{};
+    if (LAZY && a.lazy_in) lzs = lazy_scale_of_tile(rs, a.scales);
+    if constexpr (!LAZY) compute_sync();  // the slot's and the tables' previous readers are done
+    const int chunk_words = kTile * bw / 32;  // a power of two
+    const int log2_vec = __ffs(chunk_words) - 1 - 2;  // its 16-byte vectors
     uint32_t *cw = reinterpret_cast<uint32_t *>(ub);
     {
         const int64_t cbase = tile * chunk_words;          // the tile's chunk in every code stream
@@ -403,14 +408,18 @@ __device__ __forceinline__ bool server_u_staged(const ServerArgs &a, int64_t til
         const int nvec = n * chunk_words / 4;
         // every copy issued at once (cp.async: no register round trip), then one wait
         for (int v = threadIdx.x; v < nvec; v += kThreads) {
-            const int w = (4 * v) / chunk_words, o = (4 * v) % chunk_words;
+            const int w = v >> log2_vec, o = 4 * (v & ((1 << log2_vec) - 1));
             uint4 *dst = reinterpret_cast<uint4 *>(cw) + v;
             if (o + 4 <= avail) cp_async16(dst, a.wwords + static_cast<int64_t>(w) * a.wwords_stride + cbase + o);
             else *dst = make_uint4(0u, 0u, 0u, 0u);
         }
-        if (has_scale<QW>())
+        if (has_scale<QW>() && ngw == 1) {
+            for (int i = threadIdx.x; i < n; i += kThreads) cp_async4(wsc + i, a.wscales + i * a.wscales_stride + gw0);
+        } else if (has_scale<QW>()) {
             for (int i = threadIdx.x; i < n * ngw; i += kThreads)
                 cp_async4(wsc + i, a.wscales + static_cast<int64_t>(i / ngw) * a.wscales_stride + gw0 + i % ngw);
+        }
+        if (LAZY && a.lazy_in && lzs.g1 < 0 && a.qs.grp.gkind == GK_SEG) cache_tile_groups(a.qs.grp, tile, d, *tgs);
         if (seg) cache_tile_groups(GW, tile, d, gs.tg);
         cp_async_wait_all();
     }
@@ -420,10 +429,24 @@ __device__ __forceinline__ bool server_u_staged(const ServerArgs &a, int64_t til
     compute_sync();  // every thread has read the staged codes
     if constexpr (LAZY) {
         if (a.lazy_in) {  // es holds the previous round's w: its residual (lo is the tile's start)
-            const LazyScale lzs = lazy_scale_of_tile(a.qs, a.scales, tile, d);
+            const bool segs = lzs.g1 < 0 && a.qs.grp.gkind == GK_SEG;
 #pragma unroll
-            for (int k = 0; k < kSlots; ++k)
-                if (in[k]) lazy_residual4<FULL>(a.qs, a.scales, lzs, 4 * slot_of(tile, k), hi, es[k]);
+            for (int k = 0; k < kSlots; ++k) {
+                if (!in[k]) continue;
+                const int64_t j0 = 4 * slot_of(tile, k);
+                if (!segs) {
+                    lazy_residual4<FULL>(a.qs, a.scales, lzs, j0, hi, es[k]);
+                    continue;
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    if (!FULL && j0 + i >= hi) continue;
+                    float dec;
+                    (void)encode1<QK_SIGN>(es[k][i], __ldg(a.scales + tile_group_of(a.qs.grp, *tgs, tile, j0 + i)), a.qs,
+                                           0.0f, 0, 0.0f, dec);
+                    es[k][i] = __fsub_rn(es[k][i], dec);
+                }
+            }
         }
     }
     const float nf = static_cast<float>(n);
@@ -477,13 +500,14 @@ __global__ void __launch_bounds__(kThreads, MODE == MODE_S ? 2 : 3) server_group
             const int64_t tl = static_cast<int64_t>(tile) * kTile, lo = max(c0, tl), hi = min(c1, tl + kTile);
             const bool full = lo == tl && hi == tl + kTile;
             bool done = false;
+            const TileRef rw = tile_ref(a.qw.grp, tile, a.d);
             if (staged)
-                done = full ? server_u_staged<MODE, QW, true>(a, tile, lo, hi, ub, utab, stab, wsc, gs)
-                            : server_u_staged<MODE, QW, false>(a, tile, lo, hi, ub, utab, stab, wsc, gs);
+                done = full ? server_u_staged<MODE, QW, true>(a, tile, lo, hi, ub, utab, stab, wsc, gs, rw, rw, nullptr)
+                            : server_u_staged<MODE, QW, false>(a, tile, lo, hi, ub, utab, stab, wsc, gs, rw, rw, nullptr);
             if (!done) {
                 compute_sync();  // stab's and tg's previous readers are done
-                if (full) server_u_range<MODE, QW, true>(a, tile, lo, hi, ub, utab, stab, gs.tg);
-                else server_u_range<MODE, QW, false>(a, tile, lo, hi, ub, utab, stab, gs.tg);
+                if (full) server_u_range<MODE, QW, true>(a, tile, lo, hi, ub, utab, stab, gs.tg, rw);
+                else server_u_range<MODE, QW, false>(a, tile, lo, hi, ub, utab, stab, gs.tg, rw);
             }
             range_partials<QS>(ub, tile, lo, hi, a.d, a.qs, a.partials, gs, turn);
         }
@@ -508,24 +532,31 @@ __global__ void __launch_bounds__(kThreads, MODE == MODE_S ? 2 : 3) server_lazy_
     __shared__ float utab_s[256];
     __shared__ float stab[256];
     __shared__ float wsc[kWorkerScales];
+    __shared__ DF red256[kThreads];
+    __shared__ TileGroups tgs;
     pdl_trigger();
-    const float *utab = build_worker_utab<QW>(a, utab_s);
-    __syncthreads();
-    pdl_wait();
     const int64_t tile = blockIdx.x;
     const int64_t d = a.d, lo = tile * kTile, hi = min(lo + static_cast<int64_t>(kTile), d);
+    // both messages' groups of the tile and the decode table before the predecessor has finished (the
+    // first barrier of the decode lies between the table and its readers)
+    const TileRef rw = has_scale<QW>() ? tile_ref(a.qw.grp, tile, d) : TileRef{0, 1};
+    const TileRef rs = tile_ref(a.qs.grp, tile, d);
+    const float *utab = build_worker_utab<QW>(a, utab_s);
+    if constexpr (!STAGED) __syncthreads();
+    pdl_wait();
     const bool full = hi == lo + kTile;
     if constexpr (STAGED) {
-        const bool done = full ? server_u_staged<MODE, QW, true, true>(a, tile, lo, hi, ub, utab, stab, wsc, gs)
-                               : server_u_staged<MODE, QW, false, true>(a, tile, lo, hi, ub, utab, stab, wsc, gs);
+        const bool done = full ? server_u_staged<MODE, QW, true, true>(a, tile, lo, hi, ub, utab, stab, wsc, gs, rw, rs, &tgs)
+                               : server_u_staged<MODE, QW, false, true>(a, tile, lo, hi, ub, utab, stab, wsc, gs, rw, rs, &tgs);
         if (!done) {  // outside what the host checked: report it, store nothing
             if (threadIdx.x == 0) report_status(a.status, kStatusCheck);
             return;
         }
     } else {
-        if (full) server_u_range<MODE, QW, true, true>(a, tile, lo, hi, ub, utab, stab, gs.tg);
-        else server_u_range<MODE, QW, false, true>(a, tile, lo, hi, ub, utab, stab, gs.tg);
+        if (full) server_u_range<MODE, QW, true, true>(a, tile, lo, hi, ub, utab, stab, gs.tg, rs);
+        else server_u_range<MODE, QW, false, true>(a, tile, lo, hi, ub, utab, stab, gs.tg, rs);
     }
+    DF acc{0.0f, 0.0f};
 #pragma unroll
     for (int k = 0; k < kSlots; ++k) {
         const int64_t qs = slot_of(tile, k);
@@ -537,9 +568,15 @@ __global__ void __launch_bounds__(kThreads, MODE == MODE_S ? 2 : 3) server_lazy_
             float dec;
             const uint32_t code = encode1<QK_SIGN>(w[i], 0.0f, a.qs, 0.0f, 0, 0.0f, dec);
             c[i] = (4 * qs + i < d) ? code : 0u;
+            df_accumulate(acc, fabsf(w[i]));  // w beyond d is 0
         }
         store_codes4<false, false>(a.words, qs, 1, c, 0, d);
         if (a.ef && 4 * qs < d) store4(a.es, qs, d, w);
+    }
+    if (rs.ng() == 1) {  // the tile's norm is the one group's partial
+        const DF tot = block_sum_lane0(acc, red256);
+        if (threadIdx.x == 0) a.partials[rs.part()] = static_cast<double>(tot.hi) + static_cast<double>(tot.lo);
+        return;
     }
     int turn = 0;
     range_partials<QK_SIGN>(ub, tile, lo, hi, d, a.qs, a.partials, gs, turn);
@@ -682,9 +719,11 @@ __device__ __forceinline__ void unif_decode_sum(const unsigned char *codes, int 
 // NW: the worker count when it is 8, known at compile time (the per-worker bounds, the average's
 // division and the decode loops then fold; for scaled-sign workers the table is the whole average
 // and the per-worker path is not compiled in), or 0 for a count known at run time.
-// SHORT: one of the messages has several scales per tile (short blocks): the workers' values are
-// decoded with the chunk's scale, one per warp, slot and worker, and Q_s takes chunk_scales.
-template <int MODE, int QW, int QS, bool FULL, int NW, bool SHORT>
+// GENERAL: one of the messages has several scales per tile (short blocks) or one for several whole
+// tiles: the workers' values are decoded with the chunk's scale, one per warp, slot and worker, and
+// the broadcast takes chunk_scales, or leaves w and the tile's partial norm (and, for the scaled
+// sign, the codes) as PASS_STASH and PASS_LAZY do.
+template <int MODE, int QW, int QS, bool FULL, int NW, bool GENERAL>
 __device__ __forceinline__ bool server_staged_tile(const ServerArgs &a, int64_t tile, const unsigned char *st,
                                                    bool ok, uint64_t *empty, int Lw, float Lwf, const float *utab,
                                                    float *wtab, const uint32_t (&flip)[8], TileSmem &sm)
@@ -702,8 +741,15 @@ __device__ __forceinline__ bool server_staged_tile(const ServerArgs &a, int64_t 
     bool done = false;
     // wtab is rebuilt below; the previous tile's reads of it end at its scale reduction's barrier,
     // which a Q_s without scales does not have
-    if constexpr (!SHORT && !has_scale<QS>() && (QW == QK_SIGN || QW == QK_UNIF)) compute_sync();
-    if constexpr (SHORT) {
+    if constexpr (!GENERAL && !has_scale<QS>() && (QW == QK_SIGN || QW == QK_UNIF)) compute_sync();
+    float s_prev = 0.0f;  // PASS_LAZY: the scale of the kept w in e_s
+    TileRef ref{};
+    if constexpr (GENERAL && has_scale<QS>()) {
+        if (a.pass == PASS_STASH || a.pass == PASS_LAZY) ref = tile_ref(a.qs.grp, tile, d);
+        if (threadIdx.x == 0) sm.part = ref.part();
+        if (QS == QK_SIGN && a.lazy_in) s_prev = a.scales[ref.g0];
+    }
+    if constexpr (GENERAL) {
         done = true;
         if (!compute_all(ok)) return false;
 #pragma unroll
@@ -738,7 +784,7 @@ __device__ __forceinline__ bool server_staged_tile(const ServerArgs &a, int64_t 
 #pragma unroll
             for (int i = 0; i < 4; ++i) acc[k][i] = pow2n ? __fmul_rn(acc[k][i], inv_n) : __fdiv_rn(acc[k][i], nf);
     }
-    if constexpr (!SHORT && QW == QK_SIGN) {
+    if constexpr (!GENERAL && QW == QK_SIGN) {
       {
         done = NW == 8 || n <= 8;
         // Scaled-sign workers: the worker-order sum of the first m = min(n, 8) workers depends
@@ -788,7 +834,7 @@ __device__ __forceinline__ bool server_staged_tile(const ServerArgs &a, int64_t 
         }
       }
     }
-    if (!SHORT && !done) {
+    if (!GENERAL && !done) {
         // scaled-sign workers (n > 8): acc already holds the sum of workers 0..7
         constexpr bool partial = QW == QK_SIGN;
         if constexpr (!partial) {
@@ -866,12 +912,22 @@ __device__ __forceinline__ bool server_staged_tile(const ServerArgs &a, int64_t 
             to_arr(reinterpret_cast<const float4 *>(st + P.off_b)[ls], ms);
             to_arr(reinterpret_cast<const float4 *>(st + P.off_c)[ls], vs);
         }
+        if constexpr (GENERAL && QS == QK_SIGN) {
+            if (a.lazy_in) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    float dec;
+                    (void)encode1<QK_SIGN>(es[i], s_prev, a.qs, 0.0f, 0, 0.0f, dec);
+                    es[i] = __fsub_rn(es[i], dec);
+                }
+            }
+        }
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             float step = acc[k][i];
             if (MODE == MODE_S) step = adam_step(step, ms[i], vs[i], a.hp);
             u[i] = (FULL || j0 + i < d) ? __fadd_rn(step, es[i]) : 0.0f;  // invalid u are 0
-            if constexpr (SHORT) continue;  // chunk_scales forms its own sums
+            if constexpr (GENERAL) continue;  // the norms are formed below
             if constexpr (QS == QK_SIGN) df_accumulate(l1, fabsf(u[i]));
             else mx = fmaxf(mx, fabsf(u[i]));
         }
@@ -881,11 +937,14 @@ __device__ __forceinline__ bool server_staged_tile(const ServerArgs &a, int64_t 
             store4<FULL>(a.vs, q, d, vs);
         }
     }
-    if constexpr (SHORT && has_scale<QS>()) {
-        chunk_scales<QS>(USmem{ubuf}, tile, d, chunk_shift(a.qs.grp), a.scales, sm);
-        encode_store<QS, FULL, false>(USmem{ubuf}, ChunkScales{sm.csc}, tile, d, a.qs, a.words, a.es, a.ef, a.seed,
-                                      static_cast<uint32_t>(a.n), a.t,
-                                      (QS == QK_UNIF && a.qs.bits <= 8) ? sm.qtab : nullptr);
+    if constexpr (GENERAL && has_scale<QS>()) {
+        constexpr int spans = QS == QK_SIGN ? PASS_LAZY : PASS_STASH;  // groups that span tiles
+        if (a.pass == spans)
+            finish_tile<QS, FULL, false, spans>(USmem{ubuf}, tile, d, a.qs, a.words, a.scales, a.es, a.ef, spans, a.seed,
+                                                static_cast<uint32_t>(a.n), a.t, a.partials, sm, ref);
+        else
+            finish_tile<QS, FULL, false, PASS_SHORT>(USmem{ubuf}, tile, d, a.qs, a.words, a.scales, a.es, a.ef, PASS_SHORT,
+                                                     a.seed, static_cast<uint32_t>(a.n), a.t, a.partials, sm, ref);
     } else {
         finish_tile_smem<QS, FULL, false>(ubuf, l1, mx, tile, d, a.qs, a.words, a.scales, a.es, a.ef, a.seed,
                                           static_cast<uint32_t>(a.n), a.t, sm);
@@ -901,9 +960,9 @@ __device__ __forceinline__ bool server_staged_tile(const ServerArgs &a, int64_t 
 // m_s, v_s with Adam at the server) and the n workers' code chunks with bulk copies, and the n
 // worker scales with 4-byte cp.async, into a ring of stages guarded by full/empty mbarriers; the
 // compute warps decode, average, re-quantize and write e_s and the broadcast straight to HBM.
-// Used when the scale groups of Q_s and Q_w lie inside 4096-tiles (or are absent); SHORT: some tile
-// holds several.
-template <int MODE, int QW, int QS, bool SHORT>
+// Used when no tile lies in several scale groups of Q_s or Q_w of which one spans tiles; GENERAL: some
+// tile holds several groups, or some group several tiles.
+template <int MODE, int QW, int QS, bool GENERAL>
 __global__ void __launch_bounds__(kThreads + 32, server_ctas_per_sm(MODE, QW, QS)) server_staged_kernel(const ServerArgs a)
 {
     extern __shared__ __align__(128) unsigned char dsm[];
@@ -966,12 +1025,13 @@ __global__ void __launch_bounds__(kThreads + 32, server_ctas_per_sm(MODE, QW, QS
             }
             if (scaled_w) {
                 float *sc = reinterpret_cast<float *>(st + P.off_scales);
-                if constexpr (SHORT) {
+                if constexpr (GENERAL) {
                     // worker w's scales of the tile, at w * per; past the last group the stream's
                     // padding is read (a multiple of 64 scales)
                     const int lp = 5 - chunk_shift(a.qw.grp), per = 1 << lp;
+                    const int64_t first = lp ? tile * per : tile_ref(a.qw.grp, tile, a.d).g0;
                     for (int i = lane; i < a.n * per; i += 32)
-                        cp_async4(sc + i, a.wscales + (i >> lp) * a.wscales_stride + tile * per + (i & (per - 1)));
+                        cp_async4(sc + i, a.wscales + (i >> lp) * a.wscales_stride + first + (i & (per - 1)));
                 } else {
                     for (int w = lane; w < a.n; w += 32) cp_async4(sc + w, a.wscales + w * a.wscales_stride + tile);
                 }
@@ -1002,7 +1062,7 @@ __global__ void __launch_bounds__(kThreads + 32, server_ctas_per_sm(MODE, QW, QS
         const float *ut = use_tab ? utab : nullptr;
         const bool whole = (tile + 1) * kTile <= d;
         bool go;
-        if constexpr (SHORT) {
+        if constexpr (GENERAL) {
             go = whole ? server_staged_tile<MODE, QW, QS, true, 0, true>(a, tile, st, ok, &empty[s], Lw, Lwf, ut, wtab, flip, sm)
                        : server_staged_tile<MODE, QW, QS, false, 0, true>(a, tile, st, ok, &empty[s], Lw, Lwf, ut, wtab, flip, sm);
         } else {
@@ -1017,7 +1077,7 @@ __global__ void __launch_bounds__(kThreads + 32, server_ctas_per_sm(MODE, QW, QS
     }
 }
 
-template <int MODE, int QW, int QS, bool SHORT>
+template <int MODE, int QW, int QS, bool GENERAL>
 static cudaError_t launch_server_staged_kernel(const ServerArgs &a, cudaStream_t s)
 {
     // Function attributes are per device: one flag per device ordinal.  Two threads that race on a
@@ -1028,19 +1088,19 @@ static cudaError_t launch_server_staged_kernel(const ServerArgs &a, cudaStream_t
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
     if (!attr_set[dev].load(std::memory_order_acquire)) {
-        e = cudaFuncSetAttribute(server_staged_kernel<MODE, QW, QS, SHORT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(server_staged_kernel<MODE, QW, QS, GENERAL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  kServerMaxDynSmem);
         if (e != cudaSuccess) return e;
         attr_set[dev].store(true, std::memory_order_release);
     }
-    return launch_pdl(server_staged_kernel<MODE, QW, QS, SHORT>, dim3(a.plan.grid), dim3(kThreads + 32),
+    return launch_pdl(server_staged_kernel<MODE, QW, QS, GENERAL>, dim3(a.plan.grid), dim3(kThreads + 32),
                       a.plan.smem_bytes, s, true, cudaSharedmemCarveoutMaxShared, a);
 }
 
 template <int MODE, int QW, int QS>
 static cudaError_t launch_server_staged(const ServerArgs &a, cudaStream_t s)
 {
-    if (a.plan.short_blocks) return launch_server_short<MODE, QS>(a, s);
+    if (a.plan.general) return launch_server_general<MODE, QS>(a, s);
     return launch_server_staged_kernel<MODE, QW, QS, false>(a, s);
 }
 

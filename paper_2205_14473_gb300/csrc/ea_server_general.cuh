@@ -1,14 +1,14 @@
-// ea_server_short.cuh -- launches of the staged server for messages with several scales per tile
-// (PASS_SHORT), in translation units of their own.
+// ea_server_general.cuh -- launches of the staged server where a message has several scales per tile
+// (PASS_SHORT) or one for several tiles, in translation units of their own.
 #pragma once
 
 #include "ea_server.cuh"
 
 namespace ea {
 
-// The staged server where a message has short blocks (instantiated in ea_server_short_<mode>_q<QS>.cu).
+// (instantiated in ea_server_general_<mode>_q<QS>.cu).
 template <int MODE, int QS>
-cudaError_t launch_server_short(const ServerArgs &a, cudaStream_t s)
+cudaError_t launch_server_general(const ServerArgs &a, cudaStream_t s)
 {
     switch (a.qw.kind) {
     case QK_SIGN: return launch_server_staged_kernel<MODE, QK_SIGN, QS, true>(a, s);

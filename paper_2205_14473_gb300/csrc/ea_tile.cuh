@@ -15,6 +15,7 @@ struct TileSmem {
     double bcast;
     float bcastf;
     float csc[kChunks];  // PASS_SHORT: the scale of each chunk
+    int64_t part;        // PASS_STASH, PASS_LAZY: the tile's first partial norm (thread 0 writes and reads it)
     float qtab[256];  // the uniform grid's fl(i / L) of the tile's own quantizer (build_qtab)
 };
 
@@ -282,8 +283,9 @@ __device__ __forceinline__ void finish_tile_smem(const float4 *ubuf, DF l1, floa
                                    (QK == QK_UNIF && q.bits <= 8) ? sm.qtab : nullptr);
 }
 
-// PASS_LAZY on a tile that lies inside one scale group: a compile-time refinement of the pass
-// (one partial norm, no per-coordinate group bounds), chosen per tile by the lazy kernels.
+// PASS_LAZY on a tile that lies inside one scale group, as a compile-time refinement chosen per tile
+// by the worker's kernel (the general form's group lookups cost registers: with Adam at the worker,
+// a single form for both spilled 92 bytes a thread, and ResNet-18's messages took 5% longer).
 constexpr int PASS_LAZY_ONE = 16;
 
 // The tile's end for a quantizer with scale groups, u read through `src` (URegs or USmem).
@@ -294,12 +296,12 @@ constexpr int PASS_LAZY_ONE = 16;
 // tile loop is instruction-bound).
 // PASS: PASS_FUSED, PASS_SHORT or PASS_STASH as a compile-time constant (the other path is then not compiled
 // in), or -1 to follow `pass`.
-// part_idx (PASS_LAZY_ONE): where the tile's partial norm goes, looked up early by the caller.
+// ref (PASS_STASH, PASS_LAZY): the tile's groups; sm.part is set by the caller.
 template <int QK, bool FULL = false, bool BALLOT = true, int PASS = -1, class USrc>
 __device__ __forceinline__ void finish_tile(const USrc &src, int64_t tile, int64_t d, const QParams &q,
                                             uint32_t *words, float *scales, float *resid, int ef, int pass,
                                             uint64_t seed, uint32_t id, uint32_t t, double *partials,
-                                            TileSmem &sm, int64_t part_idx = 0)
+                                            TileSmem &sm, const TileRef &ref)
 {
     if constexpr (PASS >= 0) pass = PASS;
     if constexpr (!has_scale<QK>()) {
@@ -343,40 +345,21 @@ __device__ __forceinline__ void finish_tile(const USrc &src, int64_t tile, int64
                                            (QK == QK_UNIF && q.bits <= 8) ? sm.qtab : nullptr);
             return;
         }
-        if constexpr (PASS == PASS_LAZY_ONE && QK == QK_SIGN) {
-            // u (with error feedback), the codes, and the one group's partial norm of the tile
-            // (a compensated sum to ~2^-44, like the per-group loop below; one barrier)
-            DF acc{0.0f, 0.0f};
-#pragma unroll
-            for (int k = 0; k < kSlots; ++k) {
-                const int64_t qs = slot_of(tile, k);
-                float uk[4];
-                src.get(k, uk);
-                if (ef && (FULL || 4 * qs < d)) store4<FULL>(resid, qs, d, uk);
-                uint32_t c[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    float dec;
-                    const uint32_t code = encode1<QK>(uk[i], 0.0f, q, 0.0f, 0, 0.0f, dec);
-                    c[i] = (FULL || 4 * qs + i < d) ? code : 0u;
-                    df_accumulate(acc, fabsf(uk[i]));  // u beyond d is 0
-                }
-                store_codes4<FULL, BALLOT>(words, qs, 1, c, 0, d);
-            }
-            const DF tot = block_sum_lane0(acc, sm.red256);
-            if (threadIdx.x == 0) partials[part_idx] = static_cast<double>(tot.hi) + static_cast<double>(tot.lo);
-            return;
-        }
         // PASS_STASH: u into resid for encode_kernel.  PASS_LAZY (scaled sign): u into resid, where
         // the residual is formed from it and the scale later (lazy_residual; without error feedback
-        // the residual stays 0), and the codes now: the sign of u needs no scale.
+        // the residual stays 0), and the codes now: the sign of u needs no scale.  PASS_LAZY_ONE forms
+        // the norm on the way.
+        DF all{0.0f, 0.0f};
 #pragma unroll
         for (int k = 0; k < kSlots; ++k) {
             const int64_t qs = slot_of(tile, k);
             float uk[4];
             src.get(k, uk);
-            if ((PASS != PASS_LAZY || ef) && (FULL || 4 * qs < d)) store4<FULL>(resid, qs, d, uk);
-            if constexpr (PASS == PASS_LAZY && QK == QK_SIGN) {
+            if constexpr (PASS == PASS_LAZY_ONE)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) df_accumulate(all, fabsf(uk[i]));  // u beyond d is 0
+            if (((PASS != PASS_LAZY && PASS != PASS_LAZY_ONE) || ef) && (FULL || 4 * qs < d)) store4<FULL>(resid, qs, d, uk);
+            if constexpr ((PASS == PASS_LAZY || PASS == PASS_LAZY_ONE) && QK == QK_SIGN) {
                 uint32_t c[4];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
@@ -387,8 +370,34 @@ __device__ __forceinline__ void finish_tile(const USrc &src, int64_t tile, int64
                 store_codes4<FULL, BALLOT>(words, qs, 1, c, 0, d);
             }
         }
+        if (PASS == PASS_LAZY_ONE || ref.ng() == 1) {
+            if constexpr (QK == QK_SIGN) {
+                if constexpr (PASS != PASS_LAZY_ONE)
+#pragma unroll
+                    for (int k = 0; k < kSlots; ++k) {
+                        float uk[4];
+                        src.get(k, uk);
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) df_accumulate(all, fabsf(uk[i]));
+                    }
+                const DF tot = block_sum_lane0(all, sm.red256);
+                if (threadIdx.x == 0) partials[sm.part] = static_cast<double>(tot.hi) + static_cast<double>(tot.lo);
+            } else {
+                float mx = 0.0f;
+#pragma unroll
+                for (int k = 0; k < kSlots; ++k) {
+                    float uk[4];
+                    src.get(k, uk);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) mx = fmaxf(mx, fabsf(uk[i]));
+                }
+                mx = block_max_warp0(mx, sm.redm);
+                if (threadIdx.x == 0) partials[sm.part] = static_cast<double>(mx);
+            }
+            return;
+        }
         const Grouping &G = q.grp;
-        for (int64_t gi = first_group_of_tile(G, tile);; ++gi) {
+        for (int64_t gi = ref.g0;; ++gi) {
             const int64_t gb = group_begin(G, gi, d), ge = group_end(G, gi, d);
             const int64_t lo = max(gb, tile_lo), hi = min(ge, tile_hi);
             double part;
@@ -417,7 +426,7 @@ __device__ __forceinline__ void finish_tile(const USrc &src, int64_t tile, int64
                 }
                 part = static_cast<double>(block_max(mx, sm.redm, &sm.bcastf));
             }
-            if (threadIdx.x == 0) partials[G.pair_base[gi] + (tile - gb / kTile)] = part;
+            if (threadIdx.x == 0) partials[sm.part + (gi - ref.g0)] = part;
             if (ge >= tile_hi) break;
         }
     }
@@ -433,11 +442,11 @@ struct LazyScale {
     float s1;          // the scale of g1
 };
 
-__device__ __forceinline__ LazyScale lazy_scale_of_tile(const QParams &q, const float *scales, int64_t tile, int64_t d)
+__device__ __forceinline__ LazyScale lazy_scale_of_tile(const TileRef &ref, const float *scales)
 {
     LazyScale ls;
-    ls.g1 = tile_single_group(q.grp, tile, d);
-    ls.hint = first_group_of_tile(q.grp, tile);
+    ls.g1 = ref.ng() == 1 ? ref.g0 : -1;
+    ls.hint = ref.g0;
     ls.s1 = ls.g1 >= 0 ? scales[ls.g1] : 0.0f;
     return ls;
 }
@@ -458,31 +467,23 @@ __device__ __forceinline__ void lazy_residual4(const QParams &q, const float *sc
     }
 }
 
-// The same for all of this thread's slots of tile `tile`.
-// The same for a tile inside one group, whose previous scale is s.
-template <bool FULL>
-__device__ __forceinline__ void lazy_residual_one(const QParams &q, float s, int64_t tile, int64_t d,
-                                                  float (&e)[kSlots][4])
+// The same for all of this thread's slots of tile `tile`.  ONE: the tile lies inside one group.
+template <bool FULL, bool ONE>
+__device__ __forceinline__ void lazy_residual(const QParams &q, const float *scales, const LazyScale &ls, int64_t tile,
+                                              int64_t d, float (&e)[kSlots][4])
 {
+    if (ONE || ls.g1 >= 0) {  // one branch for the tile
 #pragma unroll
-    for (int k = 0; k < kSlots; ++k) {
-        const int64_t j0 = 4 * slot_of(tile, k);
+        for (int k = 0; k < kSlots; ++k) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            if (FULL || j0 + i < d) {
+            for (int i = 0; i < 4; ++i) {
                 float dec;
-                (void)encode1<QK_SIGN>(e[k][i], s, q, 0.0f, 0, 0.0f, dec);
-                e[k][i] = __fsub_rn(e[k][i], dec);
+                (void)encode1<QK_SIGN>(e[k][i], ls.s1, q, 0.0f, 0, 0.0f, dec);
+                if (FULL || 4 * slot_of(tile, k) + i < d) e[k][i] = __fsub_rn(e[k][i], dec);
             }
         }
+        return;
     }
-}
-
-template <bool FULL>
-__device__ __forceinline__ void lazy_residual(const QParams &q, const float *scales, int64_t tile, int64_t d,
-                                              float (&e)[kSlots][4])
-{
-    const LazyScale ls = lazy_scale_of_tile(q, scales, tile, d);
 #pragma unroll
     for (int k = 0; k < kSlots; ++k) lazy_residual4<FULL>(q, scales, ls, 4 * slot_of(tile, k), d, e[k]);
 }

@@ -6,20 +6,12 @@ namespace ea {
 // One tile of worker_kernel; FULL: the tile lies inside [0, d) (every tile but a ragged last one).
 // Each slot's u goes to ubuf (only this thread reads it again), so that no register holds u across
 // the scale's reduction and more CTAs fit on an SM.
+// ref: the tile's groups (PASS_STASH, PASS_LAZY), looked up by the caller.
 template <int MODE, int QK, bool FULL, int PASS>
-__device__ __forceinline__ void worker_tile(const WorkerArgs &a, int64_t tile, float4 *ubuf, TileSmem &sm)
+__device__ __forceinline__ void worker_tile(const WorkerArgs &a, int64_t tile, float4 *ubuf, TileSmem &sm,
+                                            const TileRef &ref)
 {
     const int64_t d = a.d;
-    // PASS_LAZY_ONE: the tile's group, its previous scale and the slot of its partial norm, looked
-    // up before the tile's loads so that these short dependent loads overlap them
-    int64_t part_idx = 0;
-    float s_prev = 0.0f;
-    if constexpr (PASS == PASS_LAZY_ONE) {
-        const Grouping &G = a.q.grp;
-        const int64_t g1 = first_group_of_tile(G, tile);
-        part_idx = G.pair_base[g1] + (tile - group_begin(G, g1, d) / kTile);
-        if (a.lazy_in) s_prev = a.scales[g1];
-    }
     float g[kSlots][4], e[kSlots][4], m[kSlots][4], v[kSlots][4];
 #pragma unroll
     for (int k = 0; k < kSlots; ++k) {
@@ -31,14 +23,16 @@ __device__ __forceinline__ void worker_tile(const WorkerArgs &a, int64_t tile, f
             load4<FULL>(a.v, q, d, v[k]);
         }
     }
+    constexpr bool lazy = PASS == PASS_LAZY || PASS == PASS_LAZY_ONE;
+    LazyScale ls{};
+    if constexpr (lazy)
+        if (a.lazy_in) ls = lazy_scale_of_tile(ref, a.scales);
     // the grid's fl(i/L) table, built while the loads are in flight (read after the scale
     // reduction's barrier)
     build_qtab<QK>(a.q, sm.qtab);
-    if constexpr (PASS == PASS_LAZY) {
+    if constexpr (lazy) {
         // e holds the previous round's u: its residual is u - Q(u) with the previous scales
-        if (a.lazy_in) lazy_residual<FULL>(a.q, a.scales, tile, d, e);
-    } else if constexpr (PASS == PASS_LAZY_ONE) {
-        if (a.lazy_in) lazy_residual_one<FULL>(a.q, s_prev, tile, d, e);
+        if (a.lazy_in) lazy_residual<FULL, PASS == PASS_LAZY_ONE>(a.q, a.scales, ls, tile, d, e);
     }
 #pragma unroll
     for (int k = 0; k < kSlots; ++k) {
@@ -58,7 +52,7 @@ __device__ __forceinline__ void worker_tile(const WorkerArgs &a, int64_t tile, f
         }
     }
     finish_tile<QK, FULL, true, PASS>(USmem{ubuf}, tile, d, a.q, a.words, a.scales, a.e, a.ef, a.pass, a.seed, a.id, a.t,
-                                      a.partials, sm, part_idx);
+                                      a.partials, sm, ref);
 }
 
 // Algorithm 2 for one worker on one 4096-coordinate tile.  With Adam at the worker:
@@ -78,13 +72,15 @@ __global__ void __launch_bounds__(kThreads, MODE == MODE_S ? 4 : 3)
     __shared__ TileSmem sm;
     __shared__ float4 ubuf[kSlots * kThreads];
     pdl_trigger();
-    pdl_wait();
     const int64_t tile = blockIdx.x;
+    const TileRef ref = tile_ref(a.q.grp, tile, a.d);
+    if (threadIdx.x == 0) sm.part = ref.part();
+    pdl_wait();
     if ((tile + 1) * kTile <= a.d) {
-        if (tile_single_group(a.q.grp, tile, a.d) >= 0) worker_tile<MODE, QK_SIGN, true, PASS_LAZY_ONE>(a, tile, ubuf, sm);
-        else worker_tile<MODE, QK_SIGN, true, PASS_LAZY>(a, tile, ubuf, sm);
+        if (ref.ng() == 1) worker_tile<MODE, QK_SIGN, true, PASS_LAZY_ONE>(a, tile, ubuf, sm, ref);
+        else worker_tile<MODE, QK_SIGN, true, PASS_LAZY>(a, tile, ubuf, sm, ref);
     } else {
-        worker_tile<MODE, QK_SIGN, false, PASS_LAZY>(a, tile, ubuf, sm);
+        worker_tile<MODE, QK_SIGN, false, PASS_LAZY>(a, tile, ubuf, sm, ref);
     }
 }
 
@@ -95,19 +91,24 @@ __global__ void __launch_bounds__(kThreads, MODE == MODE_S ? 4 : 3)
     __shared__ TileSmem sm;
     __shared__ float4 ubuf[kSlots * kThreads];
     pdl_trigger();
-    pdl_wait();
     const int64_t tile = blockIdx.x;
+    TileRef ref{};
+    if (has_scale<QK>() && a.pass == PASS_STASH) {
+        ref = tile_ref(a.q.grp, tile, a.d);
+        if (threadIdx.x == 0) sm.part = ref.part();
+    }
+    pdl_wait();
     // the scale pass as a compile-time constant: each instantiation carries only its own path
     const bool full = (tile + 1) * kTile <= a.d;
     if (a.pass == PASS_FUSED) {
-        if (full) worker_tile<MODE, QK, true, PASS_FUSED>(a, tile, ubuf, sm);
-        else worker_tile<MODE, QK, false, PASS_FUSED>(a, tile, ubuf, sm);
+        if (full) worker_tile<MODE, QK, true, PASS_FUSED>(a, tile, ubuf, sm, ref);
+        else worker_tile<MODE, QK, false, PASS_FUSED>(a, tile, ubuf, sm, ref);
     } else if (has_scale<QK>() && a.pass == PASS_SHORT) {
-        if (full) worker_tile<MODE, QK, true, PASS_SHORT>(a, tile, ubuf, sm);
-        else worker_tile<MODE, QK, false, PASS_SHORT>(a, tile, ubuf, sm);
+        if (full) worker_tile<MODE, QK, true, PASS_SHORT>(a, tile, ubuf, sm, ref);
+        else worker_tile<MODE, QK, false, PASS_SHORT>(a, tile, ubuf, sm, ref);
     } else {
-        if (full) worker_tile<MODE, QK, true, PASS_STASH>(a, tile, ubuf, sm);
-        else worker_tile<MODE, QK, false, PASS_STASH>(a, tile, ubuf, sm);
+        if (full) worker_tile<MODE, QK, true, PASS_STASH>(a, tile, ubuf, sm, ref);
+        else worker_tile<MODE, QK, false, PASS_STASH>(a, tile, ubuf, sm, ref);
     }
 }
 
@@ -229,21 +230,21 @@ __global__ void __launch_bounds__(kThreads, 2) encode_kernel(const EncodeArgs a)
     __shared__ float qtab_s[256];
     pdl_trigger();
     const float *qtab = build_qtab<QK>(a.q, qtab_s);
-    __syncthreads();
-    pdl_wait();
     const int64_t tile = blockIdx.x;
     const int64_t d = a.d;
     const Grouping &G = a.q.grp;
+    const TileRef ref = tile_ref(G, tile, d);
+    __syncthreads();
+    pdl_wait();
     const int L = (QK == QK_UNIF) ? unif_L(a.q.bits) : 0;
     const float Lf = static_cast<float>(L);
-    const int64_t hint = first_group_of_tile(G, tile);
+    const int64_t hint = ref.g0;
     float u[kSlots][4];
 #pragma unroll
     for (int k = 0; k < kSlots; ++k) load4(a.buf, slot_of(tile, k), d, u[k]);
     // a tile inside one group (the common case) has one scale: the fused tile encode
-    const int64_t g1 = tile_single_group(G, tile, d);
-    if (g1 >= 0) {
-        const float s = a.scales[g1];
+    if (ref.ng() == 1) {
+        const float s = a.scales[ref.g0];
         if ((tile + 1) * kTile <= d)
             encode_store<QK, true, true>(URegs{u}, s, tile, d, a.q, a.words, a.buf, a.ef, a.seed, a.id, a.t, qtab);
         else
@@ -289,7 +290,7 @@ __global__ void __launch_bounds__(kThreads, 2) encode_kernel(const EncodeArgs a)
 // AS_ANY: a group lookup.
 enum ApplyScales : int { AS_TILE, AS_SLOT, AS_ANY };
 template <int QK, bool FULL, int BITS, int SCALES>
-__device__ __forceinline__ void apply_tile(const ApplyArgs &a, int64_t tile, float *qtab_s)
+__device__ __forceinline__ void apply_tile(const ApplyArgs &a, int64_t tile, const TileRef &ref, float *qtab_s)
 {
     const int64_t d = a.d;
     const Grouping &G = a.q.grp;
@@ -322,10 +323,10 @@ __device__ __forceinline__ void apply_tile(const ApplyArgs &a, int64_t tile, flo
         __syncthreads();
     }
     // one scale for the whole tile: 4096-blocks, or a tile inside one group
-    const int64_t g1 = (!has_scale<QK>() || SCALES == AS_SLOT) ? 0 : SCALES == AS_TILE ? tile : tile_single_group(G, tile, d);
+    const int64_t g1 = (!has_scale<QK>() || SCALES == AS_SLOT) ? 0 : SCALES == AS_TILE ? tile : ref.ng() == 1 ? ref.g0 : -1;
     const bool tile_scale = SCALES != AS_ANY || g1 >= 0;
     const float s_tile = (has_scale<QK>() && SCALES != AS_SLOT && tile_scale) ? __ldg(a.scales + g1) : 0.0f;
-    const int64_t hint = SCALES == AS_ANY ? first_group_of_tile(G, tile) : 0;
+    const int64_t hint = SCALES == AS_ANY ? ref.g0 : 0;
 #pragma unroll
     for (int k = 0; k < kSlots; ++k) {
         const int64_t q = slot_of(tile, k);
@@ -354,19 +355,19 @@ __device__ __forceinline__ void apply_tile(const ApplyArgs &a, int64_t tile, flo
 }
 
 template <int QK, int BITS>
-__device__ __forceinline__ void apply_body(const ApplyArgs &a, float *qtab_s)
+__device__ __forceinline__ void apply_body(const ApplyArgs &a, const TileRef &ref, float *qtab_s)
 {
     const int64_t tile = blockIdx.x;
     const bool full = (tile + 1) * kTile <= a.d;
     if (a.q.grp.gkind == GK_BLOCK && a.q.grp.G == kTile) {
-        if (full) apply_tile<QK, true, BITS, AS_TILE>(a, tile, qtab_s);
-        else apply_tile<QK, false, BITS, AS_TILE>(a, tile, qtab_s);
+        if (full) apply_tile<QK, true, BITS, AS_TILE>(a, tile, ref, qtab_s);
+        else apply_tile<QK, false, BITS, AS_TILE>(a, tile, ref, qtab_s);
     } else if (has_scale<QK>() && a.q.grp.gkind == GK_BLOCK && a.q.grp.log2G >= kLog2Chunk) {
-        if (full) apply_tile<QK, true, BITS, AS_SLOT>(a, tile, qtab_s);
-        else apply_tile<QK, false, BITS, AS_SLOT>(a, tile, qtab_s);
+        if (full) apply_tile<QK, true, BITS, AS_SLOT>(a, tile, ref, qtab_s);
+        else apply_tile<QK, false, BITS, AS_SLOT>(a, tile, ref, qtab_s);
     } else {
-        if (full) apply_tile<QK, true, BITS, AS_ANY>(a, tile, qtab_s);
-        else apply_tile<QK, false, BITS, AS_ANY>(a, tile, qtab_s);
+        if (full) apply_tile<QK, true, BITS, AS_ANY>(a, tile, ref, qtab_s);
+        else apply_tile<QK, false, BITS, AS_ANY>(a, tile, ref, qtab_s);
     }
 }
 
@@ -376,19 +377,21 @@ __global__ void __launch_bounds__(kThreads) apply_kernel(const ApplyArgs a)
 {
     __shared__ float qtab_s[256];
     pdl_trigger();
+    TileRef ref{};
+    if (has_scale<QK>()) ref = tile_ref(a.q.grp, blockIdx.x, a.d);
     pdl_wait();
     if constexpr (QK == QK_UNIF) {
         switch (a.q.bits) {  // the widths ea_init accepts
-        case 2: apply_body<QK, 2>(a, qtab_s); break;
-        case 4: apply_body<QK, 4>(a, qtab_s); break;
-        case 8: apply_body<QK, 8>(a, qtab_s); break;
-        default: apply_body<QK, 16>(a, qtab_s); break;
+        case 2: apply_body<QK, 2>(a, ref, qtab_s); break;
+        case 4: apply_body<QK, 4>(a, ref, qtab_s); break;
+        case 8: apply_body<QK, 8>(a, ref, qtab_s); break;
+        default: apply_body<QK, 16>(a, ref, qtab_s); break;
         }
     } else if constexpr (QK == QK_POW2) {
-        if (a.q.bits == 4) apply_body<QK, 4>(a, qtab_s);
-        else apply_body<QK, 8>(a, qtab_s);
+        if (a.q.bits == 4) apply_body<QK, 4>(a, ref, qtab_s);
+        else apply_body<QK, 8>(a, ref, qtab_s);
     } else {
-        apply_body<QK, QK == QK_SIGN ? 1 : 32>(a, qtab_s);
+        apply_body<QK, QK == QK_SIGN ? 1 : 32>(a, ref, qtab_s);
     }
 }
 
@@ -456,14 +459,16 @@ cudaError_t launch_encode(const EncodeArgs &a, cudaStream_t s, bool overlap)
 __global__ void __launch_bounds__(kThreads) lazy_resid_kernel(const ResidArgs a)
 {
     pdl_trigger();
-    pdl_wait();
     const int64_t tile = blockIdx.x;
+    const TileRef ref = tile_ref(a.q.grp, tile, a.d);
+    pdl_wait();
     const bool full = (tile + 1) * kTile <= a.d;
+    const LazyScale ls = lazy_scale_of_tile(ref, a.scales);
     float u[kSlots][4];
 #pragma unroll
     for (int k = 0; k < kSlots; ++k) load4(a.u, slot_of(tile, k), a.d, u[k]);
-    if (full) lazy_residual<true>(a.q, a.scales, tile, a.d, u);
-    else lazy_residual<false>(a.q, a.scales, tile, a.d, u);
+    if (full) lazy_residual<true, false>(a.q, a.scales, ls, tile, a.d, u);
+    else lazy_residual<false, false>(a.q, a.scales, ls, tile, a.d, u);
 #pragma unroll
     for (int k = 0; k < kSlots; ++k)
         if (4 * slot_of(tile, k) < a.d) store4(a.out, slot_of(tile, k), a.d, u[k]);
