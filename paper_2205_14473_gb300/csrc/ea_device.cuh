@@ -570,6 +570,21 @@ __device__ __forceinline__ void load4(const float *__restrict__ p, int64_t q, in
     }
 }
 
+// store4 of what a kernel soon reads again: no streaming hint, so that its lines stay in L2 before
+// those of the streams around it.
+template <bool FULL = false>
+__device__ __forceinline__ void store4_kept(float *__restrict__ p, int64_t q, int64_t d, const float a[4])
+{
+    const int64_t j0 = 4 * q;
+    if (FULL || j0 + 4 <= d) {
+        reinterpret_cast<float4 *>(p)[q] = to_f4(a);
+    } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (j0 + i < d) p[j0 + i] = a[i];
+    }
+}
+
 template <bool FULL = false>
 __device__ __forceinline__ void store4(float *__restrict__ p, int64_t q, int64_t d, const float a[4])
 {

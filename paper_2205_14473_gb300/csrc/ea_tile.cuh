@@ -358,7 +358,11 @@ __device__ __forceinline__ void finish_tile(const USrc &src, int64_t tile, int64
             if constexpr (PASS == PASS_LAZY_ONE)
 #pragma unroll
                 for (int i = 0; i < 4; ++i) df_accumulate(all, fabsf(uk[i]));  // u beyond d is 0
-            if (((PASS != PASS_LAZY && PASS != PASS_LAZY_ONE) || ef) && (FULL || 4 * qs < d)) store4<FULL>(resid, qs, d, uk);
+            if constexpr (PASS != PASS_LAZY && PASS != PASS_LAZY_ONE) {
+                if (FULL || 4 * qs < d) store4_kept<FULL>(resid, qs, d, uk);
+            } else {
+                if (ef && (FULL || 4 * qs < d)) store4<FULL>(resid, qs, d, uk);
+            }
             if constexpr ((PASS == PASS_LAZY || PASS == PASS_LAZY_ONE) && QK == QK_SIGN) {
                 uint32_t c[4];
 #pragma unroll

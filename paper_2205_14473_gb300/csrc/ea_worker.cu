@@ -204,9 +204,17 @@ __global__ void __launch_bounds__(kThreads) finalize_kernel(const FinalizeArgs a
     const double *partials = a.partials + static_cast<int64_t>(blockIdx.y) * a.partials_stride;
     float *scales = a.scales + static_cast<int64_t>(blockIdx.y) * a.scales_stride;
     const int64_t pb = a.q.grp.pair_base[gi], pe = a.q.grp.pair_base[gi + 1];
+    // eight loads in flight per thread: a whole vector's partials (7,325 at d = 30,000,000) are a chain of
+    // L2 latencies otherwise.  TBD
+    constexpr int U = 8;
     double acc = 0.0;
-    for (int64_t p = pb + threadIdx.x; p < pe; p += kThreads)
-        acc = (QK == QK_SIGN) ? __dadd_rn(acc, partials[p]) : fmax(acc, partials[p]);
+    for (int64_t p = pb + threadIdx.x; p < pe; p += U * kThreads) {
+        double v[U];
+#pragma unroll
+        for (int i = 0; i < U; ++i) v[i] = p + i * kThreads < pe ? partials[p + i * kThreads] : 0.0;  // norms >= 0
+#pragma unroll
+        for (int i = 0; i < U; ++i) acc = (QK == QK_SIGN) ? __dadd_rn(acc, v[i]) : fmax(acc, v[i]);
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         const double w = __shfl_down_sync(0xffffffffu, acc, o);
@@ -223,44 +231,52 @@ __global__ void __launch_bounds__(kThreads) finalize_kernel(const FinalizeArgs a
 }
 
 // Second pass, one CTA per tile: encode the stashed input with its group's scale and leave the
-// residual u - Q(u) in its place.
+// residual u - Q(u) in its place.  The tiles are taken last first: the first pass stored u without a
+// streaming hint among streams that have one, so the tiles it wrote last are still in L2, and what is
+// overwritten there was never written to memory.  TBD
+template <int QK, bool FULL>
+__device__ __forceinline__ void encode_one_group(const EncodeArgs &a, float s, int64_t tile, const float *qtab)
+{
+    float u[kSlots][4];
+#pragma unroll
+    for (int k = 0; k < kSlots; ++k) load4<FULL>(a.buf, slot_of(tile, k), a.d, u[k]);
+    encode_store<QK, FULL, true>(URegs{u}, s, tile, a.d, a.q, a.words, a.buf, a.ef, a.seed, a.id, a.t, qtab);
+    if (!a.ef) {  // without error feedback the residual is 0: clear the stash of u
+        const float z[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int k = 0; k < kSlots; ++k)
+            if (FULL || 4 * slot_of(tile, k) < a.d) store4<FULL>(a.buf, slot_of(tile, k), a.d, z);
+    }
+}
+
 template <int QK>
-__global__ void __launch_bounds__(kThreads, 2) encode_kernel(const EncodeArgs a)
+__global__ void __launch_bounds__(kThreads, 4) encode_kernel(const EncodeArgs a)
 {
     __shared__ float qtab_s[256];
     pdl_trigger();
     const float *qtab = build_qtab<QK>(a.q, qtab_s);
-    const int64_t tile = blockIdx.x;
+    const int64_t tile = a.n_tiles - 1 - static_cast<int64_t>(blockIdx.x);
     const int64_t d = a.d;
     const Grouping &G = a.q.grp;
     const TileRef ref = tile_ref(G, tile, d);
     __syncthreads();
     pdl_wait();
-    const int L = (QK == QK_UNIF) ? unif_L(a.q.bits) : 0;
-    const float Lf = static_cast<float>(L);
-    const int64_t hint = ref.g0;
-    float u[kSlots][4];
-#pragma unroll
-    for (int k = 0; k < kSlots; ++k) load4(a.buf, slot_of(tile, k), d, u[k]);
     // a tile inside one group (the common case) has one scale: the fused tile encode
     if (ref.ng() == 1) {
         const float s = a.scales[ref.g0];
-        if ((tile + 1) * kTile <= d)
-            encode_store<QK, true, true>(URegs{u}, s, tile, d, a.q, a.words, a.buf, a.ef, a.seed, a.id, a.t, qtab);
-        else
-            encode_store<QK, false, true>(URegs{u}, s, tile, d, a.q, a.words, a.buf, a.ef, a.seed, a.id, a.t, qtab);
-        if (!a.ef) {  // without error feedback the residual is 0: clear the stash of u
-            const float z[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-            for (int k = 0; k < kSlots; ++k)
-                if (4 * slot_of(tile, k) < d) store4(a.buf, slot_of(tile, k), d, z);
-        }
+        if ((tile + 1) * kTile <= d) encode_one_group<QK, true>(a, s, tile, qtab);
+        else encode_one_group<QK, false>(a, s, tile, qtab);
         return;
     }
-#pragma unroll
+    const int L = (QK == QK_UNIF) ? unif_L(a.q.bits) : 0;
+    const float Lf = static_cast<float>(L);
+    const int64_t hint = ref.g0;
+#pragma unroll 1
     for (int k = 0; k < kSlots; ++k) {
         const int64_t qs = slot_of(tile, k);
         const int64_t j0 = 4 * qs;
+        float u[4];
+        load4(a.buf, qs, d, u);
         float U[4] = {0.f, 0.f, 0.f, 0.f};
         if (QK == QK_UNIF && a.q.stochastic && j0 < d) uniforms4(a.seed, a.id, a.t, j0, U);
         uint32_t c[4];
@@ -271,9 +287,9 @@ __global__ void __launch_bounds__(kThreads, 2) encode_kernel(const EncodeArgs a)
             c[i] = 0u;
             if (j0 + i < d) {
                 const float s = a.scales[group_of(G, j0 + i, hint)];
-                c[i] = encode1<QK>(u[k][i], s, a.q, Lf, L, U[i], dec, qtab);
+                c[i] = encode1<QK>(u[i], s, a.q, Lf, L, U[i], dec, qtab);
             }
-            e[i] = a.ef ? __fsub_rn(u[k][i], dec) : 0.0f;
+            e[i] = a.ef ? __fsub_rn(u[i], dec) : 0.0f;
         }
         store_codes4(a.words, qs, a.q.bits, c, 0, d);
         if (j0 < d) store4(a.buf, qs, d, e);
