@@ -30,12 +30,14 @@ struct QHost {
     bool has_scales = false;
     std::vector<int64_t> offsets;     // GK_SEG
     std::vector<TileRef> ref;         // groups that span tiles: every tile's groups
+    std::vector<int32_t> slow;        // see Grouping
     std::vector<int64_t> pair_base;   // PASS_STASH, PASS_GROUPED
     std::vector<int64_t> cuts;        // PASS_GROUPED: the waves
     int grid = 0, slots = 0;          // PASS_GROUPED: persistent CTAs and tile slots per CTA
     // device copies (inside the workspace)
     int64_t *d_offsets = nullptr, *d_pair_base = nullptr, *d_cuts = nullptr;
     TileRef *d_ref = nullptr;
+    int32_t *d_slow = nullptr;
     unsigned long long *d_arrive = nullptr;  // PASS_GROUPED: the wave barrier's counter
 };
 
@@ -43,6 +45,7 @@ struct QHost {
 struct Layout {
     size_t e_w, m_w, v_w, e_s, m_s, v_s, codes_w, scales_w, codes_s, scales_s, partials;
     size_t off_w, ref_w, pb_w, off_s, ref_s, pb_s, status;
+    size_t slow_w, slow_s;
     size_t cuts_w, arr_w, cuts_s, arr_s;  // the grouped pass (groups that span tiles)
     size_t rview;                         // PASS_LAZY: where a residual view is formed
     int64_t dpad, wcode_stride, wscale_stride;
@@ -220,6 +223,11 @@ int setup_quant(const ea_quantizer &q, int64_t d, const char *name, QHost &out)
                 part += g - g0 + 1;
                 g0 = group_end(g) == hi ? g + 1 : g;
             }
+            if (out.gkind == GK_SEG && n_tiles < (int64_t{1} << 31)) {
+                for (int64_t t = 0; t < n_tiles; ++t)
+                    if (out.ref[t].ng() > 1 || (t + 1) * kTile > d) out.slow.push_back(static_cast<int32_t>(t));
+                if (out.slow.size() > static_cast<size_t>(n_tiles / 8)) out.slow.clear();  // the common case then
+            }
         }
     }
     return EA_OK;
@@ -278,6 +286,8 @@ Layout make_layout(const ea_config &c, const QHost &qw, const QHost &qs)
     L.ref_s = qs.ref.size() * sizeof(TileRef);
     L.pb_s = qs.pass == PASS_STASH ? qs.pair_base.size() * 8 : 0;
     L.status = 4;
+    L.slow_w = qw.slow.size() * 4;
+    L.slow_s = qs.slow.size() * 4;
     // the grouped pass, whenever groups span tiles (ea_init picks it when its waves fit)
     const bool gw = qw.pass == PASS_STASH, gs = qs.pass == PASS_STASH;
     L.cuts_w = gw ? static_cast<size_t>(qw.n_groups + 1) * 8 : 0;
@@ -292,7 +302,7 @@ size_t layout_bytes(const Layout &L)
 {
     const size_t parts[] = {L.e_w, L.m_w, L.v_w, L.e_s, L.m_s, L.v_s, L.codes_w, L.scales_w, L.codes_s,
                             L.scales_s, L.partials, L.off_w, L.ref_w, L.pb_w, L.off_s, L.ref_s, L.pb_s, L.status,
-                            L.cuts_w, L.arr_w, L.cuts_s, L.arr_s, L.rview};
+                            L.cuts_w, L.arr_w, L.cuts_s, L.arr_s, L.rview, L.slow_w, L.slow_s};
     size_t total = 0;
     for (size_t p : parts) total += align_up(p, kAlign);
     return total;
@@ -307,6 +317,8 @@ Grouping device_grouping(const QHost &q)
     g.n_groups = q.n_groups;
     g.offsets = q.d_offsets;
     g.ref = q.d_ref;
+    g.slow = q.d_slow;
+    g.n_slow = static_cast<int>(q.slow.size());
     g.pair_base = q.d_pair_base;
     return g;
 }
@@ -660,6 +672,8 @@ int ea_init(const ea_config *cfg, void *workspace, size_t workspace_bytes, void 
     h->qs.d_cuts = reinterpret_cast<int64_t *>(take(L.cuts_s));
     h->qs.d_arrive = reinterpret_cast<unsigned long long *>(take(L.arr_s));
     h->rview = reinterpret_cast<float *>(take(L.rview));
+    h->qw.d_slow = reinterpret_cast<int32_t *>(take(L.slow_w));
+    h->qs.d_slow = reinterpret_cast<int32_t *>(take(L.slow_s));
     // scaled-sign messages whose groups span tiles: the sign codes need no scale, so one pass writes
     // them and keeps u (PASS_LAZY); its workspace is that of the two passes
     if (h->qw.pass == PASS_STASH && h->qw.kind == EA_Q_SIGN_L1) {
@@ -702,6 +716,8 @@ int ea_init(const ea_config *cfg, void *workspace, size_t workspace_bytes, void 
         if (r == EA_OK && n) r = check_cuda(h, cudaMemcpyAsync(dst, src, n, cudaMemcpyHostToDevice, s), "table upload");
     };
     upload(h->qw.d_offsets, h->qw.offsets.data(), L.off_w);
+    upload(h->qw.d_slow, h->qw.slow.data(), L.slow_w);
+    upload(h->qs.d_slow, h->qs.slow.data(), L.slow_s);
     upload(h->qw.d_ref, h->qw.ref.data(), L.ref_w);
     upload(h->qw.d_pair_base, h->qw.pair_base.data(), L.pb_w);
     upload(h->qs.d_offsets, h->qs.offsets.data(), L.off_s);

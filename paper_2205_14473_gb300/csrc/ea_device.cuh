@@ -83,28 +83,6 @@ __device__ __forceinline__ void df_accumulate(DF &acc, float x)
 // warp that does not take part in the reductions.
 __device__ __forceinline__ void compute_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kThreads) : "memory"); }
 
-// CTA-wide sum; every thread receives the same binary64 value (fixed combination order).
-__device__ __forceinline__ double block_sum(DF v, DF *red, double *bcast)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        DF w{__shfl_down_sync(0xffffffffu, v.hi, o), __shfl_down_sync(0xffffffffu, v.lo, o)};
-        v = df_add(v, w);
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) red[warp] = v;
-    compute_sync();
-    if (threadIdx.x == 0) {
-        DF t = red[0];
-#pragma unroll
-        for (int w = 1; w < kWarps; ++w) t = df_add(t, red[w]);
-        *bcast = static_cast<double>(t.hi) + static_cast<double>(t.lo);
-    }
-    compute_sync();
-    const double r = *bcast;
-    return r;
-}
-
 // Group scale of the scaled sign, ||u||_1 / G, for a group that is exactly this CTA's tile.
 // Every thread leaves its partial pair in red256; warp 0 combines the 256 pairs (8 per lane in a
 // tree, then a 5-level shuffle tree) and broadcasts the scale through *bcastf.  For G a
@@ -186,24 +164,6 @@ __device__ __forceinline__ float block_max_warp0(float a, uint32_t *red)
     if (lane == 0) red[threadIdx.x >> 5] = b;
     compute_sync();
     return threadIdx.x < 32 ? __uint_as_float(__reduce_max_sync(0xffffffffu, lane < kWarps ? red[lane] : 0u)) : 0.0f;
-}
-
-// CTA-wide maximum of non-negative values (exact: compares bit patterns).
-__device__ __forceinline__ float block_max(float a, uint32_t *red, float *bcast)
-{
-    const uint32_t b = __reduce_max_sync(0xffffffffu, __float_as_uint(a));
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) red[warp] = b;
-    compute_sync();
-    if (threadIdx.x == 0) {
-        uint32_t m = red[0];
-#pragma unroll
-        for (int w = 1; w < kWarps; ++w) m = max(m, red[w]);
-        *bcast = __uint_as_float(m);
-    }
-    compute_sync();
-    const float r = *bcast;
-    return r;
 }
 
 // Group scale of the scaled sign: ||u||_1 / G, the division in binary64, one rounding to binary32.
@@ -396,8 +356,40 @@ __host__ __device__ __forceinline__ int chunk_shift(const Grouping &g)
     return (g.gkind == GK_BLOCK && g.log2G >= kLog2Chunk && g.log2G < 12) ? g.log2G - kLog2Chunk : 5;
 }
 
-// The segments (GK_SEG) of one tile, for per-coordinate lookups from shared memory: the tile's
-// first group and the offsets, from the tile's start, of the groups that start inside it.
+// Which tile a CTA of a kernel with a CTA per tile takes.  What takes longer than a whole tile inside one
+// group -- a ragged last tile, a tile of several groups -- is a path of its own, and goes first, where
+// the rest of the grid runs beside it, and not into the last wave.  So the tiles are taken last first;
+// and where a few segments' boundaries make such tiles (Grouping::slow lists them, a ragged last one
+// among them), the first n_slow CTAs take those, and the CTAs whose turn they would be (the grid has
+// n_slow more) have none.  TBD
+struct CtaTile {
+    int64_t tile;  // -1: none
+    bool plain;    // a whole tile inside one group
+    TileRef ref;
+};
+__device__ __forceinline__ CtaTile cta_tile(const Grouping &g, int64_t d)
+{
+    CtaTile t;
+    t.plain = false;
+    if (static_cast<int>(blockIdx.x) < g.n_slow) {
+        t.tile = g.slow[blockIdx.x];
+        t.ref = tile_ref(g, t.tile, d);
+        return t;
+    }
+    t.tile = static_cast<int64_t>(gridDim.x - 1 - blockIdx.x);
+    t.ref = tile_ref(g, t.tile, d);
+    t.plain = t.ref.ng() == 1 && (t.tile + 1) * kTile <= d;
+    if (!t.plain && g.n_slow) t.tile = -1;
+    return t;
+}
+// The same tile again on the plain path (blockIdx arithmetic: it stays out of the threads' registers).
+__device__ __forceinline__ int64_t plain_tile() { return static_cast<int64_t>(gridDim.x - 1 - blockIdx.x); }
+
+// The groups (segments or blocks) of one tile, for per-coordinate lookups from shared memory: the
+// tile's first group and the offsets, from the tile's start, of the groups that start inside it.
+// What is done with them is written in rolled loops: a tile that holds several groups is rare, its code
+// is fetched cold, and unrolled over a thread's 16 coordinates that took longer than the rest of the
+// kernel.  TBD
 constexpr int kTileBounds = 64;
 struct TileGroups {
     int64_t g0;
@@ -418,7 +410,7 @@ __device__ __forceinline__ void cache_tile_groups(const Grouping &g, int64_t til
     }
     if (nb <= kTileBounds)
         for (int i = threadIdx.x; i < nb; i += blockDim.x)
-            tg.b[i] = static_cast<uint16_t>(g.offsets[g0 + 1 + i] - tl);
+            tg.b[i] = static_cast<uint16_t>((g.gkind == GK_BLOCK ? (g0 + 1 + i) * g.G : g.offsets[g0 + 1 + i]) - tl);
 }
 
 // Group of coordinate j of the cached tile (falls back to the global scan past kTileBounds groups).

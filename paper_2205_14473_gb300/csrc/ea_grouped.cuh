@@ -30,77 +30,12 @@ constexpr int kRangeScales = kGroupedScales;  // scales of the groups a CTA enco
 
 // Per-CTA shared state of the grouped kernels.
 struct GroupSmem {
-    DF red[2][kWarps];            // per-warp partial sums, by parity of the reduction's turn
-    uint32_t redm[2][kWarps];     // per-warp partial maxima, likewise
+    PartRed parts;                // group_partials
     float qtab[256];              // the message's uniform grid fl(i / L) (build_qtab)
     int abort;                    // the wave barrier ran out of time: the CTA stops
     float gsc[kRangeScales];      // scales of the groups of the CTA's ranges in this wave, in order
     TileGroups tg;                // segments of a tile that holds several
 };
-
-// For every group of Q that meets [lo, hi) (a range of tile `tile`), reduce this CTA's part of it
-// -- |u| summed (compensated, to ~2^-44) for the scaled sign, max |u| for Example 1's grid -- over
-// u in ub and store it as the group's partial for this tile.  One barrier per group: the warps'
-// results go to red[turn & 1] and thread 0 combines them in warp order.  All threads call it.
-template <int QK>
-__device__ __forceinline__ void range_partials(const float4 *ub, int64_t tile, int64_t lo, int64_t hi, int64_t d,
-                                               const QParams &q, double *partials, GroupSmem &gs, int &turn)
-{
-    const Grouping &G = q.grp;
-    const TileRef ref = tile_ref(G, tile, d);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int64_t gi = ref.ng() == 1 ? ref.g0 : group_of(G, lo, ref.g0);; ++gi, ++turn) {
-        const int64_t gb = group_begin(G, gi, d), ge = group_end(G, gi, d);
-        const int64_t a = max(gb, lo), b = min(ge, hi);
-        const int par = turn & 1;
-        if constexpr (QK == QK_SIGN) {
-            DF acc{0.0f, 0.0f};
-#pragma unroll
-            for (int k = 0; k < kSlots; ++k) {
-                const int64_t j0 = 4 * slot_of(tile, k);
-                const float4 v = ub[k * kThreads + threadIdx.x];
-                const float u[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    if (j0 + i >= a && j0 + i < b) df_accumulate(acc, fabsf(u[i]));
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const DF w{__shfl_down_sync(0xffffffffu, acc.hi, o), __shfl_down_sync(0xffffffffu, acc.lo, o)};
-                acc = df_add(acc, w);
-            }
-            if (lane == 0) gs.red[par][warp] = acc;
-            compute_sync();
-            if (threadIdx.x == 0) {
-                DF t = gs.red[par][0];
-#pragma unroll
-                for (int w = 1; w < kWarps; ++w) t = df_add(t, gs.red[par][w]);
-                partials[ref.part() + (gi - ref.g0)] = static_cast<double>(t.hi) + static_cast<double>(t.lo);
-            }
-        } else {
-            float mx = 0.0f;
-#pragma unroll
-            for (int k = 0; k < kSlots; ++k) {
-                const int64_t j0 = 4 * slot_of(tile, k);
-                const float4 v = ub[k * kThreads + threadIdx.x];
-                const float u[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    if (j0 + i >= a && j0 + i < b) mx = fmaxf(mx, fabsf(u[i]));
-            }
-            const uint32_t m = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));  // exact on bit patterns
-            if (lane == 0) gs.redm[par][warp] = m;
-            compute_sync();
-            if (threadIdx.x == 0) {
-                uint32_t t = gs.redm[par][0];
-#pragma unroll
-                for (int w = 1; w < kWarps; ++w) t = max(t, gs.redm[par][w]);
-                partials[ref.part() + (gi - ref.g0)] = static_cast<double>(__uint_as_float(t));
-            }
-        }
-        if (ge >= hi) break;
-    }
-}
 
 // The wave barrier: every CTA's partials of wave w are stored once all gridDim.x CTAs have arrived
 // (arrivals count across waves and launches: this one completes at (epoch * n_waves + w + 1) *

@@ -68,6 +68,8 @@ struct Grouping {
     const int64_t *offsets;     // GK_SEG: n_groups + 1 offsets (device)
     const TileRef *ref;         // every tile's groups (device); null for GK_WHOLE, and where every
                                 // group lies inside one tile
+    const int32_t *slow;        // GK_SEG: the tiles that hold several groups, and a ragged last one, in
+    int n_slow;                 // order (device), if they are few; a kernel takes these first (cta_tile)
     const int64_t *pair_base;   // n_groups + 1: first partial-sum slot of each group (device)
 };
 

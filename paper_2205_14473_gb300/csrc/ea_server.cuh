@@ -138,6 +138,7 @@ __global__ void __launch_bounds__(kThreads, 2) server_kernel(const ServerArgs a)
     __shared__ float utab_s[256];  // fl(i / L) for the workers' uniform grid, i = -L..L (b_w <= 8)
     __shared__ float stab[256];
     __shared__ TileGroups tg;
+    __shared__ float4 ubuf[kSlots * kThreads];
     const int64_t tile = blockIdx.x;
     const int64_t d = a.d;
 
@@ -146,10 +147,11 @@ __global__ void __launch_bounds__(kThreads, 2) server_kernel(const ServerArgs a)
     if (has_scale<QS>() && a.pass == PASS_STASH) {
         ref = tile_ref(a.qs.grp, tile, d);
         if (threadIdx.x == 0) sm.part = ref.part();
+        if (ref.ng() > 1) cache_tile_groups(a.qs.grp, tile, d, sm.tg);  // read after the decode's barriers
     }
     build_qtab<QS>(a.qs, sm.qtab);  // read after the scale reduction's barrier
     const float *utab = build_worker_utab<QW>(a, utab_s);
-    if (utab) __syncthreads();
+    __syncthreads();
     pdl_wait();
 
     float es[kSlots][4], ms[kSlots][4], vs[kSlots][4];
@@ -168,32 +170,34 @@ __global__ void __launch_bounds__(kThreads, 2) server_kernel(const ServerArgs a)
     const float nf = static_cast<float>(a.n);
     const bool pow2n = (a.n & (a.n - 1)) == 0;
     const float inv_n = __frcp_rn(nf);  // exact when n is a power of two
-    float u[kSlots][4];
 #pragma unroll
     for (int k = 0; k < kSlots; ++k) {
         const int64_t q = slot_of(tile, k);
         const int64_t j0 = 4 * q;
+        float u[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             float step = pow2n ? __fmul_rn(acc[k][i], inv_n) : __fdiv_rn(acc[k][i], nf);
             if (MODE == MODE_S) step = adam_step(step, ms[k][i], vs[k][i], a.hp);
-            u[k][i] = (j0 + i < d) ? __fadd_rn(step, es[k][i]) : 0.0f;
+            u[i] = (j0 + i < d) ? __fadd_rn(step, es[k][i]) : 0.0f;
         }
+        ubuf[k * kThreads + threadIdx.x] = to_f4(u);
         if (MODE == MODE_S && j0 < d) {
             store4(a.ms, q, d, ms[k]);
             store4(a.vs, q, d, vs[k]);
         }
     }
-    finish_tile<QS>(URegs{u}, tile, d, a.qs, a.words, a.scales, a.es, a.ef, a.pass, a.seed,
+    finish_tile<QS>(USmem{ubuf}, tile, d, a.qs, a.words, a.scales, a.es, a.ef, a.pass, a.seed,
                     static_cast<uint32_t>(a.n), a.t, a.partials, sm, ref);
 }
 
 // Phase one of a grouped server tile: w (the average, after the Adam step with Adam at the server,
 // plus e_s) of the coordinate range [lo, hi) of tile `tile` (0 elsewhere) into ub; m_s and v_s
-// updated and stored in the range.  FULL: the range is the whole tile.  rs: Q_s's groups (LAZY).
+// updated and stored in the range.  FULL: the range is the whole tile.  rs, tgs: Q_s's groups (LAZY).
 template <int MODE, int QW, bool FULL, bool LAZY = false>
 __device__ __forceinline__ void server_u_range(const ServerArgs &a, int64_t tile, int64_t lo, int64_t hi, float4 *ub,
-                                               const float *utab, float *stab, TileGroups &tg, const TileRef &rs)
+                                               const float *utab, float *stab, TileGroups &tg, const TileRef &rs,
+                                               const TileGroups *tgs)
 {
     LazyScale lzs{};
     if (LAZY && a.lazy_in) lzs = lazy_scale_of_tile(rs, a.scales);
@@ -214,7 +218,7 @@ __device__ __forceinline__ void server_u_range(const ServerArgs &a, int64_t tile
                 load4<FULL>(a.ms, q, hi, ms);
                 load4<FULL>(a.vs, q, hi, vs);
             }
-            if (LAZY && a.lazy_in) lazy_residual4<FULL>(a.qs, a.scales, lzs, j0, hi, es);
+            if (LAZY && a.lazy_in) lazy_residual4<FULL>(a.qs, a.scales, lzs, *tgs, tile, j0, hi, es);
         }
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -314,7 +318,7 @@ __device__ __forceinline__ void decode_sum_staged(const ServerArgs &a, int64_t t
 #pragma unroll
         for (int k = 0; k < kSlots; ++k) {
             const int64_t j0 = 4 * slot_of(tile, k);
-#pragma unroll
+#pragma unroll 1
             for (int i = 0; i < 4; ++i) {
                 const int64_t j = j0 + i < a.d ? j0 + i : a.d - 1;
                 const int64_t g = (seg ? tile_group_of(GW, tg, tile, j) : group_of(GW, j, gw0)) - gw0;
@@ -366,7 +370,7 @@ __device__ __forceinline__ void decode_sum_staged(const ServerArgs &a, int64_t t
 // replaces the codes in ub (0 outside the range); m_s, v_s are updated and stored in the range.
 // Returns false, having done nothing, when the tile's scale table would not fit (the caller then
 // takes server_u_range).  rw, rs: the tile's groups of Q_w and (LAZY) Q_s, which the caller looked up
-// early; tgs: room for Q_s's segments of a tile that holds several (LAZY).
+// early; tgs: Q_s's groups of a tile that holds several, and gs.tg Q_w's (LAZY; filled by the caller).
 template <int MODE, int QW, bool FULL, bool LAZY = false>
 __device__ __forceinline__ bool server_u_staged(const ServerArgs &a, int64_t tile, int64_t lo, int64_t hi, float4 *ub,
                                                 const float *utab, float *stab, float *wsc, GroupSmem &gs,
@@ -377,9 +381,9 @@ __device__ __forceinline__ bool server_u_staged(const ServerArgs &a, int64_t til
     const int bw = code_bits<QW>(a.qw);
     const Grouping &GW = a.qw.grp;
     const int64_t gw0 = has_scale<QW>() ? rw.g0 : 0;
-    const int ngw = has_scale<QW>() ? rw.ng() : 1;
+    const int ngw = (has_scale<QW>() && !(LAZY && FULL)) ? rw.ng() : 1;  // LAZY: FULL tiles lie in one group
     if (n * ngw > kWorkerScales || ngw > kStagedTileGroups) return false;
-    const bool seg = has_scale<QW>() && ngw > 1 && GW.gkind == GK_SEG;
+    const bool seg = has_scale<QW>() && ngw > 1;
     float es[kSlots][4], ms[kSlots][4], vs[kSlots][4];
     bool in[kSlots];
 #pragma unroll
@@ -419,8 +423,7 @@ __device__ __forceinline__ bool server_u_staged(const ServerArgs &a, int64_t til
             for (int i = threadIdx.x; i < n * ngw; i += kThreads)
                 cp_async4(wsc + i, a.wscales + static_cast<int64_t>(i / ngw) * a.wscales_stride + gw0 + i % ngw);
         }
-        if (LAZY && a.lazy_in && lzs.g1 < 0 && a.qs.grp.gkind == GK_SEG) cache_tile_groups(a.qs.grp, tile, d, *tgs);
-        if (seg) cache_tile_groups(GW, tile, d, gs.tg);
+        if (seg && !LAZY) cache_tile_groups(GW, tile, d, gs.tg);
         cp_async_wait_all();
     }
     compute_sync();
@@ -429,24 +432,7 @@ __device__ __forceinline__ bool server_u_staged(const ServerArgs &a, int64_t til
     compute_sync();  // every thread has read the staged codes
     if constexpr (LAZY) {
         if (a.lazy_in) {  // es holds the previous round's w: its residual (lo is the tile's start)
-            const bool segs = lzs.g1 < 0 && a.qs.grp.gkind == GK_SEG;
-#pragma unroll
-            for (int k = 0; k < kSlots; ++k) {
-                if (!in[k]) continue;
-                const int64_t j0 = 4 * slot_of(tile, k);
-                if (!segs) {
-                    lazy_residual4<FULL>(a.qs, a.scales, lzs, j0, hi, es[k]);
-                    continue;
-                }
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    if (!FULL && j0 + i >= hi) continue;
-                    float dec;
-                    (void)encode1<QK_SIGN>(es[k][i], __ldg(a.scales + tile_group_of(a.qs.grp, *tgs, tile, j0 + i)), a.qs,
-                                           0.0f, 0, 0.0f, dec);
-                    es[k][i] = __fsub_rn(es[k][i], dec);
-                }
-            }
+            lazy_residual<FULL, FULL>(a.qs, a.scales, lzs, *tgs, ub, tile, hi, es);
         }
     }
     const float nf = static_cast<float>(n);
@@ -506,10 +492,10 @@ __global__ void __launch_bounds__(kThreads, MODE == MODE_S ? 2 : 3) server_group
                             : server_u_staged<MODE, QW, false>(a, tile, lo, hi, ub, utab, stab, wsc, gs, rw, rw, nullptr);
             if (!done) {
                 compute_sync();  // stab's and tg's previous readers are done
-                if (full) server_u_range<MODE, QW, true>(a, tile, lo, hi, ub, utab, stab, gs.tg, rw);
-                else server_u_range<MODE, QW, false>(a, tile, lo, hi, ub, utab, stab, gs.tg, rw);
+                if (full) server_u_range<MODE, QW, true>(a, tile, lo, hi, ub, utab, stab, gs.tg, rw, nullptr);
+                else server_u_range<MODE, QW, false>(a, tile, lo, hi, ub, utab, stab, gs.tg, rw, nullptr);
             }
-            range_partials<QS>(ub, tile, lo, hi, a.d, a.qs, a.partials, gs, turn);
+            group_partials<QS>(USmem{ub}, tile, lo, hi, a.d, a.qs, tile_ref(a.qs.grp, tile, a.d), nullptr, a.partials, gs.parts, turn);
         }
         if (!wave_barrier(gp, w, a.status, gs)) return;
         encode_wave<QS>(uslot, t0, t_end, c0, c1, a.d, a.qs, a.words, a.partials, a.scales, a.es, a.ef, a.seed,
@@ -517,6 +503,48 @@ __global__ void __launch_bounds__(kThreads, MODE == MODE_S ? 2 : 3) server_group
     }
 }
 
+
+// One tile of server_lazy_kernel; PLAIN: a whole tile inside one group of each message.
+template <int MODE, int QW, bool STAGED, bool PLAIN>
+__device__ __forceinline__ void server_lazy_tile(const ServerArgs &a, int64_t tile, const TileRef &rw, const TileRef &rs,
+                                                 float4 *ub, const float *utab, float *stab, float *wsc, GroupSmem &gs,
+                                                 TileGroups &tgs, DF *red256)
+{
+    const int64_t d = a.d, lo = tile * kTile, hi = PLAIN ? lo + kTile : min(lo + static_cast<int64_t>(kTile), d);
+    if constexpr (STAGED) {
+        if (!server_u_staged<MODE, QW, PLAIN, true>(a, tile, lo, hi, ub, utab, stab, wsc, gs, rw, rs, &tgs)) {
+            // outside what the host checked: report it, store nothing
+            if (threadIdx.x == 0) report_status(a.status, kStatusCheck);
+            return;
+        }
+    } else {
+        server_u_range<MODE, QW, PLAIN, true>(a, tile, lo, hi, ub, utab, stab, gs.tg, rs, &tgs);
+    }
+    DF acc{0.0f, 0.0f};
+#pragma unroll
+    for (int k = 0; k < kSlots; ++k) {
+        const int64_t qs = slot_of(tile, k);
+        const float4 v = ub[k * kThreads + threadIdx.x];
+        const float w[4] = {v.x, v.y, v.z, v.w};
+        uint32_t c[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            float dec;
+            const uint32_t code = encode1<QK_SIGN>(w[i], 0.0f, a.qs, 0.0f, 0, 0.0f, dec);
+            c[i] = (PLAIN || 4 * qs + i < d) ? code : 0u;
+            df_accumulate(acc, fabsf(w[i]));  // w beyond d is 0
+        }
+        store_codes4<PLAIN, false>(a.words, qs, 1, c, 0, d);
+        if (a.ef && (PLAIN || 4 * qs < d)) store4<PLAIN>(a.es, qs, d, w);
+    }
+    if (PLAIN || rs.ng() == 1) {  // the tile's norm is the one group's partial
+        const DF tot = block_sum_lane0(acc, red256);
+        if (threadIdx.x == 0) a.partials[rs.part()] = static_cast<double>(tot.hi) + static_cast<double>(tot.lo);
+        return;
+    }
+    int turn = 0;
+    group_partials<QK_SIGN>(USmem{ub}, tile, lo, hi, d, a.qs, rs, &tgs, a.partials, gs.parts, turn);
+}
 
 // PASS_LAZY for a scaled-sign broadcast whose groups span tiles, one CTA per tile.  w (the average,
 // after the Adam step with Adam at the server, plus the residual formed from the previous round's
@@ -535,57 +563,25 @@ __global__ void __launch_bounds__(kThreads, MODE == MODE_S ? 2 : 3) server_lazy_
     __shared__ DF red256[kThreads];
     __shared__ TileGroups tgs;
     pdl_trigger();
-    const int64_t tile = blockIdx.x;
-    const int64_t d = a.d, lo = tile * kTile, hi = min(lo + static_cast<int64_t>(kTile), d);
-    // both messages' groups of the tile and the decode table before the predecessor has finished (the
-    // first barrier of the decode lies between the table and its readers)
-    const TileRef rw = has_scale<QW>() ? tile_ref(a.qw.grp, tile, d) : TileRef{0, 1};
-    const TileRef rs = tile_ref(a.qs.grp, tile, d);
+    const CtaTile ct = cta_tile(a.qs.grp, a.d);
+    if (ct.tile < 0) return;
+    // both messages' groups of the tile and the decode table before the predecessor has finished
+    const TileRef rw = has_scale<QW>() ? tile_ref(a.qw.grp, ct.tile, a.d) : TileRef{0, 1};
     const float *utab = build_worker_utab<QW>(a, utab_s);
-    if constexpr (!STAGED) __syncthreads();
+    if (STAGED && has_scale<QW>() && rw.ng() > 1) cache_tile_groups(a.qw.grp, ct.tile, a.d, gs.tg);
+    if (ct.ref.ng() > 1) cache_tile_groups(a.qs.grp, ct.tile, a.d, tgs);
+    __syncthreads();
     pdl_wait();
-    const bool full = hi == lo + kTile;
-    if constexpr (STAGED) {
-        const bool done = full ? server_u_staged<MODE, QW, true, true>(a, tile, lo, hi, ub, utab, stab, wsc, gs, rw, rs, &tgs)
-                               : server_u_staged<MODE, QW, false, true>(a, tile, lo, hi, ub, utab, stab, wsc, gs, rw, rs, &tgs);
-        if (!done) {  // outside what the host checked: report it, store nothing
-            if (threadIdx.x == 0) report_status(a.status, kStatusCheck);
-            return;
-        }
-    } else {
-        if (full) server_u_range<MODE, QW, true, true>(a, tile, lo, hi, ub, utab, stab, gs.tg, rs);
-        else server_u_range<MODE, QW, false, true>(a, tile, lo, hi, ub, utab, stab, gs.tg, rs);
-    }
-    DF acc{0.0f, 0.0f};
-#pragma unroll
-    for (int k = 0; k < kSlots; ++k) {
-        const int64_t qs = slot_of(tile, k);
-        const float4 v = ub[k * kThreads + threadIdx.x];
-        const float w[4] = {v.x, v.y, v.z, v.w};
-        uint32_t c[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            float dec;
-            const uint32_t code = encode1<QK_SIGN>(w[i], 0.0f, a.qs, 0.0f, 0, 0.0f, dec);
-            c[i] = (4 * qs + i < d) ? code : 0u;
-            df_accumulate(acc, fabsf(w[i]));  // w beyond d is 0
-        }
-        store_codes4<false, false>(a.words, qs, 1, c, 0, d);
-        if (a.ef && 4 * qs < d) store4(a.es, qs, d, w);
-    }
-    if (rs.ng() == 1) {  // the tile's norm is the one group's partial
-        const DF tot = block_sum_lane0(acc, red256);
-        if (threadIdx.x == 0) a.partials[rs.part()] = static_cast<double>(tot.hi) + static_cast<double>(tot.lo);
-        return;
-    }
-    int turn = 0;
-    range_partials<QK_SIGN>(ub, tile, lo, hi, d, a.qs, a.partials, gs, turn);
+    if (ct.plain && rw.ng() == 1)
+        server_lazy_tile<MODE, QW, STAGED, true>(a, plain_tile(), rw, ct.ref, ub, utab, stab, wsc, gs, tgs, red256);
+    else
+        server_lazy_tile<MODE, QW, STAGED, false>(a, ct.tile, rw, ct.ref, ub, utab, stab, wsc, gs, tgs, red256);
 }
 
 template <int MODE, bool STAGED>
 static cudaError_t launch_server_lazy_st(const ServerArgs &a, cudaStream_t s)
 {
-    const dim3 grid(static_cast<unsigned>(a.n_tiles)), block(kThreads);
+    const dim3 grid(static_cast<unsigned>(a.n_tiles + a.qs.grp.n_slow)), block(kThreads);
     switch (a.qw.kind) {
     case QK_SIGN: return launch_pdl(server_lazy_kernel<MODE, QK_SIGN, STAGED>, grid, block, 0, s, true, kCarveoutPercent, a);
     case QK_UNIF: return launch_pdl(server_lazy_kernel<MODE, QK_UNIF, STAGED>, grid, block, 0, s, true, kCarveoutPercent, a);
@@ -938,8 +934,8 @@ __device__ __forceinline__ bool server_staged_tile(const ServerArgs &a, int64_t 
         }
     }
     if constexpr (GENERAL && has_scale<QS>()) {
-        constexpr int spans = QS == QK_SIGN ? PASS_LAZY : PASS_STASH;  // groups that span tiles
-        if (a.pass == spans)
+        constexpr int spans = QS == QK_SIGN ? PASS_LAZY_ONE : PASS_STASH_ONE;  // groups of several tiles
+        if (a.pass == (QS == QK_SIGN ? PASS_LAZY : PASS_STASH))
             finish_tile<QS, FULL, false, spans>(USmem{ubuf}, tile, d, a.qs, a.words, a.scales, a.es, a.ef, spans, a.seed,
                                                 static_cast<uint32_t>(a.n), a.t, a.partials, sm, ref);
         else
@@ -1000,7 +996,8 @@ __global__ void __launch_bounds__(kThreads + 32, server_ctas_per_sm(MODE, QW, QS
     if (warp == kWarps) {  // ---------------------------------------------------------- producer
         int64_t it = 0;
         bool ok = true;
-        for (int64_t tile = blockIdx.x; tile < a.n_tiles; tile += gridDim.x, ++it) {
+        for (int64_t at = blockIdx.x; at < a.n_tiles; at += gridDim.x, ++it) {
+            const int64_t tile = a.n_tiles - 1 - at;  // the ragged one first (see cta_tile)
             const int s = static_cast<int>(it % S);
             if (it >= S && !mbar_wait(&empty[s], static_cast<uint32_t>(((it / S) & 1) ^ 1))) {
                 ok = false;
@@ -1054,7 +1051,8 @@ __global__ void __launch_bounds__(kThreads + 32, server_ctas_per_sm(MODE, QW, QS
     for (int w = 0; w < 8; ++w) flip[w] = ((threadIdx.x >> w) & 1u) ? 0u : 0x80000000u;
     const bool n8 = a.n == 8;  // full tiles with eight workers: the compile-time count
     int64_t it = 0;
-    for (int64_t tile = blockIdx.x; tile < a.n_tiles; tile += gridDim.x, ++it) {
+    for (int64_t at = blockIdx.x; at < a.n_tiles; at += gridDim.x, ++it) {
+        const int64_t tile = a.n_tiles - 1 - at;
         const int s = static_cast<int>(it % S);
         // bounded wait; the tile's first barrier makes every compute thread agree on the outcome
         const bool ok = mbar_wait(&full[s], static_cast<uint32_t>((it / S) & 1));

@@ -8,11 +8,17 @@
 
 namespace ea {
 
+// Per-warp results of group_partials, by parity of the reduction's turn.
+struct PartRed {
+    DF red[2][kWarps];
+    uint32_t redm[2][kWarps];
+};
+
 struct TileSmem {
     DF red256[kThreads];  // per-thread partial pairs of the l1 scale
-    DF red[kWarps];
+    PartRed parts;
+    TileGroups tg;        // PASS_STASH, PASS_LAZY: the groups of a tile that holds several
     uint32_t redm[kWarps];
-    double bcast;
     float bcastf;
     float csc[kChunks];  // PASS_SHORT: the scale of each chunk
     int64_t part;        // PASS_STASH, PASS_LAZY: the tile's first partial norm (thread 0 writes and reads it)
@@ -56,6 +62,81 @@ template <class Scale>
 constexpr bool kPerSlot = false;
 template <>
 constexpr bool kPerSlot<ChunkScales> = true;
+
+// For every group of Q that meets [lo, hi) (a range of tile `tile`), reduce this CTA's part of it
+// -- |u| summed (compensated, to ~2^-44) for the scaled sign, max |u| for Example 1's grid -- over
+// u read through `src` (shared memory) and store it as the group's partial for this tile.  One barrier per
+// group: the warps' results go to pr by turn & 1 and thread 0 combines them in warp order.  tg: the
+// tile's groups in shared memory, or null.  All threads call it.
+template <int QK>
+__device__ __forceinline__ void group_partials(const USmem &src, int64_t tile, int64_t lo, int64_t hi, int64_t d,
+                                               const QParams &q, const TileRef &ref, const TileGroups *tg,
+                                               double *partials, PartRed &pr, int &turn)
+{
+    const Grouping &G = q.grp;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t tl = tile * kTile;
+    const int end = static_cast<int>(hi - tl);
+    const bool cached = tg != nullptr && tg->nb <= kTileBounds;
+#pragma unroll 1
+    for (int64_t gi = (ref.ng() == 1 || lo == tl) ? ref.g0 : group_of(G, lo, ref.g0);; ++gi, ++turn) {
+        const int i0 = static_cast<int>(gi - ref.g0);
+        int a = 0, b = kTile;  // the group's part of the range, from the tile's start
+        if (cached) {
+            if (i0 > 0) a = tg->b[i0 - 1];
+            if (i0 < tg->nb) b = tg->b[i0];
+        } else if (ref.ng() > 1) {
+            a = static_cast<int>(max(group_begin(G, gi, d) - tl, static_cast<int64_t>(0)));
+            b = static_cast<int>(min(group_end(G, gi, d) - tl, static_cast<int64_t>(kTile)));
+        }
+        a = max(a, static_cast<int>(lo - tl));
+        const bool last = b >= end;
+        b = min(b, end);
+        const int par = turn & 1;
+        DF acc{0.0f, 0.0f};
+        float mx = 0.0f;
+#pragma unroll 1
+        for (int k = 0; k < kSlots; ++k) {
+            const int x = 4 * (k * kThreads + threadIdx.x);
+            float u[4];
+            src.get(k, u);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (x + i < a || x + i >= b) continue;
+                if constexpr (QK == QK_SIGN) df_accumulate(acc, fabsf(u[i]));
+                else mx = fmaxf(mx, fabsf(u[i]));
+            }
+        }
+        if constexpr (QK == QK_SIGN) {
+#pragma unroll 1
+            for (int o = 16; o > 0; o >>= 1) {
+                const DF w{__shfl_down_sync(0xffffffffu, acc.hi, o), __shfl_down_sync(0xffffffffu, acc.lo, o)};
+                acc = df_add(acc, w);
+            }
+            if (lane == 0) pr.red[par][warp] = acc;
+        } else {
+            const uint32_t m = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));  // exact on bit patterns
+            if (lane == 0) pr.redm[par][warp] = m;
+        }
+        compute_sync();
+        if (threadIdx.x == 0) {
+            double part;
+            if constexpr (QK == QK_SIGN) {
+                DF t = pr.red[par][0];
+#pragma unroll 1
+                for (int w = 1; w < kWarps; ++w) t = df_add(t, pr.red[par][w]);
+                part = static_cast<double>(t.hi) + static_cast<double>(t.lo);
+            } else {
+                uint32_t t = pr.redm[par][0];
+#pragma unroll 1
+                for (int w = 1; w < kWarps; ++w) t = max(t, pr.redm[par][w]);
+                part = static_cast<double>(__uint_as_float(t));
+            }
+            partials[ref.part() + i0] = part;
+        }
+        if (last) break;
+    }
+}
 
 // PASS_SHORT: the scales of the tile's blocks of 2^sh chunks, from u read through `src`, into
 // sm.csc (one per chunk) and scales[].  A warp reduces its four chunks at once: for the scaled sign
@@ -287,6 +368,7 @@ __device__ __forceinline__ void finish_tile_smem(const float4 *ubuf, DF l1, floa
 // by the worker's kernel (the general form's group lookups cost registers: with Adam at the worker,
 // a single form for both spilled 92 bytes a thread, and ResNet-18's messages took 5% longer).
 constexpr int PASS_LAZY_ONE = 16;
+constexpr int PASS_STASH_ONE = 17;  // likewise PASS_STASH, where the caller knows it
 
 // The tile's end for a quantizer with scale groups, u read through `src` (URegs or USmem).
 //   PASS_FUSED: the tile is exactly one scale group (blocks of 4096): reduce, encode, store.
@@ -296,7 +378,8 @@ constexpr int PASS_LAZY_ONE = 16;
 // tile loop is instruction-bound).
 // PASS: PASS_FUSED, PASS_SHORT or PASS_STASH as a compile-time constant (the other path is then not compiled
 // in), or -1 to follow `pass`.
-// ref (PASS_STASH, PASS_LAZY): the tile's groups; sm.part is set by the caller.
+// ref (PASS_STASH, PASS_LAZY): the tile's groups; sm.part, and sm.tg where they are several, are set
+// by the caller.  src is then USmem, or u is in shared memory (only the one-group forms take URegs).
 template <int QK, bool FULL = false, bool BALLOT = true, int PASS = -1, class USrc>
 __device__ __forceinline__ void finish_tile(const USrc &src, int64_t tile, int64_t d, const QParams &q,
                                             uint32_t *words, float *scales, float *resid, int ef, int pass,
@@ -349,6 +432,8 @@ __device__ __forceinline__ void finish_tile(const USrc &src, int64_t tile, int64
         // the residual is formed from it and the scale later (lazy_residual; without error feedback
         // the residual stays 0), and the codes now: the sign of u needs no scale.  PASS_LAZY_ONE forms
         // the norm on the way.
+        constexpr bool lazy = PASS == PASS_LAZY || PASS == PASS_LAZY_ONE;
+        constexpr bool one = PASS == PASS_LAZY_ONE || PASS == PASS_STASH_ONE;
         DF all{0.0f, 0.0f};
 #pragma unroll
         for (int k = 0; k < kSlots; ++k) {
@@ -358,12 +443,12 @@ __device__ __forceinline__ void finish_tile(const USrc &src, int64_t tile, int64
             if constexpr (PASS == PASS_LAZY_ONE)
 #pragma unroll
                 for (int i = 0; i < 4; ++i) df_accumulate(all, fabsf(uk[i]));  // u beyond d is 0
-            if constexpr (PASS != PASS_LAZY && PASS != PASS_LAZY_ONE) {
+            if constexpr (!lazy) {
                 if (FULL || 4 * qs < d) store4_kept<FULL>(resid, qs, d, uk);
             } else {
                 if (ef && (FULL || 4 * qs < d)) store4<FULL>(resid, qs, d, uk);
             }
-            if constexpr ((PASS == PASS_LAZY || PASS == PASS_LAZY_ONE) && QK == QK_SIGN) {
+            if constexpr (lazy && QK == QK_SIGN) {
                 uint32_t c[4];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
@@ -374,7 +459,7 @@ __device__ __forceinline__ void finish_tile(const USrc &src, int64_t tile, int64
                 store_codes4<FULL, BALLOT>(words, qs, 1, c, 0, d);
             }
         }
-        if (PASS == PASS_LAZY_ONE || ref.ng() == 1) {
+        if (one || ref.ng() == 1) {
             if constexpr (QK == QK_SIGN) {
                 if constexpr (PASS != PASS_LAZY_ONE)
 #pragma unroll
@@ -400,38 +485,9 @@ __device__ __forceinline__ void finish_tile(const USrc &src, int64_t tile, int64
             }
             return;
         }
-        const Grouping &G = q.grp;
-        for (int64_t gi = ref.g0;; ++gi) {
-            const int64_t gb = group_begin(G, gi, d), ge = group_end(G, gi, d);
-            const int64_t lo = max(gb, tile_lo), hi = min(ge, tile_hi);
-            double part;
-            if constexpr (QK == QK_SIGN) {
-                DF acc{0.0f, 0.0f};
-#pragma unroll
-                for (int k = 0; k < kSlots; ++k) {
-                    const int64_t j0 = 4 * slot_of(tile, k);
-                    float uk[4];
-                    src.get(k, uk);
-#pragma unroll
-                    for (int i = 0; i < 4; ++i)
-                        if (j0 + i >= lo && j0 + i < hi) df_accumulate(acc, fabsf(uk[i]));
-                }
-                part = block_sum(acc, sm.red, &sm.bcast);
-            } else {
-                float mx = 0.0f;
-#pragma unroll
-                for (int k = 0; k < kSlots; ++k) {
-                    const int64_t j0 = 4 * slot_of(tile, k);
-                    float uk[4];
-                    src.get(k, uk);
-#pragma unroll
-                    for (int i = 0; i < 4; ++i)
-                        if (j0 + i >= lo && j0 + i < hi) mx = fmaxf(mx, fabsf(uk[i]));
-                }
-                part = static_cast<double>(block_max(mx, sm.redm, &sm.bcastf));
-            }
-            if (threadIdx.x == 0) partials[sm.part + (gi - ref.g0)] = part;
-            if (ge >= tile_hi) break;
+        if constexpr (!one) {
+            int turn = 0;
+            group_partials<QK>(src, tile, tile_lo, tile_hi, d, q, ref, &sm.tg, partials, sm.parts, turn);
         }
     }
 }
@@ -455,15 +511,16 @@ __device__ __forceinline__ LazyScale lazy_scale_of_tile(const TileRef &ref, cons
     return ls;
 }
 
-// The residual of the kept u of coordinates j0 .. j0+3 (in place in e); coordinates >= d unchanged.
+// The residual of the kept u of coordinates j0 .. j0+3 (in place in e); coordinates >= d unchanged.  tg:
+// the tile's groups.
 template <bool FULL>
-__device__ __forceinline__ void lazy_residual4(const QParams &q, const float *scales, const LazyScale &ls, int64_t j0,
-                                               int64_t d, float (&e)[4])
+__device__ __forceinline__ void lazy_residual4(const QParams &q, const float *scales, const LazyScale &ls,
+                                               const TileGroups &tg, int64_t tile, int64_t j0, int64_t d, float (&e)[4])
 {
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         if (FULL || j0 + i < d) {
-            const float s = ls.g1 >= 0 ? ls.s1 : scales[group_of(q.grp, j0 + i, ls.hint)];
+            const float s = ls.g1 >= 0 ? ls.s1 : scales[tile_group_of(q.grp, tg, tile, j0 + i)];
             float dec;
             (void)encode1<QK_SIGN>(e[i], s, q, 0.0f, 0, 0.0f, dec);
             e[i] = __fsub_rn(e[i], dec);
@@ -471,10 +528,12 @@ __device__ __forceinline__ void lazy_residual4(const QParams &q, const float *sc
     }
 }
 
-// The same for all of this thread's slots of tile `tile`.  ONE: the tile lies inside one group.
+// The same for all of this thread's slots of tile `tile`.  ONE: the tile lies inside one group.  buf: the
+// threads' slots of shared memory, through which a tile of several groups goes one slot at a time.
 template <bool FULL, bool ONE>
-__device__ __forceinline__ void lazy_residual(const QParams &q, const float *scales, const LazyScale &ls, int64_t tile,
-                                              int64_t d, float (&e)[kSlots][4])
+__device__ __forceinline__ void lazy_residual(const QParams &q, const float *scales, const LazyScale &ls,
+                                              const TileGroups &tg, float4 *buf, int64_t tile, int64_t d,
+                                              float (&e)[kSlots][4])
 {
     if (ONE || ls.g1 >= 0) {  // one branch for the tile
 #pragma unroll
@@ -489,7 +548,16 @@ __device__ __forceinline__ void lazy_residual(const QParams &q, const float *sca
         return;
     }
 #pragma unroll
-    for (int k = 0; k < kSlots; ++k) lazy_residual4<FULL>(q, scales, ls, 4 * slot_of(tile, k), d, e[k]);
+    for (int k = 0; k < kSlots; ++k) buf[k * kThreads + threadIdx.x] = to_f4(e[k]);
+#pragma unroll 1
+    for (int k = 0; k < kSlots; ++k) {
+        float v[4];
+        to_arr(buf[k * kThreads + threadIdx.x], v);
+        lazy_residual4<FULL>(q, scales, ls, tg, tile, 4 * slot_of(tile, k), d, v);
+        buf[k * kThreads + threadIdx.x] = to_f4(v);
+    }
+#pragma unroll
+    for (int k = 0; k < kSlots; ++k) to_arr(buf[k * kThreads + threadIdx.x], e[k]);
 }
 
 }  // namespace ea

@@ -32,7 +32,7 @@ __device__ __forceinline__ void worker_tile(const WorkerArgs &a, int64_t tile, f
     build_qtab<QK>(a.q, sm.qtab);
     if constexpr (lazy) {
         // e holds the previous round's u: its residual is u - Q(u) with the previous scales
-        if (a.lazy_in) lazy_residual<FULL, PASS == PASS_LAZY_ONE>(a.q, a.scales, ls, tile, d, e);
+        if (a.lazy_in) lazy_residual<FULL, PASS == PASS_LAZY_ONE>(a.q, a.scales, ls, sm.tg, ubuf, tile, d, e);
     }
 #pragma unroll
     for (int k = 0; k < kSlots; ++k) {
@@ -72,16 +72,20 @@ __global__ void __launch_bounds__(kThreads, MODE == MODE_S ? 4 : 3)
     __shared__ TileSmem sm;
     __shared__ float4 ubuf[kSlots * kThreads];
     pdl_trigger();
-    const int64_t tile = blockIdx.x;
-    const TileRef ref = tile_ref(a.q.grp, tile, a.d);
-    if (threadIdx.x == 0) sm.part = ref.part();
-    pdl_wait();
-    if ((tile + 1) * kTile <= a.d) {
-        if (ref.ng() == 1) worker_tile<MODE, QK_SIGN, true, PASS_LAZY_ONE>(a, tile, ubuf, sm, ref);
-        else worker_tile<MODE, QK_SIGN, true, PASS_LAZY>(a, tile, ubuf, sm, ref);
-    } else {
-        worker_tile<MODE, QK_SIGN, false, PASS_LAZY>(a, tile, ubuf, sm, ref);
+    const CtaTile ct = cta_tile(a.q.grp, a.d);
+    if (ct.tile < 0) return;
+    if (threadIdx.x == 0) sm.part = ct.ref.part();
+    if (ct.plain) {
+        pdl_wait();
+        worker_tile<MODE, QK_SIGN, true, PASS_LAZY_ONE>(a, plain_tile(), ubuf, sm, ct.ref);
+        return;
     }
+    if (ct.ref.ng() > 1) {
+        cache_tile_groups(a.q.grp, ct.tile, a.d, sm.tg);
+        __syncthreads();
+    }
+    pdl_wait();
+    worker_tile<MODE, QK_SIGN, false, PASS_LAZY>(a, ct.tile, ubuf, sm, ct.ref);
 }
 
 template <int MODE, int QK>
@@ -91,11 +95,15 @@ __global__ void __launch_bounds__(kThreads, MODE == MODE_S ? 4 : 3)
     __shared__ TileSmem sm;
     __shared__ float4 ubuf[kSlots * kThreads];
     pdl_trigger();
-    const int64_t tile = blockIdx.x;
+    const int64_t tile = plain_tile();  // the ragged one first, see cta_tile
     TileRef ref{};
     if (has_scale<QK>() && a.pass == PASS_STASH) {
         ref = tile_ref(a.q.grp, tile, a.d);
         if (threadIdx.x == 0) sm.part = ref.part();
+        if (ref.ng() > 1) {
+            cache_tile_groups(a.q.grp, tile, a.d, sm.tg);
+            __syncthreads();
+        }
     }
     pdl_wait();
     // the scale pass as a compile-time constant: each instantiation carries only its own path
@@ -183,7 +191,7 @@ __global__ void __launch_bounds__(kThreads, MODE == MODE_S ? 4 : 2) worker_group
             const int64_t tl = static_cast<int64_t>(tile) * kTile, lo = max(c0, tl), hi = min(c1, tl + kTile);
             if (lo == tl && hi == tl + kTile) worker_u_range<MODE, true>(a, tile, lo, hi, ub);
             else worker_u_range<MODE, false>(a, tile, lo, hi, ub);
-            range_partials<QK>(ub, tile, lo, hi, a.d, a.q, a.partials, gs, turn);
+            group_partials<QK>(USmem{ub}, tile, lo, hi, a.d, a.q, tile_ref(a.q.grp, tile, a.d), nullptr, a.partials, gs.parts, turn);
         }
         if (!wave_barrier(gp, w, a.status, gs)) return;
         encode_wave<QK>(uslot, t0, t_end, c0, c1, a.d, a.q, a.words, a.partials, a.scales, a.e, a.ef, a.seed, a.id,
@@ -231,8 +239,8 @@ __global__ void __launch_bounds__(kThreads) finalize_kernel(const FinalizeArgs a
 }
 
 // Second pass, one CTA per tile: encode the stashed input with its group's scale and leave the
-// residual u - Q(u) in its place.  The tiles are taken last first: the first pass stored u without a
-// streaming hint among streams that have one, so the tiles it wrote last are still in L2, and what is
+// residual u - Q(u) in its place.  The first pass takes the tiles last first and this one first first:
+// u was stored without a streaming hint among streams that have one, so the tiles written last are still in L2, and what is
 // overwritten there was never written to memory.  TBD
 template <int QK, bool FULL>
 __device__ __forceinline__ void encode_one_group(const EncodeArgs &a, float s, int64_t tile, const float *qtab)
@@ -253,12 +261,14 @@ template <int QK>
 __global__ void __launch_bounds__(kThreads, 4) encode_kernel(const EncodeArgs a)
 {
     __shared__ float qtab_s[256];
+    __shared__ TileGroups tg;
     pdl_trigger();
     const float *qtab = build_qtab<QK>(a.q, qtab_s);
-    const int64_t tile = a.n_tiles - 1 - static_cast<int64_t>(blockIdx.x);
+    const int64_t tile = blockIdx.x;
     const int64_t d = a.d;
     const Grouping &G = a.q.grp;
     const TileRef ref = tile_ref(G, tile, d);
+    if (ref.ng() > 1) cache_tile_groups(G, tile, d, tg);
     __syncthreads();
     pdl_wait();
     // a tile inside one group (the common case) has one scale: the fused tile encode
@@ -270,7 +280,6 @@ __global__ void __launch_bounds__(kThreads, 4) encode_kernel(const EncodeArgs a)
     }
     const int L = (QK == QK_UNIF) ? unif_L(a.q.bits) : 0;
     const float Lf = static_cast<float>(L);
-    const int64_t hint = ref.g0;
 #pragma unroll 1
     for (int k = 0; k < kSlots; ++k) {
         const int64_t qs = slot_of(tile, k);
@@ -286,7 +295,7 @@ __global__ void __launch_bounds__(kThreads, 4) encode_kernel(const EncodeArgs a)
             float dec = 0.0f;
             c[i] = 0u;
             if (j0 + i < d) {
-                const float s = a.scales[group_of(G, j0 + i, hint)];
+                const float s = a.scales[tile_group_of(G, tg, tile, j0 + i)];
                 c[i] = encode1<QK>(u[i], s, a.q, Lf, L, U[i], dec, qtab);
             }
             e[i] = a.ef ? __fsub_rn(u[i], dec) : 0.0f;
@@ -306,7 +315,7 @@ __global__ void __launch_bounds__(kThreads, 4) encode_kernel(const EncodeArgs a)
 // AS_ANY: a group lookup.
 enum ApplyScales : int { AS_TILE, AS_SLOT, AS_ANY };
 template <int QK, bool FULL, int BITS, int SCALES>
-__device__ __forceinline__ void apply_tile(const ApplyArgs &a, int64_t tile, const TileRef &ref, float *qtab_s)
+__device__ __forceinline__ void apply_tile(const ApplyArgs &a, int64_t tile, const TileRef &ref, const TileGroups &tg, float *qtab_s)
 {
     const int64_t d = a.d;
     const Grouping &G = a.q.grp;
@@ -339,10 +348,9 @@ __device__ __forceinline__ void apply_tile(const ApplyArgs &a, int64_t tile, con
         __syncthreads();
     }
     // one scale for the whole tile: 4096-blocks, or a tile inside one group
-    const int64_t g1 = (!has_scale<QK>() || SCALES == AS_SLOT) ? 0 : SCALES == AS_TILE ? tile : ref.ng() == 1 ? ref.g0 : -1;
-    const bool tile_scale = SCALES != AS_ANY || g1 >= 0;
+    const int64_t g1 = (!has_scale<QK>() || SCALES == AS_SLOT) ? 0 : SCALES == AS_TILE ? tile : FULL || ref.ng() == 1 ? ref.g0 : -1;
+    const bool tile_scale = SCALES != AS_ANY || FULL || g1 >= 0;
     const float s_tile = (has_scale<QK>() && SCALES != AS_SLOT && tile_scale) ? __ldg(a.scales + g1) : 0.0f;
-    const int64_t hint = SCALES == AS_ANY ? ref.g0 : 0;
 #pragma unroll
     for (int k = 0; k < kSlots; ++k) {
         const int64_t q = slot_of(tile, k);
@@ -362,7 +370,7 @@ __device__ __forceinline__ void apply_tile(const ApplyArgs &a, int64_t tile, con
         for (int i = 0; i < 4; ++i) {
             if (FULL || j0 + i < d) {
                 float s = SCALES == AS_SLOT ? s_slot[k] : s_tile;
-                if (has_scale<QK>() && !tile_scale) s = __ldg(a.scales + group_of(G, j0 + i, hint));
+                if (has_scale<QK>() && !tile_scale) s = __ldg(a.scales + tile_group_of(G, tg, tile, j0 + i));
                 x[k][i] = __fsub_rn(x[k][i], decode1<QK>(c[i], s, a.q, Lf, L, qtab));
             }
         }
@@ -370,21 +378,18 @@ __device__ __forceinline__ void apply_tile(const ApplyArgs &a, int64_t tile, con
     }
 }
 
+// AS_TILE and AS_SLOT take any whole tile, AS_ANY one inside one group; the rest is the general form.
 template <int QK, int BITS>
-__device__ __forceinline__ void apply_body(const ApplyArgs &a, const TileRef &ref, float *qtab_s)
+__device__ __forceinline__ void apply_body(const ApplyArgs &a, const CtaTile &ct, const TileGroups &tg, float *qtab_s)
 {
-    const int64_t tile = blockIdx.x;
-    const bool full = (tile + 1) * kTile <= a.d;
-    if (a.q.grp.gkind == GK_BLOCK && a.q.grp.G == kTile) {
-        if (full) apply_tile<QK, true, BITS, AS_TILE>(a, tile, ref, qtab_s);
-        else apply_tile<QK, false, BITS, AS_TILE>(a, tile, ref, qtab_s);
-    } else if (has_scale<QK>() && a.q.grp.gkind == GK_BLOCK && a.q.grp.log2G >= kLog2Chunk) {
-        if (full) apply_tile<QK, true, BITS, AS_SLOT>(a, tile, ref, qtab_s);
-        else apply_tile<QK, false, BITS, AS_SLOT>(a, tile, ref, qtab_s);
-    } else {
-        if (full) apply_tile<QK, true, BITS, AS_ANY>(a, tile, ref, qtab_s);
-        else apply_tile<QK, false, BITS, AS_ANY>(a, tile, ref, qtab_s);
-    }
+    if ((ct.tile + 1) * kTile <= a.d && a.q.grp.gkind == GK_BLOCK && a.q.grp.G == kTile)
+        apply_tile<QK, true, BITS, AS_TILE>(a, plain_tile(), ct.ref, tg, qtab_s);
+    else if (has_scale<QK>() && (ct.tile + 1) * kTile <= a.d && a.q.grp.gkind == GK_BLOCK && a.q.grp.log2G >= kLog2Chunk)
+        apply_tile<QK, true, BITS, AS_SLOT>(a, plain_tile(), ct.ref, tg, qtab_s);
+    else if (ct.plain)
+        apply_tile<QK, true, BITS, AS_ANY>(a, plain_tile(), ct.ref, tg, qtab_s);
+    else
+        apply_tile<QK, false, BITS, AS_ANY>(a, ct.tile, ct.ref, tg, qtab_s);
 }
 
 // One CTA per 4096-tile; the code width is dispatched once per CTA.
@@ -393,21 +398,27 @@ __global__ void __launch_bounds__(kThreads) apply_kernel(const ApplyArgs a)
 {
     __shared__ float qtab_s[256];
     pdl_trigger();
-    TileRef ref{};
-    if (has_scale<QK>()) ref = tile_ref(a.q.grp, blockIdx.x, a.d);
+    __shared__ TileGroups tg;
+    const CtaTile ct = cta_tile(a.q.grp, a.d);
+    if (ct.tile < 0) return;
+    const bool per_slot = a.q.grp.gkind == GK_BLOCK && a.q.grp.log2G >= kLog2Chunk && (ct.tile + 1) * kTile <= a.d;
+    if (has_scale<QK>() && !per_slot && ct.ref.ng() > 1) {
+        cache_tile_groups(a.q.grp, ct.tile, a.d, tg);
+        __syncthreads();
+    }
     pdl_wait();
     if constexpr (QK == QK_UNIF) {
         switch (a.q.bits) {  // the widths ea_init accepts
-        case 2: apply_body<QK, 2>(a, ref, qtab_s); break;
-        case 4: apply_body<QK, 4>(a, ref, qtab_s); break;
-        case 8: apply_body<QK, 8>(a, ref, qtab_s); break;
-        default: apply_body<QK, 16>(a, ref, qtab_s); break;
+        case 2: apply_body<QK, 2>(a, ct, tg, qtab_s); break;
+        case 4: apply_body<QK, 4>(a, ct, tg, qtab_s); break;
+        case 8: apply_body<QK, 8>(a, ct, tg, qtab_s); break;
+        default: apply_body<QK, 16>(a, ct, tg, qtab_s); break;
         }
     } else if constexpr (QK == QK_POW2) {
-        if (a.q.bits == 4) apply_body<QK, 4>(a, ref, qtab_s);
-        else apply_body<QK, 8>(a, ref, qtab_s);
+        if (a.q.bits == 4) apply_body<QK, 4>(a, ct, tg, qtab_s);
+        else apply_body<QK, 8>(a, ct, tg, qtab_s);
     } else {
-        apply_body<QK, QK == QK_SIGN ? 1 : 32>(a, ref, qtab_s);
+        apply_body<QK, QK == QK_SIGN ? 1 : 32>(a, ct, tg, qtab_s);
     }
 }
 
@@ -423,7 +434,7 @@ __global__ void fill_kernel(float *p, int64_t count, float value)
 template <int MODE>
 static cudaError_t launch_worker_mode(const WorkerArgs &a, cudaStream_t s, bool overlap)
 {
-    const dim3 grid(static_cast<unsigned>(a.n_tiles)), block(kThreads);
+    const dim3 grid(static_cast<unsigned>(a.n_tiles + (a.pass == PASS_LAZY ? a.q.grp.n_slow : 0))), block(kThreads);
     if (a.pass == PASS_LAZY)
         return a.q.kind == QK_SIGN ? launch_pdl(worker_lazy_kernel<MODE>, grid, block, 0, s, overlap, kCarveoutPercent, a) : cudaErrorNotSupported;
     switch (a.q.kind) {
@@ -474,17 +485,21 @@ cudaError_t launch_encode(const EncodeArgs &a, cudaStream_t s, bool overlap)
 // The residual u - Q(u) of the u kept by PASS_LAZY, into a.out, one CTA per tile (a view of it).
 __global__ void __launch_bounds__(kThreads) lazy_resid_kernel(const ResidArgs a)
 {
+    __shared__ TileGroups tg;
+    __shared__ float4 buf[kSlots * kThreads];
     pdl_trigger();
     const int64_t tile = blockIdx.x;
     const TileRef ref = tile_ref(a.q.grp, tile, a.d);
+    if (ref.ng() > 1) cache_tile_groups(a.q.grp, tile, a.d, tg);
+    __syncthreads();
     pdl_wait();
     const bool full = (tile + 1) * kTile <= a.d;
     const LazyScale ls = lazy_scale_of_tile(ref, a.scales);
     float u[kSlots][4];
 #pragma unroll
     for (int k = 0; k < kSlots; ++k) load4(a.u, slot_of(tile, k), a.d, u[k]);
-    if (full) lazy_residual<true, false>(a.q, a.scales, ls, tile, a.d, u);
-    else lazy_residual<false, false>(a.q, a.scales, ls, tile, a.d, u);
+    if (full) lazy_residual<true, false>(a.q, a.scales, ls, tg, buf, tile, a.d, u);
+    else lazy_residual<false, false>(a.q, a.scales, ls, tg, buf, tile, a.d, u);
 #pragma unroll
     for (int k = 0; k < kSlots; ++k)
         if (4 * slot_of(tile, k) < a.d) store4(a.out, slot_of(tile, k), a.d, u[k]);
@@ -499,7 +514,7 @@ cudaError_t launch_lazy_resid(const ResidArgs &a, cudaStream_t s, bool overlap)
 
 cudaError_t launch_apply(const ApplyArgs &a, cudaStream_t s, bool overlap)
 {
-    const dim3 grid(static_cast<unsigned>((a.d + kTile - 1) / kTile)), block(kThreads);
+    const dim3 grid(static_cast<unsigned>((a.d + kTile - 1) / kTile + a.q.grp.n_slow)), block(kThreads);
     switch (a.q.kind) {
     case QK_SIGN: return launch_pdl(apply_kernel<QK_SIGN>, grid, block, 0, s, overlap, kCarveoutPercent, a);
     case QK_UNIF: return launch_pdl(apply_kernel<QK_UNIF>, grid, block, 0, s, overlap, kCarveoutPercent, a);
