@@ -116,6 +116,12 @@ int ea_server_step(ea_handle *h);
  * EA_E_ORDER before the first ea_server_step. */
 int ea_worker_apply(ea_handle *h, float *x);
 
+/* A whole round: ea_worker_compress of worker i with gs[i] for every i in order, ea_server_step and
+ * ea_worker_apply(x), with the same results, checks and errors (the calls before one that is refused have
+ * been made).  gs: n addresses in host memory, read before this returns.  Messages that take one launch
+ * share launches, up to 32 workers each. */
+int ea_round_step(ea_handle *h, const float *const *gs, float *x);
+
 /* alpha_t, beta and theta_t (= beta2) for the calls that follow, e.g. between rounds: Assumption 2
  * sets theta_t = 1 - theta/T and alpha_t = alpha/sqrt(T) from the horizon T; the experiments decay
  * alpha in steps.  Same ranges as ea_config; EA_E_INVAL otherwise (nothing changed). */
@@ -129,8 +135,8 @@ int ea_bits_sent(const ea_handle *h, uint64_t *up_bits, uint64_t *down_bits);
 /* Rounds completed (ea_server_step calls). */
 int ea_round_index(const ea_handle *h, int64_t *t);
 
-/* Kernel launches that one round makes on the stream: n worker compresses, one server step and one
- * apply.  A message whose scale groups lie inside 4096-coordinate tiles takes one launch.  When the
+/* Kernel launches that one round of separate calls makes on the stream: n worker compresses, one server
+ * step and one apply (ea_round_step makes fewer).  A message whose scale groups lie inside 4096-coordinate tiles takes one launch.  When the
  * groups span tiles:
  *   - a scaled-sign message takes one pass, which writes the codes (the signs, which need no scale)
  *     with the groups' partial norms, and a finalize forms the scales: one finalize for all worker

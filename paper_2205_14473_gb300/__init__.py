@@ -16,6 +16,7 @@ from __future__ import annotations
 
 import ctypes
 import dataclasses
+import itertools
 import os
 import threading
 
@@ -29,7 +30,7 @@ EA_E_CUDA, EA_E_TIMEOUT, EA_E_DEVICE_CHECK, EA_E_UNSUPPORTED = -5, -6, -7, -8
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "_lib", "libea.so")
-EXPORTED = ["ea_workspace_bytes", "ea_init", "ea_worker_compress", "ea_server_step", "ea_worker_apply",
+EXPORTED = ["ea_workspace_bytes", "ea_init", "ea_worker_compress", "ea_server_step", "ea_worker_apply", "ea_round_step",
             "ea_bits_sent", "ea_round_index", "ea_round_launches", "ea_get_view", "ea_sync_status", "ea_last_error", "ea_destroy",
             "ea_worker_compress_noalloc", "ea_set_hparams", "ea_selftest_bounded_wait"]
 
@@ -72,6 +73,7 @@ def lib() -> ctypes.CDLL:
             L.ea_worker_compress.argtypes = [_P, ctypes.c_int32, _P]
             L.ea_server_step.argtypes = [_P]
             L.ea_worker_apply.argtypes = [_P, _P]
+            L.ea_round_step.argtypes = [_P, _P, _P]
             L.ea_bits_sent.argtypes = [_P, ctypes.POINTER(ctypes.c_uint64), ctypes.POINTER(ctypes.c_uint64)]
             L.ea_round_index.argtypes = [_P, ctypes.POINTER(ctypes.c_int64)]
             L.ea_round_launches.argtypes = [_P, ctypes.POINTER(ctypes.c_int32)]
@@ -117,6 +119,12 @@ def ea_server_step(h: int) -> None:
 
 def ea_worker_apply(h: int, x_ptr: int) -> None:
     _check(lib().ea_worker_apply(h, x_ptr), h)
+
+
+def ea_round_step(h: int, g_ptrs, x_ptr: int) -> None:
+    """ea_worker_compress for every worker, ea_server_step and ea_worker_apply in one call; g_ptrs is a
+    ctypes array of the n gradients' addresses."""
+    _check(lib().ea_round_step(h, g_ptrs, x_ptr), h)
 
 
 def ea_set_hparams(h: int, alpha: float, beta1: float, beta2: float) -> None:
@@ -249,7 +257,13 @@ class EARound:
 
     def step(self, grads, x) -> None:
         """One full round: every worker compresses its gradient, the server broadcasts, x moves."""
-        for i in range(self.cfg.n):
+        n, d = self.cfg.n, self.cfg.d
+        if len(grads) >= n and x.is_contiguous() and x.numel() >= d and all(
+                g.dtype.is_floating_point and g.is_contiguous() and g.numel() >= d for g in itertools.islice(grads, n)):
+            ptrs = (_P * n)(*[grads[i].data_ptr() for i in range(n)])
+            ea_round_step(self.h, ptrs, x.data_ptr())
+            return
+        for i in range(n):  # what is not accepted fails where its own call does
             self.worker_compress(i, grads[i])
         self.server_step()
         self.apply(x)

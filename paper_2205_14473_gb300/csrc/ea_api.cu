@@ -558,6 +558,71 @@ int second_pass(ea_handle *h, const QHost &q, const double *partials, float *buf
     return check_cuda(h, launch_encode(e, h->stream, may_overlap(h)), "encode launch");
 }
 
+int check_compress(ea_handle *h, int32_t worker, const float *g)
+{
+    if (worker < 0 || worker >= h->cfg.n) return fail(h, EA_E_INVAL, "worker %d out of [0, %d)", worker, h->cfg.n);
+    const int r = check_dev_ptr(h, g, "g");
+    if (r != EA_OK) return r;
+    if (h->compressed[worker])
+        return fail(h, EA_E_ORDER, "worker %d already compressed in round %lld", worker, static_cast<long long>(h->t));
+    return EA_OK;
+}
+
+// The messages of workers first .. first + count - 1, from gs[0 .. count - 1] (checked by the caller).
+// Where a message is one launch, up to kWorkerBatch of them share it; the messages whose scale
+// needs further launches go one after another (they share the partial norms).
+int compress_workers(ea_handle *h, int32_t first, const float *const *gs, int32_t count)
+{
+    const bool lazy = h->qw.pass == PASS_LAZY, W = h->cfg.placement == EA_ADAM_AT_WORKER;
+    const bool together = h->qw.pass != PASS_STASH && h->qw.pass != PASS_GROUPED;
+    const int64_t dp = h->lay.dpad;
+    WorkerArgs a{};
+    a.d = h->cfg.d;
+    a.n_tiles = h->n_tiles;
+    a.q = device_quant(h->qw);
+    a.hp = round_hyper(h);
+    a.ef = h->cfg.error_feedback;
+    a.pass = h->qw.pass;
+    a.seed = h->cfg.seed;
+    a.t = static_cast<uint32_t>(h->t);
+    a.status = h->status;
+    for (int32_t at = 0; at < count;) {
+        const int32_t w = first + at;
+        a.lazy_in = lazy ? h->lazy_w[w] : 0;
+        a.count = 1;
+        while (together && a.count < kWorkerBatch && at + a.count < count && (!lazy || h->lazy_w[w + a.count] == a.lazy_in))
+            ++a.count;
+        for (int i = 0; i < a.count; ++i) {
+            const int64_t k = w + i;
+            a.w[i] = WorkerBufs{gs[at + i], W ? h->m + k * dp : nullptr, W ? h->v + k * dp : nullptr, h->e + k * dp,
+                                h->wcodes + k * h->lay.wcode_stride, h->wscales + k * h->lay.wscale_stride,
+                                h->partials + (lazy ? k * h->qw.n_pairs : 0)};
+        }
+        a.id = static_cast<uint32_t>(w);
+        int r;
+        if (h->qw.pass == PASS_GROUPED) {
+            a.gp = device_group_plan(h->qw, h->epoch_w);
+            r = check_cuda(h, launch_worker_grouped(W ? MODE_W : MODE_S, a, h->qw.grid, h->stream), "worker launch");
+            if (r == EA_OK) ++h->epoch_w;
+            h->split_full = true;
+        } else {
+            r = check_cuda(h, launch_worker(W ? MODE_W : MODE_S, a, h->stream, may_overlap(h)), "worker launch");
+        }
+        if (r == EA_OK && h->qw.pass == PASS_STASH) r = second_pass(h, h->qw, a.w[0].partials, a.w[0].e, a.w[0].words, a.w[0].scales, a.id);
+        if (r != EA_OK) return r;
+        for (int i = 0; i < a.count; ++i) {
+            if (lazy) {  // the scales are formed for all workers before the server step
+                h->lazy_w[w + i] = h->cfg.error_feedback ? 1 : 0;
+                h->wscales_pending = true;
+            }
+            h->compressed[w + i] = 1;
+            ++h->n_compressed;
+        }
+        at += a.count;
+    }
+    return EA_OK;
+}
+
 }  // namespace
 
 void ea::set_last_error(const char *msg) { g_last_error = msg; }
@@ -737,49 +802,27 @@ int ea_init(const ea_config *cfg, void *workspace, size_t workspace_bytes, void 
 int ea_worker_compress(ea_handle *h, int32_t worker, const float *g)
 {
     if (!h) return fail(nullptr, EA_E_INVAL, "handle is NULL");
-    if (worker < 0 || worker >= h->cfg.n) return fail(h, EA_E_INVAL, "worker %d out of [0, %d)", worker, h->cfg.n);
-    int r = check_dev_ptr(h, g, "g");
-    if (r != EA_OK) return r;
-    if (h->compressed[worker])
-        return fail(h, EA_E_ORDER, "worker %d already compressed in round %lld", worker, static_cast<long long>(h->t));
-    const int64_t dp = h->lay.dpad;
-    WorkerArgs a{};
-    a.d = h->cfg.d;
-    a.n_tiles = h->n_tiles;
-    a.g = g;
-    const bool W = h->cfg.placement == EA_ADAM_AT_WORKER;
-    a.m = W ? h->m + worker * dp : nullptr;
-    a.v = W ? h->v + worker * dp : nullptr;
-    a.e = h->e + worker * dp;
-    a.q = device_quant(h->qw);
-    a.words = h->wcodes + worker * h->lay.wcode_stride;
-    a.scales = h->wscales + worker * h->lay.wscale_stride;
-    a.hp = round_hyper(h);
-    a.ef = h->cfg.error_feedback;
-    a.pass = h->qw.pass;
-    a.seed = h->cfg.seed;
-    a.id = static_cast<uint32_t>(worker);
-    a.t = static_cast<uint32_t>(h->t);
-    a.partials = h->qw.pass == PASS_LAZY ? h->partials + static_cast<int64_t>(worker) * h->qw.n_pairs : h->partials;
-    a.status = h->status;
-    a.lazy_in = h->qw.pass == PASS_LAZY ? h->lazy_w[worker] : 0;
-    if (h->qw.pass == PASS_GROUPED) {
-        a.gp = device_group_plan(h->qw, h->epoch_w);
-        r = check_cuda(h, launch_worker_grouped(W ? MODE_W : MODE_S, a, h->qw.grid, h->stream), "worker launch");
-        if (r == EA_OK) ++h->epoch_w;
-        h->split_full = true;
-    } else {
-        r = check_cuda(h, launch_worker(W ? MODE_W : MODE_S, a, h->stream, may_overlap(h)), "worker launch");
+    const int r = check_compress(h, worker, g);
+    return r == EA_OK ? compress_workers(h, worker, &g, 1) : r;
+}
+
+int ea_round_step(ea_handle *h, const float *const *gs, float *x)
+{
+    if (!h) return fail(nullptr, EA_E_INVAL, "handle is NULL");
+    if (!gs) return fail(h, EA_E_INVAL, "gradients is NULL");
+    // the workers before one that is refused are compressed, as by one call each
+    int r = EA_OK;
+    int32_t good = 0;
+    while (good < h->cfg.n && (r = check_compress(h, good, gs[good])) == EA_OK) ++good;
+    const std::string why = h->err;
+    const int rc = compress_workers(h, 0, gs, good);
+    if (rc != EA_OK) return rc;
+    if (r != EA_OK) {
+        h->err = why;
+        return r;
     }
-    if (r == EA_OK && h->qw.pass == PASS_STASH) r = second_pass(h, h->qw, a.partials, a.e, a.words, a.scales, a.id);
-    if (r != EA_OK) return r;
-    if (h->qw.pass == PASS_LAZY) {  // the scales are formed for all workers before the server step
-        h->lazy_w[worker] = h->cfg.error_feedback ? 1 : 0;
-        h->wscales_pending = true;
-    }
-    h->compressed[worker] = 1;
-    ++h->n_compressed;
-    return EA_OK;
+    r = ea_server_step(h);
+    return r == EA_OK ? ea_worker_apply(h, x) : r;
 }
 
 int ea_server_step(ea_handle *h)

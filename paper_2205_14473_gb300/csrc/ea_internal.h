@@ -132,18 +132,27 @@ struct GroupedShape {
     int ctas_per_sm, slots;
 };
 
-struct WorkerArgs {
-    int64_t d, n_tiles;
+// Workers whose messages one launch may compress (blockIdx.y).  Their buffers' addresses travel in the
+// launch parameters (56 bytes each of the 4 KB), where a thread reads them when it needs them.
+constexpr int kWorkerBatch = 32;
+
+struct WorkerBufs {
     const float *g;
     float *m, *v, *e;
-    QParams q;
     uint32_t *words;
     float *scales;
+    double *partials;
+};
+
+struct WorkerArgs {
+    int64_t d, n_tiles;
+    int count;                  // workers of this launch
+    WorkerBufs w[kWorkerBatch];
+    QParams q;
     Hyper hp;
     int ef, pass;
     uint64_t seed;
-    uint32_t id, t;
-    double *partials;
+    uint32_t id, t;           // the first worker's id
     GroupPlan gp;             // PASS_GROUPED
     uint32_t *status;         // device status word (timeouts); may be null outside a handle
     int lazy_in;              // PASS_LAZY: e holds the previous round's u, scales its scales

@@ -113,13 +113,9 @@ extern "C" int ea_worker_compress_noalloc(const ea_config *cfg, int32_t worker, 
     WorkerArgs a{};
     a.d = d;
     a.n_tiles = n_tiles;
-    a.g = g;
-    a.m = W ? m : nullptr;
-    a.v = W ? v : nullptr;
-    a.e = e;
+    a.count = 1;
+    a.w[0] = WorkerBufs{g, W ? m : nullptr, W ? v : nullptr, e, codes, scales, partials};
     a.q = qp;
-    a.words = codes;
-    a.scales = scales;
     a.hp.alpha = cfg->alpha;
     a.hp.beta1 = cfg->beta1;
     a.hp.beta2 = cfg->beta2;
@@ -136,7 +132,6 @@ extern "C" int ea_worker_compress_noalloc(const ea_config *cfg, int32_t worker, 
     a.seed = cfg->seed;
     a.id = static_cast<uint32_t>(worker);
     a.t = static_cast<uint32_t>(round);
-    a.partials = partials;
 
     cudaError_t ce = cudaSuccess;
     if (a.pass == PASS_STASH) {

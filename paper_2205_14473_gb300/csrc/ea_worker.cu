@@ -8,31 +8,34 @@ namespace ea {
 // the scale's reduction and more CTAs fit on an SM.
 // ref: the tile's groups (PASS_STASH, PASS_LAZY), looked up by the caller.
 template <int MODE, int QK, bool FULL, int PASS>
-__device__ __forceinline__ void worker_tile(const WorkerArgs &a, int64_t tile, float4 *ubuf, TileSmem &sm,
+__device__ __forceinline__ void worker_tile(const WorkerArgs &a, const WorkerBufs &p, int64_t tile, float4 *ubuf, TileSmem &sm,
                                             const TileRef &ref)
 {
     const int64_t d = a.d;
+    constexpr bool lazy = PASS == PASS_LAZY || PASS == PASS_LAZY_ONE;
+    LazyScale ls{};
+    if constexpr (lazy)
+        if (a.lazy_in) {
+            if constexpr (PASS == PASS_LAZY_ONE) ls.s1 = p.scales[ref.g0];
+            else ls = lazy_scale_of_tile(ref, p.scales);
+        }
     float g[kSlots][4], e[kSlots][4], m[kSlots][4], v[kSlots][4];
 #pragma unroll
     for (int k = 0; k < kSlots; ++k) {
         const int64_t q = slot_of(tile, k);
-        load4<FULL>(a.g, q, d, g[k]);
-        load4<FULL>(a.e, q, d, e[k]);
+        load4<FULL>(p.g, q, d, g[k]);
+        load4<FULL>(p.e, q, d, e[k]);
         if (MODE == MODE_W) {
-            load4<FULL>(a.m, q, d, m[k]);
-            load4<FULL>(a.v, q, d, v[k]);
+            load4<FULL>(p.m, q, d, m[k]);
+            load4<FULL>(p.v, q, d, v[k]);
         }
     }
-    constexpr bool lazy = PASS == PASS_LAZY || PASS == PASS_LAZY_ONE;
-    LazyScale ls{};
-    if constexpr (lazy)
-        if (a.lazy_in) ls = lazy_scale_of_tile(ref, a.scales);
     // the grid's fl(i/L) table, built while the loads are in flight (read after the scale
     // reduction's barrier)
     build_qtab<QK>(a.q, sm.qtab);
     if constexpr (lazy) {
         // e holds the previous round's u: its residual is u - Q(u) with the previous scales
-        if (a.lazy_in) lazy_residual<FULL, PASS == PASS_LAZY_ONE>(a.q, a.scales, ls, sm.tg, ubuf, tile, d, e);
+        if (a.lazy_in) lazy_residual<FULL, PASS == PASS_LAZY_ONE>(a.q, p.scales, ls, sm.tg, ubuf, tile, d, e);
     }
 #pragma unroll
     for (int k = 0; k < kSlots; ++k) {
@@ -47,12 +50,12 @@ __device__ __forceinline__ void worker_tile(const WorkerArgs &a, int64_t tile, f
         }
         ubuf[k * kThreads + threadIdx.x] = make_float4(u[0], u[1], u[2], u[3]);
         if (MODE == MODE_W && (FULL || j0 < d)) {
-            store4<FULL>(a.m, q, d, m[k]);
-            store4<FULL>(a.v, q, d, v[k]);
+            store4<FULL>(p.m, q, d, m[k]);
+            store4<FULL>(p.v, q, d, v[k]);
         }
     }
-    finish_tile<QK, FULL, true, PASS>(USmem{ubuf}, tile, d, a.q, a.words, a.scales, a.e, a.ef, a.pass, a.seed, a.id, a.t,
-                                      a.partials, sm, ref);
+    finish_tile<QK, FULL, true, PASS>(USmem{ubuf}, tile, d, a.q, p.words, p.scales, p.e, a.ef, a.pass, a.seed, (a.id + blockIdx.y), a.t,
+                                      p.partials, sm, ref);
 }
 
 // Algorithm 2 for one worker on one 4096-coordinate tile.  With Adam at the worker:
@@ -63,21 +66,25 @@ __device__ __forceinline__ void worker_tile(const WorkerArgs &a, int64_t tile, f
 // coordinate), three with Adam at the worker.  Measured: the server-side-Adam uniform grid runs
 // faster at four CTAs with a few bytes of spill than at three without, and the worker-side-Adam
 // uniform grid faster at three (80 registers, a few bytes of spill) than at two.
+// One CTA per tile and worker (blockIdx.y), a worker's tiles next to each other: the workers of one
+// launch leave no idle SMs between them, where a launch each drains the chip n times and a small
+// vector fills a part of it.  TBD
 // PASS_LAZY for the scaled sign: the same tile, the codes stored with the partial norms and u kept
 // in e (see lazy_residual); one launch per message plus finalize_kernel.
 template <int MODE>
 __global__ void __launch_bounds__(kThreads, MODE == MODE_S ? 4 : 3)
-    worker_lazy_kernel(const WorkerArgs a)
+    worker_lazy_kernel(const __grid_constant__ WorkerArgs a)
 {
     __shared__ TileSmem sm;
     __shared__ float4 ubuf[kSlots * kThreads];
     pdl_trigger();
+    const WorkerBufs &p = a.w[blockIdx.y];
     const CtaTile ct = cta_tile(a.q.grp, a.d);
     if (ct.tile < 0) return;
     if (threadIdx.x == 0) sm.part = ct.ref.part();
     if (ct.plain) {
         pdl_wait();
-        worker_tile<MODE, QK_SIGN, true, PASS_LAZY_ONE>(a, plain_tile(), ubuf, sm, ct.ref);
+        worker_tile<MODE, QK_SIGN, true, PASS_LAZY_ONE>(a, p, plain_tile(), ubuf, sm, ct.ref);
         return;
     }
     if (ct.ref.ng() > 1) {
@@ -85,16 +92,17 @@ __global__ void __launch_bounds__(kThreads, MODE == MODE_S ? 4 : 3)
         __syncthreads();
     }
     pdl_wait();
-    worker_tile<MODE, QK_SIGN, false, PASS_LAZY>(a, ct.tile, ubuf, sm, ct.ref);
+    worker_tile<MODE, QK_SIGN, false, PASS_LAZY>(a, p, ct.tile, ubuf, sm, ct.ref);
 }
 
 template <int MODE, int QK>
 __global__ void __launch_bounds__(kThreads, MODE == MODE_S ? 4 : 3)
-    worker_kernel(const WorkerArgs a)
+    worker_kernel(const __grid_constant__ WorkerArgs a)
 {
     __shared__ TileSmem sm;
     __shared__ float4 ubuf[kSlots * kThreads];
     pdl_trigger();
+    const WorkerBufs &p = a.w[blockIdx.y];
     const int64_t tile = plain_tile();  // the ragged one first, see cta_tile
     TileRef ref{};
     if (has_scale<QK>() && a.pass == PASS_STASH) {
@@ -109,14 +117,14 @@ __global__ void __launch_bounds__(kThreads, MODE == MODE_S ? 4 : 3)
     // the scale pass as a compile-time constant: each instantiation carries only its own path
     const bool full = (tile + 1) * kTile <= a.d;
     if (a.pass == PASS_FUSED) {
-        if (full) worker_tile<MODE, QK, true, PASS_FUSED>(a, tile, ubuf, sm, ref);
-        else worker_tile<MODE, QK, false, PASS_FUSED>(a, tile, ubuf, sm, ref);
+        if (full) worker_tile<MODE, QK, true, PASS_FUSED>(a, p, tile, ubuf, sm, ref);
+        else worker_tile<MODE, QK, false, PASS_FUSED>(a, p, tile, ubuf, sm, ref);
     } else if (has_scale<QK>() && a.pass == PASS_SHORT) {
-        if (full) worker_tile<MODE, QK, true, PASS_SHORT>(a, tile, ubuf, sm, ref);
-        else worker_tile<MODE, QK, false, PASS_SHORT>(a, tile, ubuf, sm, ref);
+        if (full) worker_tile<MODE, QK, true, PASS_SHORT>(a, p, tile, ubuf, sm, ref);
+        else worker_tile<MODE, QK, false, PASS_SHORT>(a, p, tile, ubuf, sm, ref);
     } else {
-        if (full) worker_tile<MODE, QK, true, PASS_STASH>(a, tile, ubuf, sm, ref);
-        else worker_tile<MODE, QK, false, PASS_STASH>(a, tile, ubuf, sm, ref);
+        if (full) worker_tile<MODE, QK, true, PASS_STASH>(a, p, tile, ubuf, sm, ref);
+        else worker_tile<MODE, QK, false, PASS_STASH>(a, p, tile, ubuf, sm, ref);
     }
 }
 
@@ -125,7 +133,7 @@ __global__ void __launch_bounds__(kThreads, MODE == MODE_S ? 4 : 3)
 // FULL: the range is the whole tile.  All four slots' loads are issued at once (the kernel's
 // register budget is sized for it), so that enough bytes are in flight per SM.
 template <int MODE, bool FULL>
-__device__ __forceinline__ void worker_u_range(const WorkerArgs &a, int64_t tile, int64_t lo, int64_t hi, float4 *ub)
+__device__ __forceinline__ void worker_u_range(const WorkerArgs &a, const WorkerBufs &p, int64_t tile, int64_t lo, int64_t hi, float4 *ub)
 {
     constexpr int H = kSlots;
 #pragma unroll
@@ -139,11 +147,11 @@ __device__ __forceinline__ void worker_u_range(const WorkerArgs &a, int64_t tile
 #pragma unroll
             for (int i = 0; i < 4; ++i) g[k][i] = e[k][i] = m[k][i] = 0.0f, v[k][i] = 1.0f;
             if (in[k]) {
-                load4<FULL>(a.g, q, hi, g[k]);
-                load4<FULL>(a.e, q, hi, e[k]);
+                load4<FULL>(p.g, q, hi, g[k]);
+                load4<FULL>(p.e, q, hi, e[k]);
                 if (MODE == MODE_W) {
-                    load4<FULL>(a.m, q, hi, m[k]);
-                    load4<FULL>(a.v, q, hi, v[k]);
+                    load4<FULL>(p.m, q, hi, m[k]);
+                    load4<FULL>(p.v, q, hi, v[k]);
                 }
             }
         }
@@ -160,8 +168,8 @@ __device__ __forceinline__ void worker_u_range(const WorkerArgs &a, int64_t tile
             }
             ub[(h + k) * kThreads + threadIdx.x] = make_float4(u[0], u[1], u[2], u[3]);
             if (MODE == MODE_W && in[k]) {
-                store4<FULL>(a.m, q, hi, m[k]);
-                store4<FULL>(a.v, q, hi, v[k]);
+                store4<FULL>(p.m, q, hi, m[k]);
+                store4<FULL>(p.v, q, hi, v[k]);
             }
         }
     }
@@ -180,6 +188,7 @@ __global__ void __launch_bounds__(kThreads, MODE == MODE_S ? 4 : 2) worker_group
     build_qtab<QK>(a.q, gs.qtab);
     __syncthreads();
     const GroupPlan &gp = a.gp;
+    const WorkerBufs &p = a.w[0];
     int turn = 0;  // reductions so far (the same count in every thread)
     for (int w = 0; w < static_cast<int>(gp.n_waves); ++w) {
         const int64_t c0 = gp.cuts[w], c1 = gp.cuts[w + 1];
@@ -189,12 +198,12 @@ __global__ void __launch_bounds__(kThreads, MODE == MODE_S ? 4 : 2) worker_group
         for (int tile = t0; tile < t_end; tile += gridDim.x, ++k) {
             float4 *ub = uslot + k * (kThreads * kSlots);
             const int64_t tl = static_cast<int64_t>(tile) * kTile, lo = max(c0, tl), hi = min(c1, tl + kTile);
-            if (lo == tl && hi == tl + kTile) worker_u_range<MODE, true>(a, tile, lo, hi, ub);
-            else worker_u_range<MODE, false>(a, tile, lo, hi, ub);
-            group_partials<QK>(USmem{ub}, tile, lo, hi, a.d, a.q, tile_ref(a.q.grp, tile, a.d), nullptr, a.partials, gs.parts, turn);
+            if (lo == tl && hi == tl + kTile) worker_u_range<MODE, true>(a, p, tile, lo, hi, ub);
+            else worker_u_range<MODE, false>(a, p, tile, lo, hi, ub);
+            group_partials<QK>(USmem{ub}, tile, lo, hi, a.d, a.q, tile_ref(a.q.grp, tile, a.d), nullptr, p.partials, gs.parts, turn);
         }
         if (!wave_barrier(gp, w, a.status, gs)) return;
-        encode_wave<QK>(uslot, t0, t_end, c0, c1, a.d, a.q, a.words, a.partials, a.scales, a.e, a.ef, a.seed, a.id,
+        encode_wave<QK>(uslot, t0, t_end, c0, c1, a.d, a.q, p.words, p.partials, p.scales, p.e, a.ef, a.seed, (a.id + blockIdx.y),
                         a.t, gs);
     }
 }
@@ -434,7 +443,8 @@ __global__ void fill_kernel(float *p, int64_t count, float value)
 template <int MODE>
 static cudaError_t launch_worker_mode(const WorkerArgs &a, cudaStream_t s, bool overlap)
 {
-    const dim3 grid(static_cast<unsigned>(a.n_tiles + (a.pass == PASS_LAZY ? a.q.grp.n_slow : 0))), block(kThreads);
+    const dim3 grid(static_cast<unsigned>(a.n_tiles + (a.pass == PASS_LAZY ? a.q.grp.n_slow : 0)), static_cast<unsigned>(a.count)),
+        block(kThreads);
     if (a.pass == PASS_LAZY)
         return a.q.kind == QK_SIGN ? launch_pdl(worker_lazy_kernel<MODE>, grid, block, 0, s, overlap, kCarveoutPercent, a) : cudaErrorNotSupported;
     switch (a.q.kind) {

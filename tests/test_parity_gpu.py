@@ -233,6 +233,52 @@ def test_lazy_views_mid_round_change_nothing(group):
     assert a.launches_per_round == cfg.n + 1 + 2 + 1
 
 
+@pytest.mark.parametrize("qw,n", [(W.sign_q(0), 3), (W.uniform_q(4, 4096, True), 33), (W.uniform_q(8, 512, False), 65),
+                                  (W.pow2_q(-17, -11, 4), 10), (W.uniform_q(8, 0, False), 2)])
+@pytest.mark.parametrize("d", [500, 9000])
+@pytest.mark.parametrize("placement", [ea.ADAM_AT_WORKER, ea.ADAM_AT_SERVER])
+def test_round_step_equals_separate_calls(qw, n, d, placement):
+    """EARound.step, whose workers share launches (up to 32 each), leaves the same bits as one call each."""
+    cfg = ea.EAConfig(d=d, n=n, qw=qw, qs=W.sign_q(4096), alpha=1e-3, placement=placement, seed=3)
+    a, b = ea.EARound(cfg), ea.EARound(cfg)
+    gen = torch.Generator(device="cuda").manual_seed(d + n)
+    xa, xb = torch.zeros(d, device="cuda"), torch.zeros(d, device="cuda")
+    for t in range(3):
+        g = [torch.randn(d, device="cuda", generator=gen) for _ in range(n)]
+        a.step(g, xa)
+        for i in range(n):
+            b.worker_compress(i, g[i])
+        b.server_step()
+        b.apply(xb)
+    worker = [ea.EA_VIEW_CODES_WORKER, ea.EA_VIEW_SCALES_WORKER, ea.EA_VIEW_E_WORKER]
+    worker += [ea.EA_VIEW_M, ea.EA_VIEW_V] if placement == ea.ADAM_AT_WORKER else []
+    for i in range(n):
+        for v in worker:
+            assert torch.equal(a.view(v, i), b.view(v, i)), (v, i)
+    for v in (ea.EA_VIEW_CODES_SERVER, ea.EA_VIEW_SCALES_SERVER, ea.EA_VIEW_E_SERVER):
+        assert torch.equal(a.view(v), b.view(v))
+    assert torch.equal(xa, xb) and a.t == b.t == 3 and a.bits_sent() == b.bits_sent()
+
+
+def test_round_step_stops_where_a_call_is_refused():
+    cfg = ea.EAConfig(d=9000, n=3, qw=W.sign_q(4096), qs=W.sign_q(4096), alpha=1e-3)
+    r = ea.EARound(cfg)
+    g = torch.zeros(9004, device="cuda")
+    x = torch.zeros(9000, device="cuda")
+    with pytest.raises(ea.EAError) as ex:
+        r.step([g[:9000], g[1:9001], g[:9000]], x)  # worker 1's gradient is not 16-byte aligned
+    assert ex.value.status == ea.EA_E_ALIGN and r.t == 0
+    with pytest.raises(ea.EAError) as ex:
+        r.worker_compress(0, g)  # worker 0 has compressed
+    assert ex.value.status == ea.EA_E_ORDER
+    r.worker_compress(1, g)
+    r.worker_compress(2, g)
+    r.server_step()
+    r.apply(x)
+    r.sync()
+    assert r.t == 1
+
+
 def test_replicas_are_identical_and_protocol():
     cfg = ea.EAConfig(d=10_000, n=2, qw=W.sign_q(4096), qs=W.sign_q(4096), alpha=1e-3)
     rnd = ea.EARound(cfg)
