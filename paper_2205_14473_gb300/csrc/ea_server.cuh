@@ -711,7 +711,8 @@ __device__ __forceinline__ void unif_decode_sum(const unsigned char *codes, int 
 
 // One tile of the staged server on the compute warps: the stage `st` holds e_s (m_s, v_s), the
 // workers' code chunks and scales.  The stage's e_s slots then hold u until the re-quantization
-// has read it; the stage is released (arrive on `empty`) after that.
+// has read it; the stage is released (arrive on `empty`) after that.  With Adam at the server, all of
+// it but those slots is released as soon as u is formed (arrive on `early`).
 // NW: the worker count when it is 8, known at compile time (the per-worker bounds, the average's
 // division and the decode loops then fold; for scaled-sign workers the table is the whole average
 // and the per-worker path is not compiled in), or 0 for a count known at run time.
@@ -721,7 +722,7 @@ __device__ __forceinline__ void unif_decode_sum(const unsigned char *codes, int 
 // sign, the codes) as PASS_STASH and PASS_LAZY do.
 template <int MODE, int QW, int QS, bool FULL, int NW, bool GENERAL>
 __device__ __forceinline__ bool server_staged_tile(const ServerArgs &a, int64_t tile, const unsigned char *st,
-                                                   bool ok, uint64_t *empty, int Lw, float Lwf, const float *utab,
+                                                   bool ok, uint64_t *early, uint64_t *empty, int Lw, float Lwf, const float *utab,
                                                    float *wtab, const uint32_t (&flip)[8], TileSmem &sm)
 {
     static_assert(NW == 0 || NW == 8, "a compile-time worker count of 8");
@@ -933,6 +934,10 @@ __device__ __forceinline__ bool server_staged_tile(const ServerArgs &a, int64_t 
             store4<FULL>(a.vs, q, d, vs);
         }
     }
+    if constexpr (MODE == MODE_S) {
+        __syncwarp();
+        if ((threadIdx.x & 31) == 0) mbar_arrive(early);
+    }
     if constexpr (GENERAL && has_scale<QS>()) {
         constexpr int spans = QS == QK_SIGN ? PASS_LAZY_ONE : PASS_STASH_ONE;  // groups of several tiles
         if (a.pass == (QS == QK_SIGN ? PASS_LAZY : PASS_STASH))
@@ -955,7 +960,10 @@ __device__ __forceinline__ bool server_staged_tile(const ServerArgs &a, int64_t 
 // warps and 1 producer warp: the producer streams, for each of the CTA's tiles, the e_s tile (and
 // m_s, v_s with Adam at the server) and the n workers' code chunks with bulk copies, and the n
 // worker scales with 4-byte cp.async, into a ring of stages guarded by full/empty mbarriers; the
-// compute warps decode, average, re-quantize and write e_s and the broadcast straight to HBM.
+// compute warps decode, average, re-quantize and write e_s and the broadcast straight to HBM.  With Adam
+// at the server a stage holds 48 KB of state, so that three CTAs per SM have one each; everything
+// but e_s is refilled while the tile is still being encoded (27,000,001 coordinates, five workers, 4- and
+// 8-bit grids: the round 515 us with one release per stage, 502 us with two).
 // Used when no tile lies in several scale groups of Q_s or Q_w of which one spans tiles; GENERAL: some
 // tile holds several groups, or some group several tiles.
 template <int MODE, int QW, int QS, bool GENERAL>
@@ -972,15 +980,17 @@ __global__ void __launch_bounds__(kThreads + 32, server_ctas_per_sm(MODE, QW, QS
     const int S = P.stages;
     uint64_t *full = reinterpret_cast<uint64_t *>(dsm);
     uint64_t *empty = full + S;
-    unsigned char *stage0 = dsm + 128 * ((2 * S * 8 + 127) / 128);
+    uint64_t *early = empty + S;  // Adam at the server only (then S <= 4: 48 KB of state per stage)
+    unsigned char *stage0 = dsm + 128;
     constexpr bool scaled_w = has_scale<QW>();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     pdl_trigger();
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
-            mbar_init(&full[s], 1 + (scaled_w ? 32 : 0));
+            mbar_init(&full[s], (MODE == MODE_S ? 2 : 1) + (scaled_w ? 32 : 0));
             mbar_init(&empty[s], kWarps);
+            if (MODE == MODE_S) mbar_init(&early[s], kWarps);
         }
         mbar_init_fence();
     }
@@ -999,7 +1009,8 @@ __global__ void __launch_bounds__(kThreads + 32, server_ctas_per_sm(MODE, QW, QS
         for (int64_t at = blockIdx.x; at < a.n_tiles; at += gridDim.x, ++it) {
             const int64_t tile = a.n_tiles - 1 - at;  // the ragged one first (see cta_tile)
             const int s = static_cast<int>(it % S);
-            if (it >= S && !mbar_wait(&empty[s], static_cast<uint32_t>(((it / S) & 1) ^ 1))) {
+            const uint32_t reused = static_cast<uint32_t>(((it / S) & 1) ^ 1);  // the phase that frees stage s
+            if (it >= S && !mbar_wait(MODE == MODE_S ? &early[s] : &empty[s], reused)) {
                 ok = false;
                 break;
             }
@@ -1009,11 +1020,12 @@ __global__ void __launch_bounds__(kThreads + 32, server_ctas_per_sm(MODE, QW, QS
             const int64_t coff = tile * static_cast<int64_t>(P.code_chunk);
             const uint32_t cb = static_cast<uint32_t>(min(static_cast<int64_t>(P.code_chunk), a.wcode_bytes - coff));
             if (lane == 0) {
-                mbar_arrive_expect_tx(&full[s], vb * (MODE == MODE_S ? 3u : 1u) + cb * static_cast<uint32_t>(a.n));
-                bulk_g2s(st + P.off_a, a.es + lo, vb, &full[s]);
+                mbar_arrive_expect_tx(&full[s], vb * (MODE == MODE_S ? 2u : 1u) + cb * static_cast<uint32_t>(a.n));
                 if (MODE == MODE_S) {
                     bulk_g2s(st + P.off_b, a.ms + lo, vb, &full[s]);
                     bulk_g2s(st + P.off_c, a.vs + lo, vb, &full[s]);
+                } else {
+                    bulk_g2s(st + P.off_a, a.es + lo, vb, &full[s]);
                 }
                 const unsigned char *wb = reinterpret_cast<const unsigned char *>(a.wwords) + coff;
                 for (int w = 0; w < a.n; ++w)
@@ -1033,6 +1045,17 @@ __global__ void __launch_bounds__(kThreads + 32, server_ctas_per_sm(MODE, QW, QS
                     for (int w = lane; w < a.n; w += 32) cp_async4(sc + w, a.wscales + w * a.wscales_stride + tile);
                 }
                 cp_async_arrive_noinc(&full[s]);
+            }
+            if constexpr (MODE == MODE_S) {  // e_s once u has been encoded from its slots
+                ok = it < S || mbar_wait(&empty[s], reused);
+                if (lane == 0) {
+                    mbar_arrive_expect_tx(&full[s], ok ? vb : 0u);
+                    if (ok) bulk_g2s(st + P.off_a, a.es + lo, vb, &full[s]);
+                }
+                if (!ok) {
+                    ++it;  // the copies above are waited for below
+                    break;
+                }
             }
         }
         // the copies of the last stages must land before the CTA may exit
@@ -1061,12 +1084,12 @@ __global__ void __launch_bounds__(kThreads + 32, server_ctas_per_sm(MODE, QW, QS
         const bool whole = (tile + 1) * kTile <= d;
         bool go;
         if constexpr (GENERAL) {
-            go = whole ? server_staged_tile<MODE, QW, QS, true, 0, true>(a, tile, st, ok, &empty[s], Lw, Lwf, ut, wtab, flip, sm)
-                       : server_staged_tile<MODE, QW, QS, false, 0, true>(a, tile, st, ok, &empty[s], Lw, Lwf, ut, wtab, flip, sm);
+            go = whole ? server_staged_tile<MODE, QW, QS, true, 0, true>(a, tile, st, ok, &early[s], &empty[s], Lw, Lwf, ut, wtab, flip, sm)
+                       : server_staged_tile<MODE, QW, QS, false, 0, true>(a, tile, st, ok, &early[s], &empty[s], Lw, Lwf, ut, wtab, flip, sm);
         } else {
-            go = !whole ? server_staged_tile<MODE, QW, QS, false, 0, false>(a, tile, st, ok, &empty[s], Lw, Lwf, ut, wtab, flip, sm)
-                 : n8   ? server_staged_tile<MODE, QW, QS, true, 8, false>(a, tile, st, ok, &empty[s], Lw, Lwf, ut, wtab, flip, sm)
-                        : server_staged_tile<MODE, QW, QS, true, 0, false>(a, tile, st, ok, &empty[s], Lw, Lwf, ut, wtab, flip, sm);
+            go = !whole ? server_staged_tile<MODE, QW, QS, false, 0, false>(a, tile, st, ok, &early[s], &empty[s], Lw, Lwf, ut, wtab, flip, sm)
+                 : n8   ? server_staged_tile<MODE, QW, QS, true, 8, false>(a, tile, st, ok, &early[s], &empty[s], Lw, Lwf, ut, wtab, flip, sm)
+                        : server_staged_tile<MODE, QW, QS, true, 0, false>(a, tile, st, ok, &early[s], &empty[s], Lw, Lwf, ut, wtab, flip, sm);
         }
         if (!go) {
             if (threadIdx.x == 0) report_status(a.status, kStatusTimeout);
