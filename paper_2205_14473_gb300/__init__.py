@@ -16,7 +16,6 @@ from __future__ import annotations
 
 import ctypes
 import dataclasses
-import itertools
 import os
 import threading
 
@@ -258,10 +257,14 @@ class EARound:
     def step(self, grads, x) -> None:
         """One full round: every worker compresses its gradient, the server broadcasts, x moves."""
         n, d = self.cfg.n, self.cfg.d
-        if len(grads) >= n and x.is_contiguous() and x.numel() >= d and all(
-                g.dtype.is_floating_point and g.is_contiguous() and g.numel() >= d for g in itertools.islice(grads, n)):
-            ptrs = (_P * n)(*[grads[i].data_ptr() for i in range(n)])
-            ea_round_step(self.h, ptrs, x.data_ptr())
+        try:
+            gs = [grads[i] for i in range(n)]
+            accepted = x.is_contiguous() and x.numel() >= d and all(
+                g.dtype.is_floating_point and g.is_contiguous() and g.numel() >= d for g in gs)
+        except (AttributeError, IndexError, KeyError, TypeError):
+            accepted = False
+        if accepted:
+            ea_round_step(self.h, (_P * n)(*[g.data_ptr() for g in gs]), x.data_ptr())
             return
         for i in range(n):  # what is not accepted fails where its own call does
             self.worker_compress(i, grads[i])

@@ -589,28 +589,28 @@ int compress_workers(ea_handle *h, int32_t first, const float *const *gs, int32_
     for (int32_t at = 0; at < count;) {
         const int32_t w = first + at;
         a.lazy_in = lazy ? h->lazy_w[w] : 0;
-        a.count = 1;
-        while (together && a.count < kWorkerBatch && at + a.count < count && (!lazy || h->lazy_w[w + a.count] == a.lazy_in))
-            ++a.count;
-        for (int i = 0; i < a.count; ++i) {
+        int m = 1;  // workers of this launch
+        while (together && m < kWorkerBatch && at + m < count && (!lazy || h->lazy_w[w + m] == a.lazy_in)) ++m;
+        WorkerBufs p[kWorkerBatch];
+        for (int i = 0; i < m; ++i) {
             const int64_t k = w + i;
-            a.w[i] = WorkerBufs{gs[at + i], W ? h->m + k * dp : nullptr, W ? h->v + k * dp : nullptr, h->e + k * dp,
-                                h->wcodes + k * h->lay.wcode_stride, h->wscales + k * h->lay.wscale_stride,
-                                h->partials + (lazy ? k * h->qw.n_pairs : 0)};
+            p[i] = WorkerBufs{gs[at + i], W ? h->m + k * dp : nullptr, W ? h->v + k * dp : nullptr, h->e + k * dp,
+                              h->wcodes + k * h->lay.wcode_stride, h->wscales + k * h->lay.wscale_stride,
+                              h->partials + (lazy ? k * h->qw.n_pairs : 0)};
         }
         a.id = static_cast<uint32_t>(w);
         int r;
         if (h->qw.pass == PASS_GROUPED) {
             a.gp = device_group_plan(h->qw, h->epoch_w);
-            r = check_cuda(h, launch_worker_grouped(W ? MODE_W : MODE_S, a, h->qw.grid, h->stream), "worker launch");
+            r = check_cuda(h, launch_worker_grouped(W ? MODE_W : MODE_S, a, p[0], h->qw.grid, h->stream), "worker launch");
             if (r == EA_OK) ++h->epoch_w;
             h->split_full = true;
         } else {
-            r = check_cuda(h, launch_worker(W ? MODE_W : MODE_S, a, h->stream, may_overlap(h)), "worker launch");
+            r = check_cuda(h, launch_worker(W ? MODE_W : MODE_S, a, p, m, h->stream, may_overlap(h)), "worker launch");
         }
-        if (r == EA_OK && h->qw.pass == PASS_STASH) r = second_pass(h, h->qw, a.w[0].partials, a.w[0].e, a.w[0].words, a.w[0].scales, a.id);
+        if (r == EA_OK && h->qw.pass == PASS_STASH) r = second_pass(h, h->qw, p[0].partials, p[0].e, p[0].words, p[0].scales, a.id);
         if (r != EA_OK) return r;
-        for (int i = 0; i < a.count; ++i) {
+        for (int i = 0; i < m; ++i) {
             if (lazy) {  // the scales are formed for all workers before the server step
                 h->lazy_w[w + i] = h->cfg.error_feedback ? 1 : 0;
                 h->wscales_pending = true;
@@ -618,7 +618,7 @@ int compress_workers(ea_handle *h, int32_t first, const float *const *gs, int32_
             h->compressed[w + i] = 1;
             ++h->n_compressed;
         }
-        at += a.count;
+        at += m;
     }
     return EA_OK;
 }

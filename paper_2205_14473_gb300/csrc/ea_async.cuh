@@ -108,10 +108,10 @@ __device__ __forceinline__ void report_status(uint32_t *status, uint32_t code)
 
 // Programmatic dependent launch.  The round's kernels are launched with programmatic stream
 // serialization (launch_pdl): each lets the next kernel on the stream be scheduled as soon as all of
-// its own CTAs have started (pdl_trigger), and each waits, before its first access to global
-// memory, until the previous kernel has completed and its writes are visible (pdl_wait).  The next
-// kernel's launch and shared-memory prologue thus overlap this one's last CTAs; the data order of
-// the stream is unchanged.  Without the launch attribute both are no-ops.
+// its own CTAs have started (pdl_trigger), and each waits, before its first access to anything that a
+// kernel writes, until the previous kernel has completed and its writes are visible (pdl_wait).  The
+// next kernel's launch, shared-memory prologue and lookups in the handle's constant tables thus
+// overlap this one's last CTAs; the data order of the stream is unchanged.  Without the launch attribute both are no-ops.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

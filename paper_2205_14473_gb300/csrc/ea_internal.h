@@ -132,8 +132,7 @@ struct GroupedShape {
     int ctas_per_sm, slots;
 };
 
-// Workers whose messages one launch may compress (blockIdx.y).  Their buffers' addresses travel in the
-// launch parameters (56 bytes each of the 4 KB), where a thread reads them when it needs them.
+// Workers whose messages one launch may compress (blockIdx.y).
 constexpr int kWorkerBatch = 32;
 
 struct WorkerBufs {
@@ -144,10 +143,23 @@ struct WorkerBufs {
     double *partials;
 };
 
+// The buffers of a launch's workers, a launch parameter that a thread reads when it needs an address.  A
+// launch of one worker carries 56 bytes of them and not the list's 1.8 KB, which took it 0.5 us longer.
+struct WorkerOne {
+    WorkerBufs w;
+#ifdef __CUDACC__
+    __device__ const WorkerBufs &at(unsigned) const { return w; }
+#endif
+};
+struct WorkerList {
+    WorkerBufs w[kWorkerBatch];
+#ifdef __CUDACC__
+    __device__ const WorkerBufs &at(unsigned y) const { return w[y]; }
+#endif
+};
+
 struct WorkerArgs {
     int64_t d, n_tiles;
-    int count;                  // workers of this launch
-    WorkerBufs w[kWorkerBatch];
     QParams q;
     Hyper hp;
     int ef, pass;
@@ -238,9 +250,14 @@ struct ApplyArgs {
 };
 
 // overlap: the launch may begin before its predecessor has finished (see launch_pdl).
-cudaError_t launch_worker(int mode, const WorkerArgs &a, cudaStream_t s, bool overlap = true);
+cudaError_t launch_worker(int mode, const WorkerArgs &a, const WorkerBufs *w, int count, cudaStream_t s,
+                          bool overlap = true);
 // The one-pass kernels of PASS_GROUPED (cooperative launches of `grid` CTAs) and their shapes.
-cudaError_t launch_worker_grouped(int mode, const WorkerArgs &a, int grid, cudaStream_t s);
+struct WorkerGroupedArgs {
+    WorkerArgs a;
+    WorkerBufs p;
+};
+cudaError_t launch_worker_grouped(int mode, const WorkerArgs &a, const WorkerBufs &p, int grid, cudaStream_t s);
 cudaError_t worker_grouped_shape(int mode, int qk, GroupedShape *out);
 template <int MODE, int QS>
 cudaError_t launch_server_grouped_for_qs(const ServerArgs &a, int grid, cudaStream_t s);

@@ -113,8 +113,7 @@ extern "C" int ea_worker_compress_noalloc(const ea_config *cfg, int32_t worker, 
     WorkerArgs a{};
     a.d = d;
     a.n_tiles = n_tiles;
-    a.count = 1;
-    a.w[0] = WorkerBufs{g, W ? m : nullptr, W ? v : nullptr, e, codes, scales, partials};
+    const WorkerBufs p{g, W ? m : nullptr, W ? v : nullptr, e, codes, scales, partials};
     a.q = qp;
     a.hp.alpha = cfg->alpha;
     a.hp.beta1 = cfg->beta1;
@@ -138,7 +137,7 @@ extern "C" int ea_worker_compress_noalloc(const ea_config *cfg, int32_t worker, 
         write_group_offsets<<<1, 32, 0, s>>>(pair_base, n_tiles);
         ce = cudaGetLastError();
     }
-    if (ce == cudaSuccess) ce = launch_worker(W ? MODE_W : MODE_S, a, s);
+    if (ce == cudaSuccess) ce = launch_worker(W ? MODE_W : MODE_S, a, &p, 1, s);
     if (ce == cudaSuccess && a.pass == PASS_STASH) {
         FinalizeArgs f{};
         f.d = d;
