@@ -136,8 +136,8 @@ int ea_bits_sent(const ea_handle *h, uint64_t *up_bits, uint64_t *down_bits);
 int ea_round_index(const ea_handle *h, int64_t *t);
 
 /* Kernel launches that one round of separate calls makes on the stream: n worker compresses, one server
- * step and one apply (ea_round_step makes fewer).  A message whose scale groups lie inside 4096-coordinate tiles takes one launch.  When the
- * groups span tiles:
+ * step and one apply (ea_round_step makes fewer).  A message without scales, with 4096-blocks, with power-of-two blocks of 128 to 2048, or whose
+ * one group is at most 4096 long takes one launch.  With other groups:
  *   - a scaled-sign message takes one pass, which writes the codes (the signs, which need no scale)
  *     with the groups' partial norms, and a finalize forms the scales: one finalize for all worker
  *     messages (at the server step, or at a view of a worker's scales or residual), one for the

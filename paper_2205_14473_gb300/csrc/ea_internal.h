@@ -99,11 +99,11 @@ enum Pass : int {
                       // partial norm per (tile, group); finalize_kernel and encode_kernel finish
     PASS_GROUPED = 2, // groups span tiles, one cooperative pass: the input stays in shared memory
                       // while the group's partial norms are combined (GroupPlan)
-    PASS_LAZY = 3     // scaled sign, groups span tiles: the codes (signs) need no scale, so one pass
+    PASS_LAZY = 3,    // scaled sign, groups span tiles: the codes (signs) need no scale, so one pass
                       // writes them with the partial norms and keeps u itself in the residual
                       // buffer; finalize_kernel forms the scales, and e = u - Q(u) is formed from
                       // (u, s) where it is next needed (the next round's pass, or a view)
-    , PASS_SHORT = 4  // several groups per tile, each a whole number of warp slots (power-of-two
+    PASS_SHORT = 4    // several groups per tile, each a whole number of warp slots (power-of-two
                       // blocks of 128 .. 2048): one pass, a scale per chunk (see chunk_scales)
 };
 

@@ -598,16 +598,6 @@ cudaError_t launch_server_lazy(const ServerArgs &a, bool staged, cudaStream_t s)
 
 constexpr int kWorkerTab = 1024;  // floats of the staged server's per-tile worker table
 
-// Bits 0, 4, ..., 28 of x moved to bits 0 .. 7 (the inverse of spread8_by4).
-__device__ __forceinline__ uint32_t gather_every4(uint32_t x)
-{
-    x &= 0x11111111u;
-    x = (x | (x >> 3)) & 0x03030303u;
-    x = (x | (x >> 6)) & 0x000f000fu;
-    x = (x | (x >> 12)) & 0x000000ffu;
-    return x;
-}
-
 // All 256 compute threads agree on `ok` (named barrier 1 with an AND reduction).
 __device__ __forceinline__ bool compute_all(bool ok)
 {
