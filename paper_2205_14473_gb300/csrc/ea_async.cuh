@@ -34,6 +34,11 @@ __device__ __forceinline__ void mbar_init_fence()
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
+// Order this thread's plain accesses to shared memory before later ones of the async (copy) proxy, which
+// an mbarrier alone does not: the reader of a stage that a bulk copy refills calls it before it arrives
+// on the stage's barrier, if it has also written there.
+__device__ __forceinline__ void proxy_fence() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t bytes)
 {
     asm volatile("mbarrier.arrive.expect_tx.release.cta.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)),

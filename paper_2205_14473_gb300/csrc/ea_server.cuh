@@ -940,7 +940,9 @@ __device__ __forceinline__ bool server_staged_tile(const ServerArgs &a, int64_t 
         finish_tile_smem<QS, FULL, false>(ubuf, l1, mx, tile, d, a.qs, a.words, a.scales, a.es, a.ef, a.seed,
                                           static_cast<uint32_t>(a.n), a.t, sm);
     }
-    // the stage is no longer read: hand it back to the producer
+    // the stage is no longer read: hand it back to the producer, whose bulk copy of the next e_s must
+    // come after the u written into these slots
+    proxy_fence();
     __syncwarp();
     if ((threadIdx.x & 31) == 0) mbar_arrive(empty);
     return true;

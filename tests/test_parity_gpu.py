@@ -155,6 +155,22 @@ def test_short_blocks(qw, qs, d, n, placement):
     _run_host(cfg, 2 if d > 100_000 else 3, seed=d + n, grad_scale=1e-3)
 
 
+@pytest.mark.parametrize("qw,qs,tiles,tail,placement", [
+    (W.sign_q(0), W.sign_q(0), 456 * 3, 777, ea.ADAM_AT_SERVER),
+    (W.uniform_q(4, 512, True), W.uniform_q(8, 512, False), 456 * 3, 777, ea.ADAM_AT_SERVER),
+    (W.uniform_q(8, 0, False), W.uniform_q(8, 0, False), 456 * 5, 777, ea.ADAM_AT_SERVER),  # beyond the grouped pass
+    (W.sign_q(8192), W.sign_q(12288), 456 * 3, 777, ea.ADAM_AT_SERVER),
+    (W.sign_q(0), W.sign_q(0), 608 * 4, 1, ea.ADAM_AT_WORKER),
+    (W.sign_q(12288), W.uniform_q(8, 512, False), 456 * 6, 4095, ea.ADAM_AT_WORKER),
+])
+def test_general_staged_server_refills_its_stages(qw, qs, tiles, tail, placement):
+    """Short blocks, and scales of several whole tiles, in the staged server with more tiles per CTA than it
+    has stages (one stage with Adam at the server, whose e_s slots are refilled after the rest), so that
+    every stage is handed back, with u written in it, and filled again."""
+    cfg = ea.EAConfig(d=4096 * tiles + tail, n=3, qw=qw, qs=qs, alpha=1e-3, placement=placement, seed=tiles)
+    _run_host(cfg, 3, seed=tiles + tail, grad_scale=1e-3)
+
+
 def test_two_pass_scale_beyond_the_grouped_capacity():
     """A whole-vector scale over 12.3 million coordinates: more tiles than the one-pass grouped
     kernels hold in shared memory at once (about 1,800 on a GB300).  The uniform-grid broadcast
