@@ -428,23 +428,25 @@ __device__ __forceinline__ int64_t tile_group_of(const Grouping &g, const TileGr
 // Coordinate j's b-bit code sits at bit j*b of the little-endian word stream.  A float4 slot q
 // (coordinates 4q .. 4q+3) spans 4b bits, so for b <= 8 it lies inside word (q*b)/8.
 
-// Load the four codes of slot q.
-__device__ __forceinline__ void load_codes4(const uint32_t *__restrict__ words, int64_t q, int bits, uint32_t c[4])
+// Load the four codes of slot q.  (Codes and scales are read by plain loads, not through the non-coherent
+// path of __ldg: the kernel that writes them may still run when the one that reads them has begun, see
+// pdl_wait.)
+__device__ __forceinline__ void load_codes4(const uint32_t *words, int64_t q, int bits, uint32_t c[4])
 {
     if (bits <= 8) {
-        const uint32_t w = __ldg(words + ((q * bits) >> 3));
+        const uint32_t w = words[(q * bits) >> 3];
         const int sh = static_cast<int>((q * bits) & 7) * 4;
         const uint32_t mask = (1u << bits) - 1u;
 #pragma unroll
         for (int i = 0; i < 4; ++i) c[i] = (w >> (sh + i * bits)) & mask;
     } else if (bits == 16) {
-        const uint2 w = __ldg(reinterpret_cast<const uint2 *>(words) + q);
+        const uint2 w = reinterpret_cast<const uint2 *>(words)[q];
         c[0] = w.x & 0xffffu;
         c[1] = w.x >> 16;
         c[2] = w.y & 0xffffu;
         c[3] = w.y >> 16;
     } else {
-        const uint4 w = __ldg(reinterpret_cast<const uint4 *>(words) + q);
+        const uint4 w = reinterpret_cast<const uint4 *>(words)[q];
         c[0] = w.x;
         c[1] = w.y;
         c[2] = w.z;

@@ -44,7 +44,7 @@ __device__ __forceinline__ void decode_sum_direct(const ServerArgs &a, int64_t t
             constexpr uint32_t pi = 0x73625140u;  // pi(w) in nibble w
             float t = 0.0f;
             for (int w = 0; w < m; ++w) {
-                const float sw = __ldg(a.wscales + static_cast<int64_t>(w) * a.wscales_stride + wg);
+                const float sw = a.wscales[static_cast<int64_t>(w) * a.wscales_stride + wg];
                 t = __fadd_rn(t, ((threadIdx.x >> ((pi >> (4 * w)) & 7u)) & 1u) ? sw : -sw);
             }
             stab[threadIdx.x] = t;
@@ -58,7 +58,7 @@ __device__ __forceinline__ void decode_sum_direct(const ServerArgs &a, int64_t t
 #pragma unroll
                 for (int w = 0; w < 8; ++w) {
                     if (w < m) {
-                        const uint32_t word = __ldg(a.wwords + static_cast<int64_t>(w) * a.wwords_stride + (q >> 3));
+                        const uint32_t word = a.wwords[static_cast<int64_t>(w) * a.wwords_stride + (q >> 3)];
                         X |= __funnelshift_r(word, word, (sh - 4 * w) & 31) & (0xfu << (4 * w));
                     }
                 }
@@ -94,7 +94,7 @@ __device__ __forceinline__ void decode_sum_direct(const ServerArgs &a, int64_t t
     for (int w = w_first; w < a.n; ++w) {
         const uint32_t *ww = a.wwords + static_cast<int64_t>(w) * a.wwords_stride;
         const float *wsc = a.wscales + static_cast<int64_t>(w) * a.wscales_stride;
-        const float s_tile = (has_scale<QW>() && wtile) ? __ldg(wsc + wg) : 0.0f;
+        const float s_tile = (has_scale<QW>() && wtile) ? wsc[wg] : 0.0f;
 #pragma unroll
         for (int k = 0; k < kSlots; ++k) {
             const int64_t q = slot_of(tile, k);
@@ -107,7 +107,7 @@ __device__ __forceinline__ void decode_sum_direct(const ServerArgs &a, int64_t t
                 if (j0 + i < d) {
                     float s = 0.0f;
                     if (has_scale<QW>())
-                        s = wtile ? s_tile : __ldg(wsc + whint + ((gl[k][i >> 1] >> (16 * (i & 1))) & 0xffffu));
+                        s = wtile ? s_tile : wsc[whint + ((gl[k][i >> 1] >> (16 * (i & 1))) & 0xffffu)];
                     acc[k][i] = __fadd_rn(acc[k][i], decode1<QW>(c[i], s, a.qw, Lwf, Lw, utab));
                 }
             }

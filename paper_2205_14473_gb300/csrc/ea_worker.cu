@@ -343,14 +343,14 @@ __device__ __forceinline__ void apply_tile(const ApplyArgs &a, int64_t tile, con
         load4<FULL>(a.x, q, d, x[k]);
         raw[k] = make_uint4(0u, 0u, 0u, 0u);
         if (FULL || 4 * q < d) {
-            if constexpr (has_scale<QK>() && SCALES == AS_SLOT) s_slot[k] = __ldg(a.scales + ((4 * q) >> G.log2G));
+            if constexpr (has_scale<QK>() && SCALES == AS_SLOT) s_slot[k] = a.scales[(4 * q) >> G.log2G];
             if constexpr (bits <= 8) {
-                raw[k].x = __ldg(a.words + ((q * bits) >> 3));
+                raw[k].x = a.words[(q * bits) >> 3];
             } else if constexpr (bits == 16) {
-                const uint2 w = __ldg(reinterpret_cast<const uint2 *>(a.words) + q);
+                const uint2 w = reinterpret_cast<const uint2 *>(a.words)[q];
                 raw[k].x = w.x, raw[k].y = w.y;
             } else {
-                raw[k] = __ldg(reinterpret_cast<const uint4 *>(a.words) + q);
+                raw[k] = reinterpret_cast<const uint4 *>(a.words)[q];
             }
         }
     }
@@ -362,7 +362,7 @@ __device__ __forceinline__ void apply_tile(const ApplyArgs &a, int64_t tile, con
     // one scale for the whole tile: 4096-blocks, or a tile inside one group
     const int64_t g1 = (!has_scale<QK>() || SCALES == AS_SLOT) ? 0 : SCALES == AS_TILE ? tile : FULL || ref.ng() == 1 ? ref.g0 : -1;
     const bool tile_scale = SCALES != AS_ANY || FULL || g1 >= 0;
-    const float s_tile = (has_scale<QK>() && SCALES != AS_SLOT && tile_scale) ? __ldg(a.scales + g1) : 0.0f;
+    const float s_tile = (has_scale<QK>() && SCALES != AS_SLOT && tile_scale) ? a.scales[g1] : 0.0f;
 #pragma unroll
     for (int k = 0; k < kSlots; ++k) {
         const int64_t q = slot_of(tile, k);
@@ -382,7 +382,7 @@ __device__ __forceinline__ void apply_tile(const ApplyArgs &a, int64_t tile, con
         for (int i = 0; i < 4; ++i) {
             if (FULL || j0 + i < d) {
                 float s = SCALES == AS_SLOT ? s_slot[k] : s_tile;
-                if (has_scale<QK>() && !tile_scale) s = __ldg(a.scales + tile_group_of(G, tg, tile, j0 + i));
+                if (has_scale<QK>() && !tile_scale) s = a.scales[tile_group_of(G, tg, tile, j0 + i)];
                 x[k][i] = __fsub_rn(x[k][i], decode1<QK>(c[i], s, a.q, Lf, L, qtab));
             }
         }

@@ -104,6 +104,19 @@ def test_null_handle_calls(ea_lib):
     assert ea_lib.ea_destroy(None) == 0
 
 
+def test_read_only_loads_are_of_constant_tables_only():
+    """A kernel of a round may begin while the one before it still writes codes and scales (programmatic
+    dependent launch); ld.global.nc is for data that nothing writes while the kernel runs, so __ldg may
+    read nothing but the handle's tables of scale groups, which are written once, before any kernel."""
+    csrc = os.path.join(ROOT, "paper_2205_14473_gb300", "csrc")
+    found = []
+    for f in sorted(os.listdir(csrc)):
+        for line in open(os.path.join(csrc, f)):
+            code = line.split("//")[0]
+            found += re.findall(r"(?:__ldg\(|ld\.global\.nc).*", code)
+    assert [f for f in found if not f.startswith("__ldg(reinterpret_cast<const longlong2 *>(g.ref) + tile)")] == []
+
+
 def test_product_path_has_no_fallback(monkeypatch, tmp_path):
     """Without libea.so the binding raises instead of computing anything elsewhere."""
     import importlib
