@@ -134,7 +134,10 @@ __device__ __forceinline__ void group_partials(const USmem &src, int64_t tile, i
             }
             partials[ref.part() + i0] = part;
         }
-        if (last) break;
+        if (last) {
+            ++turn;  // the next call, too, writes the other half of pr while thread 0 may still read this one
+            break;
+        }
     }
 }
 
