@@ -255,17 +255,26 @@ class EARound:
         ea_worker_apply(self.h, x.data_ptr())
 
     def step(self, grads, x) -> None:
-        """One full round: every worker compresses its gradient, the server broadcasts, x moves."""
+        """One full round: every worker compresses its gradient, the server broadcasts, x moves.
+
+        grads[i] is worker i's gradient.  Tensors that are all at hand -- a list or tuple of them, or one
+        tensor of n rows -- are handed over in one call, in which workers share launches.  Any other sequence
+        is asked for one gradient at a time, after the worker before it has been launched, so it may form
+        them one after another in one buffer (on the round's stream)."""
+        from torch import Tensor
+
         n, d = self.cfg.n, self.cfg.d
-        try:
-            gs = [grads[i] for i in range(n)]
-            accepted = x.is_contiguous() and x.numel() >= d and all(
-                g.dtype.is_floating_point and g.is_contiguous() and g.numel() >= d for g in gs)
-        except (AttributeError, IndexError, KeyError, TypeError):
-            accepted = False
-        if accepted:
-            ea_round_step(self.h, (_P * n)(*[g.data_ptr() for g in gs]), x.data_ptr())
-            return
+        kind = type(grads)
+        if ((kind is list or kind is tuple or kind is Tensor and grads.dim() > 0) and len(grads) >= n
+                and isinstance(x, Tensor) and x.is_contiguous() and x.numel() >= d):
+            ptrs = []
+            for g in grads[:n]:
+                if not (isinstance(g, Tensor) and g.dtype.is_floating_point and g.is_contiguous() and g.numel() >= d):
+                    break
+                ptrs.append(g.data_ptr())
+            else:
+                ea_round_step(self.h, (_P * n)(*ptrs), x.data_ptr())
+                return
         for i in range(n):  # what is not accepted fails where its own call does
             self.worker_compress(i, grads[i])
         self.server_step()
