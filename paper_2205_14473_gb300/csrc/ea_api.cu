@@ -29,7 +29,8 @@ struct QHost {
     int64_t G = 0, n_groups = 1, n_words = 0, n_pairs = 0;
     bool has_scales = false;
     std::vector<int64_t> offsets;     // GK_SEG
-    std::vector<TileRef> ref;         // groups that span tiles: every tile's groups
+    int64_t n_ref = 0;                // groups that span tiles, but not the vector: one TileRef per tile
+    std::vector<TileRef> ref;         // those (build_tile_refs)
     std::vector<int32_t> slow;        // see Grouping
     std::vector<int64_t> pair_base;   // PASS_STASH, PASS_GROUPED
     std::vector<int64_t> cuts;        // PASS_GROUPED: the waves
@@ -209,28 +210,36 @@ int setup_quant(const ea_quantizer &q, int64_t d, const char *name, QHost &out)
             out.pair_base[gi + 1] = out.pair_base[gi] + ((e - 1) / kTile - b / kTile + 1);
         }
         out.n_pairs = out.pair_base.back();
-        if (out.gkind != GK_WHOLE) {
-            out.ref.resize(n_tiles);
-            auto group_end = [&](int64_t gi) {
-                return out.gkind == GK_BLOCK ? std::min(d, (gi + 1) * out.G) : out.offsets[gi + 1];
+        if (out.gkind != GK_WHOLE) out.n_ref = n_tiles;
+        if (out.gkind == GK_SEG && n_tiles < (int64_t{1} << 31)) {
+            // the tiles with a boundary inside them, and a ragged last one
+            auto add = [&out](int64_t t) {
+                if (out.slow.empty() || out.slow.back() != t) out.slow.push_back(static_cast<int32_t>(t));
             };
-            int64_t g0 = 0, part = 0;
-            for (int64_t t = 0; t < n_tiles; ++t) {
-                const int64_t hi = std::min(d, (t + 1) * kTile);
-                int64_t g = g0;
-                while (group_end(g) < hi) ++g;  // the group of the tile's last coordinate
-                out.ref[t] = TileRef{g0, part * 8192 + (g - g0 + 1)};
-                part += g - g0 + 1;
-                g0 = group_end(g) == hi ? g + 1 : g;
-            }
-            if (out.gkind == GK_SEG && n_tiles < (int64_t{1} << 31)) {
-                for (int64_t t = 0; t < n_tiles; ++t)
-                    if (out.ref[t].ng() > 1 || (t + 1) * kTile > d) out.slow.push_back(static_cast<int32_t>(t));
-                if (out.slow.size() > static_cast<size_t>(n_tiles / 8)) out.slow.clear();  // the common case then
-            }
+            for (int64_t gi = 1; gi < out.n_groups; ++gi)
+                if (out.offsets[gi] % kTile) add(out.offsets[gi] / kTile);
+            if (d % kTile) add(n_tiles - 1);
+            if (out.slow.size() > static_cast<size_t>(n_tiles / 8)) out.slow.clear();  // the common case then
         }
     }
     return EA_OK;
+}
+
+// Every tile's groups (see TileRef).  Not part of setup_quant: the size of a workspace does not need the
+// table, which for the largest d takes gigabytes and many seconds.
+void build_tile_refs(QHost &q, int64_t d)
+{
+    q.ref.resize(static_cast<size_t>(q.n_ref));
+    auto group_end = [&](int64_t gi) { return q.gkind == GK_BLOCK ? std::min(d, (gi + 1) * q.G) : q.offsets[gi + 1]; };
+    int64_t g0 = 0, part = 0;
+    for (int64_t t = 0; t < q.n_ref; ++t) {
+        const int64_t hi = std::min(d, (t + 1) * kTile);
+        int64_t g = g0;
+        while (group_end(g) < hi) ++g;  // the group of the tile's last coordinate
+        q.ref[t] = TileRef{g0, part * 8192 + (g - g0 + 1)};
+        part += g - g0 + 1;
+        g0 = group_end(g) == hi ? g + 1 : g;
+    }
 }
 
 int validate(const ea_config *cfg, QHost &qw, QHost &qs)
@@ -280,10 +289,10 @@ Layout make_layout(const ea_config &c, const QHost &qw, const QHost &qs)
     L.partials = (lazy_w ? static_cast<size_t>(c.n) * qw.n_pairs + qs.n_pairs
                          : static_cast<size_t>(std::max(qw.n_pairs, qs.n_pairs))) * sizeof(double);
     L.off_w = qw.gkind == GK_SEG ? qw.offsets.size() * 8 : 0;
-    L.ref_w = qw.ref.size() * sizeof(TileRef);
+    L.ref_w = static_cast<size_t>(qw.n_ref) * sizeof(TileRef);
     L.pb_w = qw.pass == PASS_STASH ? qw.pair_base.size() * 8 : 0;
     L.off_s = qs.gkind == GK_SEG ? qs.offsets.size() * 8 : 0;
-    L.ref_s = qs.ref.size() * sizeof(TileRef);
+    L.ref_s = static_cast<size_t>(qs.n_ref) * sizeof(TileRef);
     L.pb_s = qs.pass == PASS_STASH ? qs.pair_base.size() * 8 : 0;
     L.status = 4;
     L.slow_w = qw.slow.size() * 4;
@@ -694,6 +703,13 @@ int ea_init(const ea_config *cfg, void *workspace, size_t workspace_bytes, void 
     h->cfg.qs.seg_lengths = nullptr;
     h->qw = std::move(qw);
     h->qs = std::move(qs);
+    try {
+        build_tile_refs(h->qw, cfg->d);
+        build_tile_refs(h->qs, cfg->d);
+    } catch (const std::bad_alloc &) {
+        delete h;
+        return fail(nullptr, EA_E_INVAL, "out of host memory");
+    }
     h->lay = L;
     h->stream = static_cast<cudaStream_t>(stream);
     h->n_tiles = (cfg->d + kTile - 1) / kTile;

@@ -3,6 +3,8 @@ declares, sizes workspaces and rejects invalid configurations before any CUDA ca
 import ctypes
 import os
 import re
+import subprocess
+import sys
 
 import pytest
 
@@ -51,6 +53,25 @@ def test_workspace_bytes_covers_state(ea_lib):
     c5 = W.WORKLOADS["c5"]
     c, keep = ea.EAConfig.from_workload(c5).to_c()
     assert ea.ea_workspace_bytes(c) < 170e9
+
+
+@pytest.mark.parametrize("q", [W.sign_q(1 << 20), W.uniform_q(8, 12_288_000, False), W.sign_q(-1, (1 << 39, 1 << 39))])
+def test_workspace_bytes_needs_no_table_of_the_tiles(ea_lib, q):
+    """The size for the largest d (2^28 tiles) from its groups alone: the host memory of the query stays
+    below one byte per tile.  In a process of its own, whose peak is then the query's."""
+    code = f"""if True:
+        import resource
+        import paper_2205_14473_gb300 as ea
+        from paper_2205_14473_gb300.workloads import QuantSpec
+        q = {q!r}
+        c, keep = ea.EAConfig(d=1 << 40, n=1, qw=q, qs=q, alpha=1e-3).to_c()
+        ea.lib()
+        before = resource.getrusage(resource.RUSAGE_SELF).ru_maxrss
+        assert ea.ea_workspace_bytes(c) > 16 << 40
+        grown = resource.getrusage(resource.RUSAGE_SELF).ru_maxrss - before
+        assert grown < 256 << 10, f"{{grown}} KB"
+    """
+    subprocess.run([sys.executable, "-c", code], cwd=ROOT, check=True, timeout=300)
 
 
 @pytest.mark.parametrize("bad,status", [
