@@ -83,12 +83,29 @@ __device__ __forceinline__ void df_accumulate(DF &acc, float x)
 // warp that does not take part in the reductions.
 __device__ __forceinline__ void compute_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kThreads) : "memory"); }
 
+// Group scale of the scaled sign: ||u||_1 / G, the division in binary64, one rounding to binary32.
+__device__ __forceinline__ float sign_scale(double l1, int64_t len)
+{
+    return len > 0 ? __double2float_rn(__ddiv_rn(l1, static_cast<double>(len))) : 0.0f;
+}
+
+// The same of a compensated pair, len <= 4096.  For len = 2^k and a normal scale, RN32((hi + lo) / len) =
+// RN32(hi + lo) * 2^-k is one binary32 addition and an exact scaling; a subnormal scale has fewer bits than
+// RN32(hi + lo) and would be rounded a second time.
+__device__ __forceinline__ float sign_scale(DF l1, int64_t len)
+{
+    if (len > 0 && (len & (len - 1)) == 0) {
+        const int k = __ffsll(len) - 1;
+        const float s = __fmul_rn(__fadd_rn(l1.hi, l1.lo), __uint_as_float(static_cast<uint32_t>(127 - k) << 23));
+        if (!(s < 0x1p-126f)) return s;
+    }
+    return sign_scale(static_cast<double>(l1.hi) + static_cast<double>(l1.lo), len);
+}
+
 // Group scale of the scaled sign, ||u||_1 / G, for a group that is exactly this CTA's tile.
 // Every thread leaves its partial pair in red256; warp 0 combines the 256 pairs (8 per lane in a
-// tree, then a 5-level shuffle tree) and broadcasts the scale through *bcastf.  For G a
-// power of two, RN32((hi + lo) / G) = RN32(hi + lo) * 2^-k is one binary32 addition and an exact
-// scaling; other lengths (a ragged last tile) divide in binary64.  Two barriers; red256 and bcastf
-// may be reused after the function returns.
+// tree, then a 5-level shuffle tree) and broadcasts the scale through *bcastf.  Two barriers; red256
+// and bcastf may be reused after the function returns.
 __device__ __forceinline__ float block_sign_scale(DF v, int64_t len, DF *red256, float *bcastf)
 {
     red256[threadIdx.x] = v;
@@ -106,17 +123,7 @@ __device__ __forceinline__ float block_sign_scale(DF v, int64_t len, DF *red256,
             DF w{__shfl_down_sync(0xffffffffu, t.hi, o), __shfl_down_sync(0xffffffffu, t.lo, o)};
             t = df_add(t, w);
         }
-        if (threadIdx.x == 0) {
-            float s = 0.0f;
-            if (len > 0 && (len & (len - 1)) == 0) {  // len <= 4096 here: 2^-k is a normal binary32
-                const int k = __ffsll(static_cast<long long>(len)) - 1;
-                s = __fmul_rn(__fadd_rn(t.hi, t.lo), __uint_as_float(static_cast<uint32_t>(127 - k) << 23));
-            } else if (len > 0) {
-                const double l1 = static_cast<double>(t.hi) + static_cast<double>(t.lo);
-                s = __double2float_rn(__ddiv_rn(l1, static_cast<double>(len)));
-            }
-            *bcastf = s;
-        }
+        if (threadIdx.x == 0) *bcastf = sign_scale(t, len);
     }
     compute_sync();
     return *bcastf;
@@ -164,12 +171,6 @@ __device__ __forceinline__ float block_max_warp0(float a, uint32_t *red)
     if (lane == 0) red[threadIdx.x >> 5] = b;
     compute_sync();
     return threadIdx.x < 32 ? __uint_as_float(__reduce_max_sync(0xffffffffu, lane < kWarps ? red[lane] : 0u)) : 0.0f;
-}
-
-// Group scale of the scaled sign: ||u||_1 / G, the division in binary64, one rounding to binary32.
-__device__ __forceinline__ float sign_scale(double l1, int64_t len)
-{
-    return len > 0 ? __double2float_rn(__ddiv_rn(l1, static_cast<double>(len))) : 0.0f;
 }
 
 // ------------------------------------------------------------------------------- quantizers

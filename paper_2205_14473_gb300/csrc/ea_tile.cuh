@@ -189,10 +189,7 @@ __device__ __forceinline__ void chunk_scales(const USrc &src, int64_t tile, int6
         if constexpr (QK == QK_SIGN) {
             DF v = sm.red256[lane];
             for (int o = 1; o < (1 << sh); o <<= 1) v = df_add(v, shfl(v, o));
-            if (len > 0 && (len & (len - 1)) == 0)
-                s = __fmul_rn(__fadd_rn(v.hi, v.lo), __uint_as_float(static_cast<uint32_t>(127 - __ffs(len) + 1) << 23));
-            else if (len > 0)
-                s = sign_scale(static_cast<double>(v.hi) + static_cast<double>(v.lo), len);
+            s = sign_scale(v, len);
         } else {
             s = sm.red256[lane].hi;
             for (int o = 1; o < (1 << sh); o <<= 1) s = fmaxf(s, __shfl_xor_sync(0xffffffffu, s, o));

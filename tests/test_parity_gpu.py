@@ -1,5 +1,7 @@
 """GPU parity: the CUDA library, called through its C-ABI binding, against the oracle on the same
 seeded inputs, every round (see tests/parity.py for the tolerances)."""
+from fractions import Fraction
+
 import numpy as np
 import pytest
 import torch
@@ -153,6 +155,21 @@ def test_short_blocks(qw, qs, d, n, placement):
     blocks longer than the vector, several tiles per persistent server CTA)."""
     cfg = ea.EAConfig(d=d, n=n, qw=qw, qs=qs, alpha=1e-3, placement=placement, seed=d)
     _run_host(cfg, 2 if d > 100_000 else 3, seed=d + n, grad_scale=1e-3)
+
+
+@pytest.mark.parametrize("G", [128, 512, 2048, 4096])
+def test_subnormal_sign_scale_is_rounded_once(G):
+    """Blocks whose mean is just below 2^-126, of multiples of 2^-149: the sum needs more than 24 bits and
+    the mean has less, so rounding both would give another scale for one block in ten and more."""
+    d = 4096 * 64
+    cfg = ea.EAConfig(d=d, n=1, qw=W.sign_q(G), qs=W.identity_q(), alpha=1e-3, placement=ea.ADAM_AT_SERVER,
+                      error_feedback=False)
+    k = np.random.default_rng(G).integers(1 << 21, 1 << 23, d)
+    r = ea.EARound(cfg)
+    r.worker_compress(0, torch.from_numpy(k.astype(np.int32).view(np.float32)).cuda())
+    got = r.view(ea.EA_VIEW_SCALES_WORKER, 0).cpu().numpy().view(np.int32)
+    want = [round(Fraction(int(s), G)) for s in k.reshape(-1, G).sum(1)]  # to even at a tie
+    assert np.array_equal(got, np.array(want, np.int32))
 
 
 @pytest.mark.parametrize("qw,qs,tiles,tail,placement", [
