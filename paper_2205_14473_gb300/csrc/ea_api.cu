@@ -492,6 +492,29 @@ StagePlan make_server_plan(const ea_config &c, const QHost &qw, const QHost &qs,
     return P;
 }
 
+// Whether a PASS_LAZY broadcast that could take the staged server takes the lazy one.  Only the latter has
+// decode tables (a sum of eight signs is one table read), and a CTA per tile; only the former is a
+// pipeline.  Where the lazy server cannot stage its worker messages (n b_w > 32; the staged server's
+// launch takes 0.11 to 0.55 of its time there), or has a scale per chunk to look up (short blocks: 0.3 to
+// 0.7), the staged one runs.  Otherwise rounds by ea_round_step measured, staged against lazy server:
+//   - sign, 1,000,000 to 30,000,000 x 1 .. 32: up to 15% longer (5,000,000 x 8: 199 and 187 us; with 4-bit
+//     grid workers 210 and 200 us); 65,536 x 32: 32.2 and 24.7 us;
+//   - small vectors of one-bit workers with a ragged last tile, for which the lazy server has a path of its
+//     own, fetched cold: 16,000 to 600,000 x 1 or 2 shorter by 0.2 to 1.7 us of 24 to 30, about the same at
+//     n * tiles = 512 (1,860,000 x 1: +0.9 and -0.7 us by placement);
+//   - from about 20 tiles per staged CTA, the pipeline wins where a tile's decode is short: Adam at the
+//     server, one-bit workers, 100,000,000 x 1 / 4 / 8 / 16: -6.2, -3.2, -0.6, +1.0%; power-of-two codes x 8
+//     -1.2%; 4-bit grid workers x 4 +1.5%; with Adam at the workers, one-bit x 1 / 2 / 4: -1.9, 0, +1.1%.
+bool lazy_server_is_faster(const ea_config &c, const QHost &qw, const QHost &qs, int64_t n_tiles, const StagePlan &P,
+                           bool lazy_staged)
+{
+    if (qs.pass != PASS_LAZY || !lazy_staged || qw.pass == PASS_SHORT) return false;
+    const bool one_bit = qw.kind == EA_Q_SIGN_L1, server_adam = c.placement == EA_ADAM_AT_SERVER;
+    if (one_bit && c.d % kTile != 0 && c.n * n_tiles <= 512) return false;
+    const bool short_decode = server_adam ? c.n <= 8 && (one_bit || qw.kind == EA_Q_POW2) : c.n == 1 && one_bit;
+    return !(short_decode && n_tiles >= 20 * static_cast<int64_t>(P.grid));
+}
+
 // The hyper-parameters of the current round (1-based t = h->t + 1 for the bias corrections).
 Hyper round_hyper(const ea_handle *h)
 {
@@ -772,6 +795,7 @@ int ea_init(const ea_config *cfg, void *workspace, size_t workspace_bytes, void 
     if (cudaGetDevice(&dev) == cudaSuccess &&
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess) {
         h->splan = make_server_plan(*cfg, h->qw, h->qs, h->n_tiles, sms);
+        if (lazy_server_is_faster(*cfg, h->qw, h->qs, h->n_tiles, h->splan, h->lazy_staged)) h->splan.enabled = 0;
         // groups that span tiles: the one-pass grouped kernels when their waves fit, else two passes
         const int mode = cfg->placement == EA_ADAM_AT_WORKER ? MODE_W : MODE_S;
         int coop = 0;

@@ -172,20 +172,32 @@ def test_subnormal_sign_scale_is_rounded_once(G):
     assert np.array_equal(got, np.array(want, np.int32))
 
 
-@pytest.mark.parametrize("qw,qs,tiles,tail,placement", [
-    (W.sign_q(0), W.sign_q(0), 456 * 3, 777, ea.ADAM_AT_SERVER),
-    (W.uniform_q(4, 512, True), W.uniform_q(8, 512, False), 456 * 3, 777, ea.ADAM_AT_SERVER),
-    (W.uniform_q(8, 0, False), W.uniform_q(8, 0, False), 456 * 5, 777, ea.ADAM_AT_SERVER),  # beyond the grouped pass
-    (W.sign_q(8192), W.sign_q(12288), 456 * 3, 777, ea.ADAM_AT_SERVER),
-    (W.sign_q(0), W.sign_q(0), 608 * 4, 1, ea.ADAM_AT_WORKER),
-    (W.sign_q(12288), W.uniform_q(8, 512, False), 456 * 6, 4095, ea.ADAM_AT_WORKER),
+@pytest.mark.parametrize("qw,qs,n,tiles,tail,placement", [
+    (W.sign_q(0), W.sign_q(0), 3, 456 * 20, 777, ea.ADAM_AT_SERVER),
+    (W.uniform_q(4, 512, True), W.uniform_q(8, 512, False), 3, 456 * 3, 777, ea.ADAM_AT_SERVER),
+    (W.uniform_q(8, 0, False), W.uniform_q(8, 0, False), 3, 456 * 5, 777, ea.ADAM_AT_SERVER),  # beyond the grouped pass
+    (W.sign_q(8192), W.sign_q(12288), 33, 456 * 2, 777, ea.ADAM_AT_SERVER),
+    (W.sign_q(0), W.sign_q(0), 33, 608 * 2, 1, ea.ADAM_AT_WORKER),
+    (W.sign_q(12288), W.uniform_q(8, 512, False), 3, 456 * 6, 4095, ea.ADAM_AT_WORKER),
 ])
-def test_general_staged_server_refills_its_stages(qw, qs, tiles, tail, placement):
+def test_general_staged_server_refills_its_stages(qw, qs, n, tiles, tail, placement):
     """Short blocks, and scales of several whole tiles, in the staged server with more tiles per CTA than it
     has stages (one stage with Adam at the server, whose e_s slots are refilled after the rest), so that
     every stage is handed back, with u written in it, and filled again."""
-    cfg = ea.EAConfig(d=4096 * tiles + tail, n=3, qw=qw, qs=qs, alpha=1e-3, placement=placement, seed=tiles)
-    _run_host(cfg, 3, seed=tiles + tail, grad_scale=1e-3)
+    cfg = ea.EAConfig(d=4096 * tiles + tail, n=n, qw=qw, qs=qs, alpha=1e-3, placement=placement, seed=tiles)
+    _run_host(cfg, 2 if n > 3 else 3, seed=tiles + tail, grad_scale=1e-3)
+
+
+@pytest.mark.parametrize("qw,qs,n", [
+    (W.sign_q(0), W.sign_q(0), 4), (W.sign_q(4096), W.sign_q(0), 4), (W.uniform_q(8, 0, False), W.sign_q(8192), 4),
+    (W.sign_q(0), W.sign_q(0), 33), (W.uniform_q(4, 0, True), W.sign_q(0), 9), (W.sign_q(1024), W.sign_q(8192), 4)])
+@pytest.mark.parametrize("tail", [-1, 0, 1])  # 512 / 4 tiles, the last one ragged or not, and one more
+@pytest.mark.parametrize("placement", [ea.ADAM_AT_WORKER, ea.ADAM_AT_SERVER])
+def test_sign_broadcast_of_either_server(qw, qs, n, tail, placement):
+    """A scaled-sign broadcast whose groups are whole tiles, on both sides of the rule that gives it to the
+    staged or the lazy server: small and ragged, messages that the lazy server cannot stage, short blocks."""
+    cfg = ea.EAConfig(d=4096 * 128 + tail, n=n, qw=qw, qs=qs, alpha=1e-3, placement=placement, seed=tail + 2)
+    _run_host(cfg, 3, seed=n + tail, grad_scale=1e-2)
 
 
 def test_two_pass_scale_beyond_the_grouped_capacity():
