@@ -50,8 +50,8 @@ def test_ragged_sizes(d, group):
 @pytest.mark.parametrize("n", [1, 2, 5, 8, 9, 16, 33])
 @pytest.mark.parametrize("group", [4096, 0])
 def test_worker_counts(n, group):
-    """Worker counts around the server's 8-worker sign table, with tile and whole-vector scales
-    (33 one-bit workers no longer fit the lazy broadcast's shared-memory staging)."""
+    """Worker counts around the server's 8-worker sign table, with tile and whole-vector scales (33 one-bit
+    workers with one scale are more than the lazy server stages: the staged server takes them)."""
     cfg = ea.EAConfig(d=9000, n=n, qw=W.sign_q(group), qs=W.sign_q(group), alpha=1e-2)
     _run_host(cfg, 4, seed=n)
 
@@ -144,8 +144,8 @@ def test_staged_server_several_tiles_per_cta(qw, qs, placement):
     (W.uniform_q(2, 4096, False), W.uniform_q(4, 1024, False)),
     (W.pow2_q(-20, -5, 8), W.sign_q(256)),
     (W.sign_q(512), W.identity_q()),
-    (W.sign_q(0), W.uniform_q(8, 512, False)),             # the direct server: whole-vector workers
-    (W.uniform_q(4, 256, True), W.sign_q(0)),              # the lazy server
+    (W.sign_q(0), W.uniform_q(8, 512, False)),             # whole-vector workers
+    (W.uniform_q(4, 256, True), W.sign_q(0)),              # short-block workers, a whole-vector broadcast
 ])
 @pytest.mark.parametrize("d,n,placement", [
     (1, 1, ea.ADAM_AT_WORKER), (127, 2, ea.ADAM_AT_SERVER), (2049, 9, ea.ADAM_AT_WORKER),
@@ -198,6 +198,69 @@ def test_sign_broadcast_of_either_server(qw, qs, n, tail, placement):
     staged or the lazy server: small and ragged, messages that the lazy server cannot stage, short blocks."""
     cfg = ea.EAConfig(d=4096 * 128 + tail, n=n, qw=qw, qs=qs, alpha=1e-3, placement=placement, seed=tail + 2)
     _run_host(cfg, 3, seed=n + tail, grad_scale=1e-2)
+
+
+def _segments(d, seed, count):
+    cuts = np.sort(np.random.default_rng(seed).choice(np.arange(1, d), count - 1, replace=False))
+    return tuple(int(v) for v in np.diff(np.concatenate([[0], cuts, [d]])))
+
+
+_DIRECT_D = 4096 * 11 + 1234
+_DIRECT_SEG = _segments(_DIRECT_D, 1, 40)
+
+
+@pytest.mark.parametrize("qw,qs,n", [
+    # server_lazy_kernel with direct loads: more bits than it stages; more groups in a tile than it stages
+    (W.sign_q(-1, _DIRECT_SEG), W.sign_q(-1, _DIRECT_SEG), 33),
+    (W.identity_q(), W.sign_q(6000), 3),
+    (W.uniform_q(8, 1000, False), W.sign_q(-1, _DIRECT_SEG), 5),
+    (W.sign_q(12), W.sign_q(1000), 2),
+    # ... and with staged workers of short blocks
+    (W.uniform_q(4, 256, True), W.sign_q(6000), 3),
+    (W.sign_q(128), W.sign_q(-1, _DIRECT_SEG), 9),
+    # server_kernel: groups that are no whole tiles in the workers' messages, a broadcast of short blocks,
+    # of one scale per tile, without scales
+    (W.sign_q(6000), W.uniform_q(8, 512, False), 3),
+    (W.uniform_q(4, 1000, True), W.sign_q(256), 9),
+    (W.sign_q(-1, _DIRECT_SEG), W.uniform_q(16, 4096, False), 3),
+    (W.uniform_q(8, 6000, False), W.pow2_q(-17, -11, 4), 3),
+    # the two-pass scale of tiles with more groups than the grouped pass takes: more than TileGroups holds
+    (W.uniform_q(4, 12, True), W.uniform_q(8, 12, False), 3),
+    (W.sign_q(4096), W.uniform_q(2, 12, True), 8),
+])
+@pytest.mark.parametrize("placement", [ea.ADAM_AT_WORKER, ea.ADAM_AT_SERVER])
+@pytest.mark.parametrize("ef", [True, False])
+def test_servers_with_direct_loads(qw, qs, n, placement, ef):
+    """What neither the staged nor the grouped server takes, small enough for every form of it."""
+    cfg = ea.EAConfig(d=_DIRECT_D, n=n, qw=qw, qs=qs, alpha=1e-3, placement=placement, error_feedback=ef, seed=n)
+    _run_host(cfg, 3, seed=n, grad_scale=1e-3)
+
+
+@pytest.mark.parametrize("qw,qs,tiles,placement", [
+    # two-pass worker messages with a few groups in a tile (the grouped worker ends at one tile per CTA)
+    (W.uniform_q(4, 1000, True), W.sign_q(4096), 640, ea.ADAM_AT_WORKER),
+    (W.uniform_q(8, 6000, False), W.sign_q(4096), 640, ea.ADAM_AT_SERVER),
+    # a two-pass broadcast of the direct server: segments between which the grouped server cannot cut the
+    # vector into waves (odd offsets), and more tiles than it holds at once
+    (W.sign_q(4096), (8, False), 2400, ea.ADAM_AT_WORKER),
+    (W.sign_q(4096), (4, True), 2400, ea.ADAM_AT_SERVER),
+])
+def test_two_pass_scale_of_several_groups_per_tile(qw, qs, tiles, placement):
+    d = 4096 * tiles + 321
+    if isinstance(qs, tuple):
+        cuts = sorted({int(v) | 1 for v in np.random.default_rng(61).integers(1, d - 1, 61)})
+        segs = tuple(b - a for a, b in zip([0, *cuts], [*cuts, d]))
+        qs = W.QuantSpec(W.Q_UNIFORM_MAX, qs[0], -1, segs, qs[1])
+    cfg = ea.EAConfig(d=d, n=2, qw=qw, qs=qs, alpha=1e-3, placement=placement, seed=53)
+    L = _run_host(cfg, 2, seed=55, grad_scale=1e-3)
+    assert L.gpu.launches_per_round == (2 * 3 + 1 + 1 if tiles == 640 else 2 * 1 + 3 + 1)
+
+
+@pytest.mark.parametrize("qw,qs", [(W.sign_q(512), W.uniform_q(8, 512, False)), (W.uniform_q(4, 128, True), W.sign_q(2048))])
+@pytest.mark.parametrize("placement", [ea.ADAM_AT_WORKER, ea.ADAM_AT_SERVER])
+def test_short_blocks_without_error_feedback(qw, qs, placement):
+    cfg = ea.EAConfig(d=20_001, n=5, qw=qw, qs=qs, alpha=1e-3, placement=placement, error_feedback=False, seed=57)
+    _run_host(cfg, 3, seed=59, grad_scale=1e-3)
 
 
 def test_two_pass_scale_beyond_the_grouped_capacity():
@@ -278,13 +341,8 @@ def test_lazy_views_mid_round_change_nothing(group):
     assert a.launches_per_round == cfg.n + 1 + 2 + 1
 
 
-@pytest.mark.parametrize("qw,n", [(W.sign_q(0), 3), (W.uniform_q(4, 4096, True), 33), (W.uniform_q(8, 512, False), 65),
-                                  (W.pow2_q(-17, -11, 4), 10), (W.uniform_q(8, 0, False), 2)])
-@pytest.mark.parametrize("d", [500, 9000])
-@pytest.mark.parametrize("placement", [ea.ADAM_AT_WORKER, ea.ADAM_AT_SERVER])
-def test_round_step_equals_separate_calls(qw, n, d, placement):
-    """EARound.step, whose workers share launches (up to 32 each), leaves the same bits as one call each."""
-    cfg = ea.EAConfig(d=d, n=n, qw=qw, qs=W.sign_q(4096), alpha=1e-3, placement=placement, seed=3)
+def _step_equals_calls(cfg):
+    d, n, placement = cfg.d, cfg.n, cfg.placement
     a, b = ea.EARound(cfg), ea.EARound(cfg)
     gen = torch.Generator(device="cuda").manual_seed(d + n)
     xa, xb = torch.zeros(d, device="cuda"), torch.zeros(d, device="cuda")
@@ -303,6 +361,27 @@ def test_round_step_equals_separate_calls(qw, n, d, placement):
     for v in (ea.EA_VIEW_CODES_SERVER, ea.EA_VIEW_SCALES_SERVER, ea.EA_VIEW_E_SERVER):
         assert torch.equal(a.view(v), b.view(v))
     assert torch.equal(xa, xb) and a.t == b.t == 3 and a.bits_sent() == b.bits_sent()
+
+
+_FEW_SEG = (20 * 4096 + 64, 15 * 4096, 9 * 4096 + 5)  # three tiles of 45 hold a boundary or are ragged
+
+
+@pytest.mark.parametrize("n", [2, 34])
+@pytest.mark.parametrize("placement", [ea.ADAM_AT_WORKER, ea.ADAM_AT_SERVER])
+def test_round_step_equals_separate_calls_with_segments(n, placement):
+    """Shared launches in which every worker's tiles with a boundary go first."""
+    d = sum(_FEW_SEG)
+    q = W.sign_q(-1, _FEW_SEG)
+    _step_equals_calls(ea.EAConfig(d=d, n=n, qw=q, qs=q, alpha=1e-3, placement=placement, seed=3))
+
+
+@pytest.mark.parametrize("qw,n", [(W.sign_q(0), 3), (W.uniform_q(4, 4096, True), 33), (W.uniform_q(8, 512, False), 65),
+                                  (W.pow2_q(-17, -11, 4), 10), (W.uniform_q(8, 0, False), 2)])
+@pytest.mark.parametrize("d", [500, 9000])
+@pytest.mark.parametrize("placement", [ea.ADAM_AT_WORKER, ea.ADAM_AT_SERVER])
+def test_round_step_equals_separate_calls(qw, n, d, placement):
+    """EARound.step, whose workers share launches (up to 32 each), leaves the same bits as one call each."""
+    _step_equals_calls(ea.EAConfig(d=d, n=n, qw=qw, qs=W.sign_q(4096), alpha=1e-3, placement=placement, seed=3))
 
 
 def test_round_step_stops_where_a_call_is_refused():
