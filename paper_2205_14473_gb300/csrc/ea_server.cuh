@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(kThreads, 2) server_kernel(const ServerArgs a)
     __shared__ float stab[256];
     __shared__ TileGroups tg;
     __shared__ float4 ubuf[kSlots * kThreads];
-    const int64_t tile = blockIdx.x;
+    const int64_t tile = plain_tile();  // last first, against the order of encode_kernel
     const int64_t d = a.d;
 
     pdl_trigger();
