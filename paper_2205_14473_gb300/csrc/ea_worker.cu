@@ -123,7 +123,10 @@ __global__ void __launch_bounds__(kThreads, MODE == MODE_S ? 4 : 3)
     } else if (has_scale<QK>() && a.pass == PASS_SHORT) {
         if (full) worker_tile<MODE, QK, true, PASS_SHORT>(a, p, tile, ubuf, sm, ref);
         else worker_tile<MODE, QK, false, PASS_SHORT>(a, p, tile, ubuf, sm, ref);
-    } else {
+    } else if (has_scale<QK>() && a.q.grp.gkind == GK_WHOLE) {
+        if (full) worker_tile<MODE, QK, true, PASS_STASH_ONE>(a, p, tile, ubuf, sm, ref);
+        else worker_tile<MODE, QK, false, PASS_STASH_ONE>(a, p, tile, ubuf, sm, ref);
+    } else if (QK != QK_SIGN) {  // (a handle's scaled sign takes worker_lazy_kernel)
         if (full) worker_tile<MODE, QK, true, PASS_STASH>(a, p, tile, ubuf, sm, ref);
         else worker_tile<MODE, QK, false, PASS_STASH>(a, p, tile, ubuf, sm, ref);
     }
@@ -250,10 +253,11 @@ __global__ void __launch_bounds__(kThreads) finalize_kernel(const FinalizeArgs a
 }
 
 // Second pass, one CTA per tile: encode the stashed input with its group's scale and leave the
-// residual u - Q(u) in its place.  The first pass takes the tiles last first and this one first first:
-// u was stored without a streaming hint among streams that have one, so the tiles written last are still in L2, and what is
-// overwritten there was never written to memory.  Whole-vector 8-bit grid, 30,000,000 x 4: the round
-// 1042 us with both passes in order and streaming hints (and two CTAs per SM here), 866 us so.
+// residual u - Q(u) in its place.  The first pass takes the tiles last first and this one first first, so
+// that it begins with what was written last; u that was stored without a streaming hint (PASS_STASH_ONE) is
+// in part still in L2 then, and what is overwritten there was never written to memory.  Whole-vector 8-bit
+// grid, 30,000,000 x 4: the round 1042 us with both passes in one order, streaming hints and two CTAs per SM
+// here, 903 us with opposite orders, no hint and four CTAs.
 template <int QK, bool FULL>
 __device__ __forceinline__ void encode_one_group(const EncodeArgs &a, float s, int64_t tile, const float *qtab)
 {
