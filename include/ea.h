@@ -7,6 +7,7 @@
  *   ea_worker_compress(h, i, g_i)  for every worker i   -- Algorithm 2, the worker's message
  *   ea_server_step(h)                                   -- Algorithm 1, the server's broadcast
  *   ea_worker_apply(h, x)          for every replica    -- Algorithms 1-2, x <- x - Q_s(...)
+ * or, with all gradients at hand, ea_round_step(h, g, x), in which workers share launches.
  * Every call is asynchronous on the stream given to ea_init and never synchronizes, except
  * ea_sync_status.  The library allocates no device memory: the caller passes one workspace of
  * ea_workspace_bytes() bytes, and owns it, the stream, the gradients and x.
@@ -136,8 +137,9 @@ int ea_bits_sent(const ea_handle *h, uint64_t *up_bits, uint64_t *down_bits);
 int ea_round_index(const ea_handle *h, int64_t *t);
 
 /* Kernel launches that one round of separate calls makes on the stream: n worker compresses, one server
- * step and one apply (ea_round_step makes fewer).  A message without scales, with 4096-blocks, with power-of-two blocks of 128 to 2048, or whose
- * one group is at most 4096 long takes one launch.  With other groups:
+ * step and one apply (ea_round_step makes fewer).  A message without scales, with 4096-blocks, with
+ * power-of-two blocks of 128 to 2048, or whose one group is at most 4096 long takes one launch.  With other
+ * groups:
  *   - a scaled-sign message takes one pass, which writes the codes (the signs, which need no scale)
  *     with the groups' partial norms, and a finalize forms the scales: one finalize for all worker
  *     messages (at the server step, or at a view of a worker's scales or residual), one for the

@@ -8,6 +8,7 @@ or cannot be loaded, the first call raises.
 
     rnd = EARound(cfg)                 # cfg: EAConfig; allocates the workspace with torch
     for t in range(T):
+        rnd.step(g, x)             # or, one by one:
         for i in range(cfg.n): rnd.worker_compress(i, g[i])
         rnd.server_step()
         rnd.apply(x)

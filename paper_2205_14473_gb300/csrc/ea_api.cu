@@ -75,8 +75,9 @@ struct ea_handle {
     std::vector<unsigned char> lazy_w;  // PASS_LAZY: worker i's e holds its last u (see lazy_residual)
     bool lazy_s = false;                // PASS_LAZY: e_s holds the last w
     bool lazy_staged = false;           // PASS_LAZY broadcast: every tile's worker messages fit the staging
-    // The last launch held the SMs at their largest shared memory for more than one tile per CTA: the
-    // next one waits for it, so that the SMs are empty and take the round's own split (launch_pdl).
+    // The last launch held the SMs at their largest shared memory (a grouped kernel, or a staged server
+    // with more than one tile per CTA): the next one waits for it, so that the SMs are empty and take the
+    // round's own split (launch_pdl).
     bool split_full = false;
     bool wscales_pending = false;       // PASS_LAZY workers: a message's scales are not formed yet
     int n_compressed = 0;
@@ -441,7 +442,7 @@ uint64_t message_bits(const QHost &q, int64_t d)
 // Shared-memory staging of the server's inputs (see server_staged_kernel): one stage holds a
 // tile's e_s (+ m_s, v_s) and the n workers' code chunks and scales.  Enabled when the scale groups of
 // both messages lie inside 4096-tiles or are whole tiles (or there are none) and one stage fits in
-// 200 KB.  Where a group spans tiles: d = 30,000,000 with one scale, four workers' 8-bit grid messages and
+// 200 KB (see also lazy_server_is_faster).  Where a group spans tiles: d = 30,000,000 with one scale, four workers' 8-bit grid messages and
 // broadcast: the round took 1312 us with a server CTA per tile that loads directly (383 us of it the
 // server's), 1042 us staged.
 StagePlan make_server_plan(const ea_config &c, const QHost &qw, const QHost &qs, int64_t n_tiles, int sms)

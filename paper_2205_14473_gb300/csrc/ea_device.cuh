@@ -362,8 +362,9 @@ __host__ __device__ __forceinline__ int chunk_shift(const Grouping &g)
 // the rest of the grid runs beside it, and not into the last wave.  So the tiles are taken last first;
 // and where a few segments' boundaries make such tiles (Grouping::slow lists them, a ragged last one
 // among them), the first n_slow CTAs take those, and the CTAs whose turn they would be (the grid has
-// n_slow more) have none.  ResNet-18's 62 tensors (23 such tiles of 2,854) with Adam at the server: a
-// worker message 30.4 us in order, 23.9 us so; apply 37 and 22.5 us, the server 120 and 91 us.
+// n_slow more) have none.  ResNet-18's 62 tensors (23 such tiles of 2,854) with Adam at the server, CUDA
+// events around the sixteen worker messages, the server step and the apply, in order and so (with the rolled
+// loops of TileGroups): a message 30.4 and 23.9 us, the server step 120 and 91 us, the apply 37 and 22.5 us.
 struct CtaTile {
     int64_t tile;  // -1: none
     bool plain;    // a whole tile inside one group

@@ -179,7 +179,7 @@ struct StagePlan {
     int grid;                  // persistent CTAs
     uint32_t stage_bytes;      // bytes of one stage
     uint32_t smem_bytes;       // dynamic shared memory per CTA (barriers + stages)
-    uint32_t off_a, off_b, off_c, off_d;  // up to four 16 KB state tiles (kernel-specific meaning)
+    uint32_t off_a, off_b, off_c;  // the e_s tile (16 KB) and, with Adam at the server, m_s and v_s
     uint32_t off_codes;        // n code chunks of code_chunk bytes
     uint32_t code_chunk;       // bytes of one worker's codes for one tile (4096 b / 8)
     uint32_t off_scales;       // the n workers' scales of the tile (binary32)
@@ -265,7 +265,7 @@ template <int MODE, int QS>
 cudaError_t server_grouped_shape_for_qs(int qw, GroupedShape *out);
 cudaError_t launch_server_grouped(int mode, const ServerArgs &a, int grid, cudaStream_t s);
 // PASS_LAZY for a scaled-sign broadcast (instantiated with the QS = QK_SIGN server kernels).
-// staged: every tile's worker codes and scales fit the shared-memory staging (lazy_server_staged).
+// staged: every tile's worker codes and scales fit the shared-memory staging (ea_handle::lazy_staged).
 template <int MODE>
 cudaError_t launch_server_lazy(const ServerArgs &a, bool staged, cudaStream_t s);
 cudaError_t server_grouped_shape(int mode, int qw, int qs, GroupedShape *out);

@@ -495,7 +495,8 @@ __global__ void __launch_bounds__(kThreads, MODE == MODE_S ? 2 : 3) server_group
                 if (full) server_u_range<MODE, QW, true>(a, tile, lo, hi, ub, utab, stab, gs.tg, rw, nullptr);
                 else server_u_range<MODE, QW, false>(a, tile, lo, hi, ub, utab, stab, gs.tg, rw, nullptr);
             }
-            group_partials<QS>(USmem{ub}, tile, lo, hi, a.d, a.qs, tile_ref(a.qs.grp, tile, a.d), nullptr, a.partials, gs.parts, turn);
+            group_partials<QS>(USmem{ub}, tile, lo, hi, a.d, a.qs, tile_ref(a.qs.grp, tile, a.d), nullptr, a.partials,
+                               gs.parts, turn);
         }
         if (!wave_barrier(gp, w, a.status, gs)) return;
         encode_wave<QS>(uslot, t0, t_end, c0, c1, a.d, a.qs, a.words, a.partials, a.scales, a.es, a.ef, a.seed,
@@ -772,7 +773,6 @@ __device__ __forceinline__ bool server_staged_tile(const ServerArgs &a, int64_t 
             for (int i = 0; i < 4; ++i) acc[k][i] = pow2n ? __fmul_rn(acc[k][i], inv_n) : __fdiv_rn(acc[k][i], nf);
     }
     if constexpr (!GENERAL && QW == QK_SIGN) {
-      {
         done = NW == 8 || n <= 8;
         // Scaled-sign workers: the worker-order sum of the first m = min(n, 8) workers depends
         // only on their m sign bits.  Thread p forms it for sign pattern p (bit w = worker w's
@@ -819,7 +819,6 @@ __device__ __forceinline__ bool server_staged_tile(const ServerArgs &a, int64_t 
                 acc[k + 1][i] = *reinterpret_cast<const float *>(tb + o1);
             }
         }
-      }
     }
     if (!GENERAL && !done) {
         // scaled-sign workers (n > 8): acc already holds the sum of workers 0..7
@@ -1076,12 +1075,17 @@ __global__ void __launch_bounds__(kThreads + 32, server_ctas_per_sm(MODE, QW, QS
         const bool whole = (tile + 1) * kTile <= d;
         bool go;
         if constexpr (GENERAL) {
-            go = whole ? server_staged_tile<MODE, QW, QS, true, 0, true>(a, tile, st, ok, &early[s], &empty[s], Lw, Lwf, ut, wtab, flip, sm)
-                       : server_staged_tile<MODE, QW, QS, false, 0, true>(a, tile, st, ok, &early[s], &empty[s], Lw, Lwf, ut, wtab, flip, sm);
+            go = whole ? server_staged_tile<MODE, QW, QS, true, 0, true>(a, tile, st, ok, &early[s], &empty[s], Lw, Lwf,
+                                                                         ut, wtab, flip, sm)
+                       : server_staged_tile<MODE, QW, QS, false, 0, true>(a, tile, st, ok, &early[s], &empty[s], Lw, Lwf,
+                                                                          ut, wtab, flip, sm);
         } else {
-            go = !whole ? server_staged_tile<MODE, QW, QS, false, 0, false>(a, tile, st, ok, &early[s], &empty[s], Lw, Lwf, ut, wtab, flip, sm)
-                 : n8   ? server_staged_tile<MODE, QW, QS, true, 8, false>(a, tile, st, ok, &early[s], &empty[s], Lw, Lwf, ut, wtab, flip, sm)
-                        : server_staged_tile<MODE, QW, QS, true, 0, false>(a, tile, st, ok, &early[s], &empty[s], Lw, Lwf, ut, wtab, flip, sm);
+            go = !whole ? server_staged_tile<MODE, QW, QS, false, 0, false>(a, tile, st, ok, &early[s], &empty[s], Lw,
+                                                                            Lwf, ut, wtab, flip, sm)
+                 : n8   ? server_staged_tile<MODE, QW, QS, true, 8, false>(a, tile, st, ok, &early[s], &empty[s], Lw,
+                                                                           Lwf, ut, wtab, flip, sm)
+                        : server_staged_tile<MODE, QW, QS, true, 0, false>(a, tile, st, ok, &early[s], &empty[s], Lw,
+                                                                           Lwf, ut, wtab, flip, sm);
         }
         if (!go) {
             if (threadIdx.x == 0) report_status(a.status, kStatusTimeout);
@@ -1170,7 +1174,6 @@ cudaError_t launch_server_for_qs(const ServerArgs &a, cudaStream_t s)
         if (a.plan.enabled) return launch_server_staged<MODE, QK_IDENT, QS>(a, s);
         return launch_pdl(server_kernel<MODE, QK_IDENT, QS>, grid, block, 0, s, true, kCarveoutPercent, a);
     }
-    return cudaGetLastError();
 }
 
 }  // namespace ea

@@ -226,12 +226,12 @@ __device__ __forceinline__ bool unif_index_fast(float u, float r, float Lf, floa
     }
 }
 
-// Encode u (valid coordinates only) with scale s, store codes (all lanes) and the residual.
-// FULL: the whole tile lies inside [0, d), so no coordinate needs a bounds check.
 // Variants of the per-coordinate encode, chosen once per tile: the uniform grid's zero scale
 // (every q = 0), deterministic or stochastic rounding, decode from the fl(i/L) table or by division.
 enum EncVar : int { ENC_PLAIN = 0, ENC_UZERO, ENC_UDET_TAB, ENC_UDET_DIV, ENC_USTO_TAB, ENC_USTO_DIV };
 
+// Encode u (valid coordinates only) with its scale, store codes (all lanes) and the residual.
+// FULL: the whole tile lies inside [0, d), so no coordinate needs a bounds check.
 // BITS: the code width as a compile-time constant (0: code_bits of the kind, or q.bits).
 // Only the coordinates of [lo, d) are encoded and stored (lo: 0, or the start of a word and a slot).
 template <int QK, bool FULL, bool BALLOT, int VAR, int BITS, class USrc, class Scale>
@@ -296,8 +296,6 @@ __device__ __forceinline__ void encode_store_v(const USrc &src, Scale sc, int64_
     }
 }
 
-// Encode u (valid coordinates only) with scale s, store codes (all lanes) and the residual.
-// FULL: the whole tile lies inside [0, d), so no coordinate needs a bounds check.
 // Example 1 with a compile-time width: for b <= 8 the caller passes qtab (fl(i/L) of the tile's
 // quantizer) and the decode is a table read; 16-bit grids divide.
 template <int QK, bool FULL, bool BALLOT, int BITS, class USrc, class Scale>

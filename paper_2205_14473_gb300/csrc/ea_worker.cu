@@ -8,8 +8,8 @@ namespace ea {
 // the scale's reduction and more CTAs fit on an SM.
 // ref: the tile's groups (PASS_STASH, PASS_LAZY), looked up by the caller.
 template <int MODE, int QK, bool FULL, int PASS>
-__device__ __forceinline__ void worker_tile(const WorkerArgs &a, const WorkerBufs &p, int64_t tile, float4 *ubuf, TileSmem &sm,
-                                            const TileRef &ref)
+__device__ __forceinline__ void worker_tile(const WorkerArgs &a, const WorkerBufs &p, int64_t tile, float4 *ubuf,
+                                            TileSmem &sm, const TileRef &ref)
 {
     const int64_t d = a.d;
     constexpr bool lazy = PASS == PASS_LAZY || PASS == PASS_LAZY_ONE;
@@ -54,8 +54,8 @@ __device__ __forceinline__ void worker_tile(const WorkerArgs &a, const WorkerBuf
             store4<FULL>(p.v, q, d, v[k]);
         }
     }
-    finish_tile<QK, FULL, true, PASS>(USmem{ubuf}, tile, d, a.q, p.words, p.scales, p.e, a.ef, a.pass, a.seed, (a.id + blockIdx.y), a.t,
-                                      p.partials, sm, ref);
+    finish_tile<QK, FULL, true, PASS>(USmem{ubuf}, tile, d, a.q, p.words, p.scales, p.e, a.ef, a.pass, a.seed,
+                                      a.id + blockIdx.y, a.t, p.partials, sm, ref);
 }
 
 // Algorithm 2 for one worker on one 4096-coordinate tile.  With Adam at the worker:
@@ -137,7 +137,8 @@ __global__ void __launch_bounds__(kThreads, MODE == MODE_S ? 4 : 3)
 // FULL: the range is the whole tile.  All four slots' loads are issued at once (the kernel's
 // register budget is sized for it), so that enough bytes are in flight per SM.
 template <int MODE, bool FULL>
-__device__ __forceinline__ void worker_u_range(const WorkerArgs &a, const WorkerBufs &p, int64_t tile, int64_t lo, int64_t hi, float4 *ub)
+__device__ __forceinline__ void worker_u_range(const WorkerArgs &a, const WorkerBufs &p, int64_t tile, int64_t lo,
+                                               int64_t hi, float4 *ub)
 {
     constexpr int H = kSlots;
 #pragma unroll
@@ -205,11 +206,11 @@ __global__ void __launch_bounds__(kThreads, MODE == MODE_S ? 4 : 2) worker_group
             const int64_t tl = static_cast<int64_t>(tile) * kTile, lo = max(c0, tl), hi = min(c1, tl + kTile);
             if (lo == tl && hi == tl + kTile) worker_u_range<MODE, true>(a, p, tile, lo, hi, ub);
             else worker_u_range<MODE, false>(a, p, tile, lo, hi, ub);
-            group_partials<QK>(USmem{ub}, tile, lo, hi, a.d, a.q, tile_ref(a.q.grp, tile, a.d), nullptr, p.partials, gs.parts, turn);
+            group_partials<QK>(USmem{ub}, tile, lo, hi, a.d, a.q, tile_ref(a.q.grp, tile, a.d), nullptr, p.partials,
+                               gs.parts, turn);
         }
         if (!wave_barrier(gp, w, a.status, gs)) return;
-        encode_wave<QK>(uslot, t0, t_end, c0, c1, a.d, a.q, p.words, p.partials, p.scales, p.e, a.ef, a.seed, (a.id + blockIdx.y),
-                        a.t, gs);
+        encode_wave<QK>(uslot, t0, t_end, c0, c1, a.d, a.q, p.words, p.partials, p.scales, p.e, a.ef, a.seed, a.id, a.t, gs);
     }
 }
 
@@ -331,7 +332,8 @@ __global__ void __launch_bounds__(kThreads, 4) encode_kernel(const EncodeArgs a)
 // AS_ANY: a group lookup.
 enum ApplyScales : int { AS_TILE, AS_SLOT, AS_ANY };
 template <int QK, bool FULL, int BITS, int SCALES>
-__device__ __forceinline__ void apply_tile(const ApplyArgs &a, int64_t tile, const TileRef &ref, const TileGroups &tg, float *qtab_s)
+__device__ __forceinline__ void apply_tile(const ApplyArgs &a, int64_t tile, const TileRef &ref, const TileGroups &tg,
+                                           float *qtab_s)
 {
     const int64_t d = a.d;
     const Grouping &G = a.q.grp;
