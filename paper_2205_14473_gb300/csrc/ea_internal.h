@@ -163,6 +163,7 @@ struct WorkerArgs {
     QParams q;
     Hyper hp;
     int ef, pass;
+    int keep;                 // PASS_STASH: u is stored to be found in L2 (see stash_is_kept)
     uint64_t seed;
     uint32_t id, t;           // the first worker's id
     GroupPlan gp;             // PASS_GROUPED

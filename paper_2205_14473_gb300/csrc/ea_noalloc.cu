@@ -128,6 +128,7 @@ extern "C" int ea_worker_compress_noalloc(const ea_config *cfg, int32_t worker, 
     }
     a.ef = cfg->error_feedback;
     a.pass = d <= kTile ? PASS_FUSED : PASS_STASH;
+    a.keep = 1;
     a.seed = cfg->seed;
     a.id = static_cast<uint32_t>(worker);
     a.t = static_cast<uint32_t>(round);

@@ -366,12 +366,10 @@ __device__ __forceinline__ void finish_tile_smem(const float4 *ubuf, DF l1, floa
 // by the worker's kernel (the general form's group lookups cost registers: with Adam at the worker,
 // a single form for both spilled 92 bytes a thread, and ResNet-18's messages took 5% longer).
 constexpr int PASS_LAZY_ONE = 16;
-// Likewise PASS_STASH, where the caller knows it.  u is then stored without a streaming hint, so that the
-// second pass finds a part of it in L2: a worker's message with one scale, the staged server's broadcast.
-// Where the tiles hold several groups u is stored with the hint; kept, it displaced what the grouped or the
-// direct server reads next.  Rounds with u kept and streamed, 4-bit grid up, 8-bit down, 62 segments:
-// 16,000,001 x 1 317 and 291 us, 20,000,001 x 2 (Adam at the server) 451 and 415 us, x 8 1,211 and 1,193 us.
-constexpr int PASS_STASH_ONE = 17;
+constexpr int PASS_STASH_ONE = 17;  // likewise PASS_STASH, where the caller knows it
+// PASS_STASH with a streaming hint on the stores of u (stash_is_kept).  The direct server (PASS = -1) stores
+// so too: 62 segments, 60,000,001 x 1, Adam at the server, the round 871 us with that u kept, 800 us so.
+constexpr int PASS_STASH_STREAM = 18;
 
 // The tile's end for a quantizer with scale groups, u read through `src` (URegs or USmem).
 //   PASS_FUSED: the tile is exactly one scale group (blocks of 4096): reduce, encode, store.
@@ -448,8 +446,8 @@ __device__ __forceinline__ void finish_tile(const USrc &src, int64_t tile, int64
                 for (int i = 0; i < 4; ++i) df_accumulate(all, fabsf(uk[i]));  // u beyond d is 0
             if constexpr (!lazy) {
                 if (FULL || 4 * qs < d) {
-                    if constexpr (PASS == PASS_STASH_ONE) store4_kept<FULL>(resid, qs, d, uk);
-                    else store4<FULL>(resid, qs, d, uk);
+                    if constexpr (PASS < 0 || PASS == PASS_STASH_STREAM) store4<FULL>(resid, qs, d, uk);
+                    else store4_kept<FULL>(resid, qs, d, uk);
                 }
             } else {
                 if (ef && (FULL || 4 * qs < d)) store4<FULL>(resid, qs, d, uk);

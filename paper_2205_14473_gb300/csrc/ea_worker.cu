@@ -123,13 +123,32 @@ __global__ void __launch_bounds__(kThreads, MODE == MODE_S ? 4 : 3)
     } else if (has_scale<QK>() && a.pass == PASS_SHORT) {
         if (full) worker_tile<MODE, QK, true, PASS_SHORT>(a, p, tile, ubuf, sm, ref);
         else worker_tile<MODE, QK, false, PASS_SHORT>(a, p, tile, ubuf, sm, ref);
-    } else if (has_scale<QK>() && a.q.grp.gkind == GK_WHOLE) {
-        if (full) worker_tile<MODE, QK, true, PASS_STASH_ONE>(a, p, tile, ubuf, sm, ref);
-        else worker_tile<MODE, QK, false, PASS_STASH_ONE>(a, p, tile, ubuf, sm, ref);
-    } else if (QK != QK_SIGN) {  // (a handle's scaled sign takes worker_lazy_kernel)
+    } else {
         if (full) worker_tile<MODE, QK, true, PASS_STASH>(a, p, tile, ubuf, sm, ref);
         else worker_tile<MODE, QK, false, PASS_STASH>(a, p, tile, ubuf, sm, ref);
     }
+}
+
+// PASS_STASH of the uniform grid with streaming stores of u (WorkerArgs::keep = 0).  A kernel of its own: as
+// a path more in worker_kernel it made that one 2 to 5% longer for messages of 1 to 5 million coordinates.
+template <int MODE>
+__global__ void __launch_bounds__(kThreads, MODE == MODE_S ? 4 : 3)
+    worker_stream_kernel(const __grid_constant__ WorkerArgs a, const __grid_constant__ WorkerOne ws)
+{
+    __shared__ TileSmem sm;
+    __shared__ float4 ubuf[kSlots * kThreads];
+    pdl_trigger();
+    const WorkerBufs &p = ws.at(0);
+    const int64_t tile = plain_tile();
+    const TileRef ref = tile_ref(a.q.grp, tile, a.d);
+    if (threadIdx.x == 0) sm.part = ref.part();
+    if (ref.ng() > 1) {
+        cache_tile_groups(a.q.grp, tile, a.d, sm.tg);
+        __syncthreads();
+    }
+    pdl_wait();
+    if ((tile + 1) * kTile <= a.d) worker_tile<MODE, QK_UNIF, true, PASS_STASH_STREAM>(a, p, tile, ubuf, sm, ref);
+    else worker_tile<MODE, QK_UNIF, false, PASS_STASH_STREAM>(a, p, tile, ubuf, sm, ref);
 }
 
 // Phase one of a grouped worker tile: u of the coordinate range [lo, hi) of tile `tile` (0
@@ -255,7 +274,7 @@ __global__ void __launch_bounds__(kThreads) finalize_kernel(const FinalizeArgs a
 
 // Second pass, one CTA per tile: encode the stashed input with its group's scale and leave the
 // residual u - Q(u) in its place.  The first pass takes the tiles last first and this one first first, so
-// that it begins with what was written last; u that was stored without a streaming hint (PASS_STASH_ONE) is
+// that it begins with what was written last; u that was stored without a streaming hint (stash_is_kept) is
 // in part still in L2 then, and what is overwritten there was never written to memory.  Whole-vector 8-bit
 // grid, 30,000,000 x 4: the round 1042 us with both passes in one order, streaming hints and two CTAs per SM
 // here, 903 us with opposite orders, no hint and four CTAs.
@@ -469,6 +488,12 @@ cudaError_t launch_worker(int mode, const WorkerArgs &a, const WorkerBufs *w, in
 {
     if (count == 1) {
         const WorkerOne one{w[0]};
+        if (a.pass == PASS_STASH && a.q.kind == QK_UNIF && !a.keep) {
+            const dim3 grid(static_cast<unsigned>(a.n_tiles)), block(kThreads);
+            return mode == MODE_W
+                       ? launch_pdl(worker_stream_kernel<MODE_W>, grid, block, 0, s, overlap, kCarveoutPercent, a, one)
+                       : launch_pdl(worker_stream_kernel<MODE_S>, grid, block, 0, s, overlap, kCarveoutPercent, a, one);
+        }
         return mode == MODE_W ? launch_worker_mode<MODE_W>(a, one, 1, s, overlap)
                               : launch_worker_mode<MODE_S>(a, one, 1, s, overlap);
     }

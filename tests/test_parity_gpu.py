@@ -240,6 +240,9 @@ def test_servers_with_direct_loads(qw, qs, n, placement, ef):
     # two-pass worker messages with a few groups in a tile (the grouped worker ends at one tile per CTA)
     (W.uniform_q(4, 1000, True), W.sign_q(4096), 640, ea.ADAM_AT_WORKER),
     (W.uniform_q(8, 6000, False), W.sign_q(4096), 640, ea.ADAM_AT_SERVER),
+    # ... and so many tiles that u is stored with a streaming hint
+    (W.uniform_q(4, 1000, True), W.sign_q(4096), 2048, ea.ADAM_AT_SERVER),
+    (W.uniform_q(8, 6000, False), W.sign_q(4096), 2048, ea.ADAM_AT_WORKER),
     # a two-pass broadcast of the direct server: segments between which the grouped server cannot cut the
     # vector into waves (odd offsets), and more tiles than it holds at once
     (W.sign_q(4096), (8, False), 2400, ea.ADAM_AT_WORKER),
@@ -247,13 +250,14 @@ def test_servers_with_direct_loads(qw, qs, n, placement, ef):
 ])
 def test_two_pass_scale_of_several_groups_per_tile(qw, qs, tiles, placement):
     d = 4096 * tiles + 321
-    if isinstance(qs, tuple):
+    two_pass_broadcast = isinstance(qs, tuple)
+    if two_pass_broadcast:
         cuts = sorted({int(v) | 1 for v in np.random.default_rng(61).integers(1, d - 1, 61)})
         segs = tuple(b - a for a, b in zip([0, *cuts], [*cuts, d]))
         qs = W.QuantSpec(W.Q_UNIFORM_MAX, qs[0], -1, segs, qs[1])
     cfg = ea.EAConfig(d=d, n=2, qw=qw, qs=qs, alpha=1e-3, placement=placement, seed=53)
     L = _run_host(cfg, 2, seed=55, grad_scale=1e-3)
-    assert L.gpu.launches_per_round == (2 * 3 + 1 + 1 if tiles == 640 else 2 * 1 + 3 + 1)
+    assert L.gpu.launches_per_round == (2 * 1 + 3 + 1 if two_pass_broadcast else 2 * 3 + 1 + 1)
 
 
 @pytest.mark.parametrize("qw,qs", [(W.sign_q(512), W.uniform_q(8, 512, False)), (W.uniform_q(4, 128, True), W.sign_q(2048))])
